@@ -333,7 +333,7 @@ int post_hooks(pasm_ctx* c, int l, float* cur, float* tmp, float* F) {
   NNGrid g{nn.nx[l], nn.ny[l], ldk, c->k};
   const float om = (float)c->opts.omega;
   rowop<float>(L, OP_RESID, v.A, cur, F, nullptr, nullptr, om, nn.R, ldk);        // r = f - A e
-  if (nn_tc_supported(ldk)) nn_forward_tc(L, g, nn.w13, nn.w2, nn.R, nn.D, nn.err);        // d = N(r), tensor cores
+  if (nn_tc_supported(ldk)) nn_forward_tc(L, g, &nn.w13, nullptr, nn.w2, nn.R, nn.D, nn.err);  // d = N(r), tensor cores
   else nn_forward(L, g, nn.buf, nn.W, nn.R, nn.D);
   rowop<float>(L, OP_RESID, v.A, nn.D, nn.R, nullptr, nullptr, om, nn.Rt, ldk);   // f - A (e + d) = r - A d
   nn_column_norms(L, v.n, ldk, nn.R, nn.Rt, nn.partial, nn.norms);
@@ -1173,7 +1173,7 @@ int pasm_init(pasm_ctx* c, int k, double tol, const double* lambda0, const doubl
     int64_t maxn = 0;
     for (int l = 0; l < c->nlev; ++l)
       if (c->nn.nx[(size_t)l]) maxn = std::max<int64_t>(maxn, c->lv[(size_t)l].n);
-    r = nn_ensure(c, maxn * c->ldk, maxn * c->ldk, false);
+    r = nn_ensure(c, nn_tc_supported(c->ldk) ? 0 : maxn * c->ldk, maxn * c->ldk, false);
     if (r) return r;
     CK(cudaMemsetAsync(c->nn.accepted, 0, sizeof(int) * 256, c->s));
   }
@@ -1574,7 +1574,7 @@ int pasm_nn_setup(pasm_ctx* c, const int32_t* nx, const float* weights) {
   nn.t = 0;
   // V-cycle use needs the n x ldk temporaries and activations of the largest grid level
   if (c->k > 0 && maxn > 0) {
-    int r = nn_ensure(c, maxn * c->ldk, maxn * c->ldk, false);
+    int r = nn_ensure(c, nn_tc_supported(c->ldk) ? 0 : maxn * c->ldk, maxn * c->ldk, false);
     if (r) return r;
   }
   nn.ready = true;
@@ -1608,14 +1608,15 @@ int pasm_nn_apply(pasm_ctx* c, int level, int k, const float* R, float* D) {
   if (!R || !D) return PASM_EINVAL;
   Scope sc(c);
   const int n = c->lv[(size_t)level].n, ldk2 = ldk_for(k);
-  r = nn_ensure(c, (int64_t)n * ldk2, (int64_t)n * ldk2, false);
+  const bool tc = c->opts.smoother == PASM_LEARNED && nn_tc_supported(ldk2);
+  r = nn_ensure(c, tc ? 0 : (int64_t)n * ldk2, (int64_t)n * ldk2, false);
   if (r) return r;
   auto& nn = c->nn;
   r = put_block_f(c, R, nn.R, n, k, ldk2);
   if (r) return r;
   NNGrid g{nn.nx[(size_t)level], nn.ny[(size_t)level], ldk2, k};
-  if (c->opts.smoother == PASM_LEARNED && nn_tc_supported(ldk2))
-    nn_forward_tc(launcher(c), g, nn.w13, nn.w2, nn.R, nn.D, nn.err);
+  if (tc)
+    nn_forward_tc(launcher(c), g, &nn.w13, nullptr, nn.w2, nn.R, nn.D, nn.err);
   else
     nn_forward(launcher(c), g, nn.buf, nn.W, nn.R, nn.D);
   CK(cudaMemcpy2DAsync(D, sizeof(float) * k, nn.D, sizeof(float) * ldk2, sizeof(float) * k, n, cudaMemcpyDefault,
@@ -1633,14 +1634,18 @@ static void nn_loss_grad_dev(pasm_ctx* c, int level, int k, int ldk2) {
   // a learned-smoother context trains layer 2 on the tensor cores (the form its V-cycles run),
   // others on float32 CUDA cores
   const bool tc = c->opts.smoother == PASM_LEARNED && nn_tc_supported(ldk2);
-  if (tc) nn_forward_train_tc(L, g, nn.buf, nn.W, nn.w2f, nn.R, nn.D, nn.err);
-  else nn_forward(L, g, nn.buf, nn.W, nn.R, nn.D);
+  if (tc) {
+    nn_tc_w2_layout(L, nn.W + 144, nn.w2f, nn.w2t);
+    nn_forward_tc(L, g, nullptr, nn.W, nn.w2f, nn.R, nn.D, nn.err);
+  } else nn_forward(L, g, nn.buf, nn.W, nn.R, nn.D);
   rowop<float>(L, OP_RESID, v.A, nn.D, nn.R, nullptr, nullptr, 0.f, nn.X, ldk2);   // E = R - A D
   nn_column_norms(L, v.n, ldk2, nn.R, nn.X, nn.partial, nn.norms);
   nn_loss_seed(L, (int64_t)v.n * ldk2, ldk2, k, nn.X, nn.norms, nn.Es, nn.loss);
   rowop<float>(L, OP_SPMM, v.A, nn.Es, nullptr, nullptr, nullptr, 0.f, nn.gD, ldk2);  // dL/dD = A^T Es
-  if (tc) nn_backward_tc(L, g, nn.buf, nn.W, nn.w2t, nn.R, nn.gD, nn.grad, nn.err);
-  else nn_backward(L, g, nn.buf, nn.W, nn.R, nn.gD, nn.grad);
+  if (tc) {
+    const int rows = nn_backward_tc(L, g, nn.W, nn.w2f, nn.w2t, nn.R, nn.gD, nn.buf.wpart, nn.err);
+    nn_sum_rows(L, kNNWeights, rows, nn.buf.wpart, nn.grad);
+  } else nn_backward(L, g, nn.buf, nn.W, nn.R, nn.gD, nn.grad);
 }
 
 int pasm_nn_loss_grad(pasm_ctx* c, int level, int k, const float* R, double* loss, float* grad) {
@@ -1649,7 +1654,8 @@ int pasm_nn_loss_grad(pasm_ctx* c, int level, int k, const float* R, double* los
   if (!R) return PASM_EINVAL;
   Scope sc(c);
   const int n = c->lv[(size_t)level].n, ldk2 = ldk_for(k);
-  r = nn_ensure(c, (int64_t)n * ldk2, (int64_t)n * ldk2, true);
+  r = nn_ensure(c, c->opts.smoother == PASM_LEARNED && nn_tc_supported(ldk2) ? 0 : (int64_t)n * ldk2,
+                (int64_t)n * ldk2, true);
   if (!r) r = put_block_f(c, R, c->nn.R, n, k, ldk2);
   if (r) return r;
   nn_loss_grad_dev(c, level, k, ldk2);
@@ -1666,7 +1672,8 @@ int pasm_nn_train(pasm_ctx* c, int level, int k, const float* R, int iters, floa
   if (!R || iters < 0 || !(lr > 0.f)) return PASM_EINVAL;
   Scope sc(c);
   const int n = c->lv[(size_t)level].n, ldk2 = ldk_for(k);
-  r = nn_ensure(c, (int64_t)n * ldk2, (int64_t)n * ldk2, true);
+  r = nn_ensure(c, c->opts.smoother == PASM_LEARNED && nn_tc_supported(ldk2) ? 0 : (int64_t)n * ldk2,
+                (int64_t)n * ldk2, true);
   if (!r) r = put_block_f(c, R, c->nn.R, n, k, ldk2);
   if (r) return r;
   auto& nn = c->nn;

@@ -133,13 +133,23 @@ __global__ void k_wgrad(int nx, int ny, int ldk, int kact, const float* __restri
   for (int o = 0; o < COUT; ++o) dst[o] = acc[o];
 }
 
-// out[w] (+)= sum_b partial[b][w]  (fixed order)
-__global__ void k_wsum(int nw, int nblk, const float* __restrict__ partial, float* __restrict__ out, int accumulate) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nw) return;
+// out[w] (+)= sum_b partial[b][w]: a block owns 32 columns, its 8 warps take every 8th row and are
+// added in order (deterministic; one thread per column over all rows was one serial chain of
+// loads: 276 us of a training step's sums at h = 1/256, k = 64).
+__global__ void __launch_bounds__(256) k_wsum(int nw, int nblk, const float* __restrict__ partial,
+                                              float* __restrict__ out, int accumulate) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int t = blockIdx.x * 32 + lane;
   double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * nw + t];
-  out[t] = accumulate ? out[t] + (float)s : (float)s;
+  if (t < nw)
+    for (int b = warp; b < nblk; b += 8) s += partial[(size_t)b * nw + t];
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && t < nw) {
+    for (int q = 1; q < 8; ++q) s += red[q][lane];
+    out[t] = accumulate ? out[t] + (float)s : (float)s;
+  }
 }
 
 // Column sums of squares of two n x ldk blocks (float64 accumulation) into
@@ -167,29 +177,50 @@ __global__ void k_colnorms2(int n, int ldk, const float* __restrict__ a, const f
   }
 }
 
-__global__ void k_colsum_d(const double* __restrict__ partial, int nblk, int width, double* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= width) return;
+// out[t] = sum_b partial[b][t]: one block per column, its threads strided over the rows, then a tree
+// in fixed order (deterministic; one thread per column was one chain of n / 64 dependent additions:
+// 112 us at h = 1/256, k = 32, against 22 us for the norms it finishes).
+__global__ void __launch_bounds__(256) k_colsum_d(const double* __restrict__ partial, int nblk, int width,
+                                                  double* __restrict__ out) {
+  __shared__ double red[8];
+  const int t = blockIdx.x;
   double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * width + t];
-  out[t] = s;
+  for (int b = threadIdx.x; b < nblk; b += 256) s += partial[(size_t)b * width + t];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) s += red[q];
+    out[t] = s;
+  }
 }
 
-// Loss gradient seed: Es[p][c] = -2 E[p][c] / (k |r_c|^2)  (0 for padded pairs)
+// Loss gradient seed: Es[p][c] = -2 E[p][c] / (k |r_c|^2)  (0 for padded pairs); the column factors
+// are formed once per block (a float64 division per entry was 95 us at h = 1/256, k = 64).
 __global__ void k_loss_seed(int64_t total, int ldk, int k, const float* __restrict__ E,
                             const double* __restrict__ norms, float* __restrict__ Es) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % ldk);
-    Es[i] = c < k ? (float)(-2.0 * E[i] / ((double)k * norms[c])) : 0.f;
+  __shared__ double f[256];
+  for (int c = threadIdx.x; c < ldk; c += blockDim.x) f[c] = c < k ? -2.0 / ((double)k * norms[c]) : 0.0;
+  __syncthreads();
+  const int64_t nv = total / 4;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(4 * i % ldk);
+    const float4 e = reinterpret_cast<const float4*>(E)[i];
+    float4 o;
+    o.x = c < k ? (float)(f[c] * e.x) : 0.f;
+    o.y = c + 1 < k ? (float)(f[c + 1] * e.y) : 0.f;
+    o.z = c + 2 < k ? (float)(f[c + 2] * e.z) : 0.f;
+    o.w = c + 3 < k ? (float)(f[c + 3] * e.w) : 0.f;
+    reinterpret_cast<float4*>(Es)[i] = o;
   }
 }
 
 // L = mean_c |E_c|^2 / |R_c|^2
 __global__ void k_loss_value(int k, int ldk, const double* __restrict__ norms, double* __restrict__ loss) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double s = 0.0;
-  for (int c = 0; c < k; ++c) s += norms[ldk + c] / norms[c];
-  *loss = s / k;
+  for (int c = threadIdx.x; c < k; c += 32) s += norms[ldk + c] / norms[c];
+  s = warp_sum(s);
+  if (threadIdx.x == 0) *loss = s / k;
 }
 
 // Adam (Kingma & Ba 2015), t from 1.
@@ -261,7 +292,7 @@ static void wgrad(const Launch& L, const NNGrid& g, const NNBuf& b, const float*
   L.bump();
   const int nw = 9 * CIN * COUT;
   L.begin(KC_NN, (double)nblk * nw * 4.0, (double)nblk * nw);
-  k_wsum<<<(nw + 127) / 128, 128, 0, L.s>>>(nw, nblk, b.wpart, gw, accumulate ? 1 : 0);
+  k_wsum<<<(nw + 31) / 32, 256, 0, L.s>>>(nw, nblk, b.wpart, gw, accumulate ? 1 : 0);
   L.bump();
 }
 
@@ -300,51 +331,10 @@ void nn_backward(const Launch& L, const NNGrid& g, const NNBuf& b, const float* 
   wgrad<1, 16, IN_ID>(L, g, b, R, b.gz1, gW, false);
 }
 
-void nn_forward_train_tc(const Launch& L, const NNGrid& g, const NNBuf& b, const float* W, uint16_t* w2f,
-                         const float* R, float* Dout, int* err) {
-  const int64_t pix = (int64_t)g.nx * g.ny * g.ldk;
-  nn_tc_w2_layout(L, W + 144, false, w2f);
-  L.begin(KC_NN, (double)pix * 4.0 * 2, (double)pix * 2.0 * 9 * 16);
-  k_conv<1, 16, IN_ID><<<grid_for(pix), kNNBlock, 0, L.s>>>(g.nx, g.ny, g.ldk, g.k, W, R, b.z1);
+void nn_sum_rows(const Launch& L, int nw, int nrows, const float* partial, float* out) {
+  L.begin(KC_NN, (double)nrows * nw * 4.0, (double)nrows * nw);
+  k_wsum<<<(nw + 31) / 32, 256, 0, L.s>>>(nw, nrows, partial, out, 0);
   L.bump();
-  nn_tc_conv16(L, g, 1, w2f, b.z1, b.z2p, err);
-  nn_tc_conv16(L, g, 2, w2f, b.z1, b.z2m, err);
-  L.begin(KC_NN, (double)pix * 16 * 4.0 * 3, (double)pix * 16 * 3);
-  k_combine<<<grid_stride(pix * 16), 256, 0, L.s>>>(pix * 16, b.z2p, b.z2m, b.h);
-  L.bump();
-  L.begin(KC_NN, (double)pix * 4.0 * 17, (double)pix * 2.0 * 9 * 16);
-  k_conv<16, 1, IN_ID><<<grid_for(pix), kNNBlock, 0, L.s>>>(g.nx, g.ny, g.ldk, g.k, W + 144 + 2304, b.h, Dout);
-  L.bump();
-}
-
-void nn_backward_tc(const Launch& L, const NNGrid& g, const NNBuf& b, const float* W, uint16_t* w2t, const float* R,
-                    const float* gD, float* gW, int* err) {
-  const int64_t pix = (int64_t)g.nx * g.ny * g.ldk;
-  nn_tc_w2_layout(L, W + 144, true, w2t);
-  L.begin(KC_NN, 0, 0);
-  k_flip<<<(144 + 127) / 128, 128, 0, L.s>>>(16, 1, W + 144 + 2304, b.wflip3);
-  L.bump();
-  // layer 3 (CUDA cores, float32)
-  wgrad<16, 1, IN_ID>(L, g, b, b.h, gD, gW + 144 + 2304, false);
-  L.begin(KC_NN, 0, (double)pix * 2.0 * 9 * 16);
-  k_conv<1, 16, IN_ID><<<grid_for(pix), kNNBlock, 0, L.s>>>(g.nx, g.ny, g.ldk, g.k, b.wflip3, gD, b.gh);
-  L.bump();
-  L.begin(KC_NN, 0, 0);
-  k_combine_back<<<grid_stride(pix * 16), 256, 0, L.s>>>(pix * 16, b.gh, b.z2p, b.z2m, b.gzp, b.gzm);
-  L.bump();
-  // layer 2 on the tensor cores: weight gradient of both branches, then the input gradients
-  const int nblk = nn_tc_wgrad_ctas(g);
-  nn_tc_wgrad16(L, g, b.z1, b.gzp, b.gzm, b.wpart, err);
-  L.begin(KC_NN, (double)nblk * 2304 * 4.0, (double)nblk * 2304);
-  k_wsum<<<(2304 + 127) / 128, 128, 0, L.s>>>(2304, nblk, b.wpart, gW + 144, 0);
-  L.bump();
-  nn_tc_conv16(L, g, 0, w2t, b.gzp, b.gap, err);
-  nn_tc_conv16(L, g, 0, w2t, b.gzm, b.gam, err);
-  // layer 1 (CUDA cores, float32)
-  L.begin(KC_NN, 0, 0);
-  k_first_back<<<grid_stride(pix * 16), 256, 0, L.s>>>(pix * 16, b.gap, b.gam, b.z1, b.gz1);
-  L.bump();
-  wgrad<1, 16, IN_ID>(L, g, b, R, b.gz1, gW, false);
 }
 
 void nn_column_norms(const Launch& L, int n, int ldk, const float* a, const float* bb, double* partial,
@@ -356,14 +346,14 @@ void nn_column_norms(const Launch& L, int n, int ldk, const float* a, const floa
   k_colnorms2<<<nblk, threads, 0, L.s>>>(n, ldk, a, bb, partial, rpb);
   L.bump();
   L.begin(KC_NN, 0, 0);
-  k_colsum_d<<<(2 * ldk + 127) / 128, 128, 0, L.s>>>(partial, nblk, 2 * ldk, norms);
+  k_colsum_d<<<2 * ldk, 256, 0, L.s>>>(partial, nblk, 2 * ldk, norms);
   L.bump();
 }
 
 void nn_loss_seed(const Launch& L, int64_t total, int ldk, int k, const float* E, const double* norms, float* Es,
                   double* loss) {
   L.begin(KC_NN, (double)total * 8.0, (double)total);
-  k_loss_seed<<<grid_stride(total), 256, 0, L.s>>>(total, ldk, k, E, norms, Es);
+  k_loss_seed<<<grid_stride(total / 4), 256, 0, L.s>>>(total, ldk, k, E, norms, Es);
   L.bump();
   L.begin(KC_NN, 0, 0);
   k_loss_value<<<1, 32, 0, L.s>>>(k, ldk, norms, loss);

@@ -44,7 +44,8 @@ constexpr int kA1Bytes = 4 * kPlane;               // 2 branches x 2 halves
 constexpr int kHBytes = HR * HW * PB * 16 * 4;     // float32 h (aliases the a1 space)
 constexpr int kRBytes = RR * RW * PB * 4;
 constexpr int kW2Bytes = 9 * 512;                  // bf16, canonical K-major, per tap 2x2 core matrices
-constexpr int kSmem = kA1Bytes + kRBytes + kW2Bytes + 16;
+constexpr int kWBytes = 2 * 144 * 4;               // layers 1 and 3, float32
+constexpr int kSmem = kA1Bytes + kRBytes + kW2Bytes + kWBytes + 16;
 static_assert(kHBytes <= kA1Bytes, "h must fit in the a1 space");
 static_assert(HW * PB == 128, "one MMA block per h row");
 constexpr uint32_t kTmemCols = HR * 2 * 16;        // h rows x 2 branches x 16 columns
@@ -83,10 +84,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Layers 1 and 3 (CUDA cores) read their weights from the kernel's parameter
-// space: every FMA takes its weight as a constant-bank operand, no load.
+// DEV = false: layers 1 and 3 (CUDA cores) take their weights by value; layer 1 reads them from the
+// kernel's parameter space (every FMA takes its weight as a constant-bank operand, no load).
+// DEV = true (training, where the weights change on the device with every step): from Wd, through
+// shared memory.
+template <bool DEV>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, int ldk, int k, int tiles_x,
-                                                       const NNOuterWeights w13, const uint8_t* __restrict__ w2g,
+                                                       const NNOuterWeights w13, const float* __restrict__ Wd,
+                                                       const uint8_t* __restrict__ w2g,
                                                        const float* __restrict__ R, float* __restrict__ D,
                                                        int* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -94,7 +99,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   float* hs = reinterpret_cast<float*>(smem);                   // [HR][HW][4][PB][4] f32 (after the MMAs)
   float* rs = reinterpret_cast<float*>(smem + kA1Bytes);        // [RR][RW][PB]
   uint8_t* w2 = smem + kA1Bytes + kRBytes;                      // 9 x [2 n-groups][2 k-chunks][8][8] bf16
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(w2 + kW2Bytes);
+  float* sw1 = reinterpret_cast<float*>(w2 + kW2Bytes);         // [tap][16]
+  float* sw3 = sw1 + 144;                                       // [tap][16]
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sw3 + 144);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -110,6 +117,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   // W2, already bf16 in the canonical layout (nn_tc_layer2_layout), by 16-byte asynchronous copies
   for (int t = tid; t < kW2Bytes / 16; t += kThreads)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(w2 + 16 * t)), "l"(w2g + 16 * t));
+  if (tid < 144) {
+    if (DEV) sw1[tid] = __ldg(Wd + tid);
+    sw3[tid] = DEV ? __ldg(Wd + 144 + 2304 + tid) : w13.w3[tid];
+  }
   // residual tile with a 3-pixel halo (zero outside the grid and for padded pairs).  A block of 8
   // real pairs is one 32-byte segment per pixel: two 16-byte asynchronous copies (cp.async, all in
   // flight at once), zero-filled outside the grid; a block with padded pairs loads element-wise.
@@ -144,8 +155,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
 #pragma unroll
       for (int tap = 0; tap < 9; ++tap) {
         const float v = rs[((row + tap / 3) * RW + (col + tap % 3)) * PB + q];
+        if (DEV) {
+          const float4* w = reinterpret_cast<const float4*>(sw1 + tap * 16);
 #pragma unroll
-        for (int o = 0; o < 16; ++o) z[o] = fmaf(w13.w1[tap * 16 + o], v, z[o]);
+          for (int o = 0; o < 4; ++o) {
+            const float4 w4 = w[o];
+            z[4 * o + 0] = fmaf(w4.x, v, z[4 * o + 0]);
+            z[4 * o + 1] = fmaf(w4.y, v, z[4 * o + 1]);
+            z[4 * o + 2] = fmaf(w4.z, v, z[4 * o + 2]);
+            z[4 * o + 3] = fmaf(w4.w, v, z[4 * o + 3]);
+          }
+        } else {
+#pragma unroll
+          for (int o = 0; o < 16; ++o) z[o] = fmaf(w13.w1[tap * 16 + o], v, z[o]);
+        }
       }
     }
     const int pix = (row * AW + col) * PB + q;  // 16-byte row index inside a plane
@@ -228,26 +251,41 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
   if (!done) return;
-  // layer 3 on the 14 x 6 tile
-  for (int t = tid; t < TR * TW * PB; t += kThreads) {
-    const int q = t % PB, col = (t / PB) % TW, row = t / (PB * TW);
-    const int x = x0 + col, y = y0 + row, c = c0 + q;
-    if (x >= nx || y >= ny) continue;
-    float acc = 0.f;
+  // layer 3 on the 14 x 6 tile: a warp takes one column of the tile, a lane one channel quad of one
+  // pair; each loaded h row serves the three output rows it touches (24 16-byte shared loads for the
+  // column's 6 outputs instead of 36 per output), the quads are added by shuffles at the end
+  if (warp >= TW) return;
+  {
+    const int q = lane & 7, c4 = lane >> 3, col = warp;
+    float4 w[9];
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-      const float4* hp =
-          reinterpret_cast<const float4*>(hs + ((row + tap / 3) * HW + (col + tap % 3)) * 16 * PB + q * 4);
+    for (int tap = 0; tap < 9; ++tap) w[tap] = *reinterpret_cast<const float4*>(sw3 + tap * 16 + 4 * c4);
+    float acc[TR];
 #pragma unroll
-      for (int c4 = 0; c4 < 4; ++c4) {
-        const float4 hv = hp[c4 * PB];
-        acc = fmaf(w13.w3[tap * 16 + 4 * c4 + 0], hv.x, acc);
-        acc = fmaf(w13.w3[tap * 16 + 4 * c4 + 1], hv.y, acc);
-        acc = fmaf(w13.w3[tap * 16 + 4 * c4 + 2], hv.z, acc);
-        acc = fmaf(w13.w3[tap * 16 + 4 * c4 + 3], hv.w, acc);
+    for (int i = 0; i < TR; ++i) acc[i] = 0.f;
+#pragma unroll
+    for (int row = 0; row < HR; ++row)
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx) {
+        const float4 hv = *reinterpret_cast<const float4*>(hs + ((row * HW + col + dx) * 4 + c4) * PB * 4 + q * 4);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const int i = row - dy;
+          if (i < 0 || i >= TR) continue;
+          acc[i] = fmaf(w[dy * 3 + dx].x, hv.x, acc[i]);
+          acc[i] = fmaf(w[dy * 3 + dx].y, hv.y, acc[i]);
+          acc[i] = fmaf(w[dy * 3 + dx].z, hv.z, acc[i]);
+          acc[i] = fmaf(w[dy * 3 + dx].w, hv.w, acc[i]);
+        }
       }
+    const int x = x0 + col, c = c0 + q;
+#pragma unroll
+    for (int i = 0; i < TR; ++i) {
+      float a = acc[i];
+      a += __shfl_xor_sync(0xffffffffu, a, 8);
+      a += __shfl_xor_sync(0xffffffffu, a, 16);
+      if (c4 == 0 && x < nx && y0 + i < ny) D[((int64_t)(y0 + i) * nx + x) * ldk + c] = c < k ? a : 0.f;
     }
-    D[((int64_t)y * nx + x) * ldk + c] = c < k ? acc : 0.f;
   }
 }
 
@@ -270,18 +308,25 @@ void nn_tc_layer2_layout(const float* W2, uint16_t* out) {
 }
 
 cudaError_t nn_tc_prepare() {
-  return cudaFuncSetAttribute(k_nn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaError_t e = cudaFuncSetAttribute(k_nn_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_nn_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  return e;
 }
 
 bool nn_tc_supported(int ldk) { return ldk % PB == 0; }
 
-void nn_forward_tc(const Launch& L, const NNGrid& g, const NNOuterWeights& w13, const void* w2, const float* R,
-                   float* D, int* err) {
+void nn_forward_tc(const Launch& L, const NNGrid& g, const NNOuterWeights* w13, const float* W, const void* w2,
+                   const float* R, float* D, int* err) {
   const int tiles_x = (g.nx + TW - 1) / TW, tiles_y = (g.ny + TR - 1) / TR;
   dim3 grid(tiles_x * tiles_y, g.ldk / PB);
   const double pix = (double)g.nx * g.ny * g.ldk;
   L.begin(KC_NN, pix * 8.0, pix * 2.0 * (2 * 9 * 16 + 2 * 9 * 256 + 9 * 16));
-  k_nn_tc<<<grid, kThreads, kSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, w13, (const uint8_t*)w2, R, D, err);
+  if (w13)
+    k_nn_tc<false><<<grid, kThreads, kSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, *w13, nullptr,
+                                                   (const uint8_t*)w2, R, D, err);
+  else
+    k_nn_tc<true><<<grid, kThreads, kSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, NNOuterWeights{}, W,
+                                                  (const uint8_t*)w2, R, D, err);
   L.bump();
 }
 

@@ -1,30 +1,35 @@
-// Training kernels of the learned post-smoother's 16 -> 16 layer on the
-// 5th-generation tensor cores (tcgen05, sm_103a): bf16 operands, float32
-// accumulation in TMEM, one elected thread issuing the MMAs.
+// Training of the learned post-smoother on the 5th-generation tensor cores
+// (tcgen05, sm_103a): the whole backward pass of the network in one kernel, every
+// activation and every intermediate gradient on chip.
 //
-//   k_tc_conv16  out = W (*) tf(in) for 16 input and 16 output channels
-//                (3 x 3 taps, zero padding): the training forward of layer 2
-//                (tf = relu or relu of the negation, giving z2+ and z2-) and
-//                its input gradient (tf = identity, W = the flipped and
-//                channel-transposed kernel, giving dL/da1+-).  Implicit GEMM as
-//                in the fused inference kernel: per output row of a 16 x 8
-//                tile, M = 128 rows (16 pixels x 8 pairs), N = 16, K = 16 per
-//                tap, 9 taps accumulated in TMEM; the tap shift is a shift of
-//                the A operand's start address.
-//   k_tc_wgrad16 per-CTA partial weight gradient of layer 2 for both branches,
-//                gW[tap][ci][co] = sum over (pixel, pair) of
-//                a+-[pixel + tap][pair][ci] * g+-[pixel][pair][co]:
-//                D[ci][co] += A[ci][k] B[co][k] with K = (pixel, pair) of the
-//                tile, 8 pairs of one pixel per 16-byte K chunk, so that the
-//                tap shift is again a start-address shift (one pixel = 256 B).
-//                M = 128 with rows 0..15 the real ci; rows 16..127 read the
-//                next pixels' data (in bounds, results unused).
+// k_tc_back, a persistent CTA per SM, walks tiles of 14 x 6 pixels x 8 pairs.  From the
+// residual r (tile + 3 pixels) and gD = dL/dN (tile + 2) it forms, per tile,
+//   a+- = bf16(relu(+-z1)), z1 = W1 * r           (tile + 2, CUDA cores, float32)
+//   z2+- = W2 * a+-                               (tile + 1, MMA)
+//   gh = W3^T * gD, h = (relu(z2+) - relu(z2-))/2 (CUDA cores, float32)
+//   g+- = bf16(+-gh / 2 where z2+- > 0)           (tile + 1)
+//   ga+- = W2^T * g+-                             (tile, MMA)
+//   gz1 = ga+ [z1 > 0] - ga- [z1 < 0]             (tile, float32)
+// and adds to the weight gradients, each summed over the tile's own pixels p:
+//   gW1[tap] += r[p + tap] gz1[p],  gW3[tap] += h[p] gD[p - tap]   (CUDA cores, float32)
+//   gW2[tap] += a+[p + tap] g+[p] + a-[p + tap] g-[p]              (MMA, in TMEM across tiles)
 //
-// Activations and gradients are float32 [pixel][pair][16 channels] in global
-// memory (the CUDA-core kernels' layout); they are rounded to bf16 (nearest
-// even) when staged in shared memory.  Every mbarrier wait is bounded; a wait
-// that gives up increments an error counter, the kernel skips what depends on
-// it and frees its TMEM.
+// One layout serves the three MMA products: [branch][pixel][channel half][pair][8 channels]
+// bf16, 256 bytes a pixel.  As the convolutions' A operand it is K-major (K = channels, rows =
+// pixel x 8 + pair; 8-row groups 256 B apart, the two channel halves 128 B); as both operands of
+// the weight gradient it is MN-major (K = pixel x 8 + pair, 256 B apart; 8-channel groups 128 B),
+// and since groups 128 B apart run on into the next pixel, the 128 M rows are the 16 channels of 8
+// consecutive pixels: rows 0..47 are the taps dx = 0, 1, 2 of one dy (the others are not used).
+// So a K step (two pixels) takes 6 MMAs (3 dy x 2 branches) instead of one per tap and branch.
+//
+// What bounds it: the phases of a tile are serial (one CTA fills the SM's shared memory), the
+// tensor pipe and the float32 pipe taking turns.  Before it, the backward pass went through HBM
+// with 13 launches and about 20 passes over [pixel][pair][16] float32 activations, and layers 1 and
+// 3 summed their weight gradients with 9 and 144 threads a block.  Loss and gradient at h = 1/256,
+// k = 64 (all kernels): 9.91 ms before, 1.44 ms with this kernel and the fused forward.
+//
+// Every mbarrier wait is bounded; a wait that gives up increments an error counter, the kernel
+// stops walking tiles, contributes zeros and frees its TMEM.
 #include "common.cuh"
 #include "smoother.cuh"
 
@@ -34,32 +39,39 @@
 namespace pasm {
 namespace {
 
-constexpr int PB = 8;                    // pairs per CTA
-constexpr int TW = 16, TR = 8;           // output tile of the convolution: 16 x 8 pixels
-constexpr int IW = TW + 2, IR = TR + 2;  // input tile with its halo: 18 x 10
-constexpr int kThreads = 256;
+constexpr int PB = 8;                    // pairs per tile
+constexpr int TW = 14, TR = 6;           // tile (pixels)
+constexpr int HW = TW + 2, HR = TR + 2;  // z2, g+-: 16 x 8 (one 128-row MMA block per row)
+constexpr int AW = TW + 4, AR = TR + 4;  // a+-, gD: 18 x 10
+constexpr int RW = TW + 6, RR = TR + 6;  // r: 20 x 12
+constexpr int kThreads = 512;
+constexpr int kGroups = kThreads / 128;  // pixel groups of the layer 1 and 3 weight gradients
 constexpr int kWaitLimit = 1 << 22;
+constexpr int kCtas = kMaxBackRows;      // persistent: one per SM
 
-// conv: A operand [half][IR][IW][PB][8 channels] bf16; weights 9 x 512 B
-constexpr int kConvPlane = IR * IW * PB * 16;     // bytes of one channel half
-constexpr int kConvHalf = kConvPlane + 64;        // distance of the two halves (bank offset)
-constexpr int kConvA = kConvHalf + kConvPlane;
-constexpr int kConvW = 9 * 512;
-constexpr int kConvSmem = kConvA + kConvW + 16;
-constexpr uint32_t kConvTmem = TR * 16;           // 128 columns
-
-// wgrad: per pixel [c/8][c%8][PB] bf16 = 256 B; a on the 18 x 10 halo tile, g on the
-// same indexing (only the 16 x 8 interior is used), each with 8 pixels of slack for the
-// padding rows of the M = 128 operand (groups 2..15 of 8 rows at 128 B steps)
-constexpr int kPix = IR * IW;
-constexpr int kSlackPix = 8;
-constexpr int kWgArr = (kPix + kSlackPix) * 256;
-constexpr int kWgSmem = 2 * kWgArr + 16;
-constexpr uint32_t kWgTmem = 256;                 // 9 taps x 16 columns, rounded up
-constexpr int kWgradCtas = 2 * 152;               // persistent: two CTAs per SM
+constexpr int kPix = 256;                           // bytes of one pixel of one branch
+constexpr int kABranch = AR * AW * kPix;
+constexpr int kGBranch = HR * HW * kPix;
+constexpr int kABytes = 2 * kABranch;
+constexpr int kGBytes = 2 * kGBranch + 2 * kPix;    // 2 pixels of slack: the last row's unused outputs read on
+constexpr int kFBytes = TR * TW * PB * 16 * 4;      // h, then gz1: [pixel][pair][16] float32
+constexpr int kRBytes = RR * RW * PB * 4;
+constexpr int kDBytes = AR * AW * PB * 4;
+constexpr int kW2Bytes = 9 * 512;                   // bf16, canonical K-major, per tap 2x2 core matrices
+constexpr int kWBytes = 2 * 144 * 4;                // layers 1 and 3
+constexpr int kSmem = kABytes + kGBytes + kFBytes + kRBytes + kDBytes + 2 * kW2Bytes + kWBytes + 64;
+static_assert(kSmem <= 227 * 1024, "one CTA per SM");
+static_assert(HW * PB == 128, "one MMA block per row");
+// the weight gradient's M rows reach 7 pixels past the last K pixel of the last tap row
+static_assert((TR + 2) * AW + TW + 7 < AR * AW, "M rows of the weight gradient stay inside the operand");
+constexpr uint32_t kTmemCols = 512;                 // 256 of z2 / ga, 48 of gW2
+constexpr uint32_t kTmemW = HR * 2 * 16;            // first column of gW2
+static_assert(kThreads * 9 * 4 <= kABytes, "the final reduction reuses the operand space");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// Shared-memory matrix descriptor, no swizzle.  K-major: lbo = distance of the two 8-element K
+// chunks, sbo = of 8-row groups; MN-major: lbo = distance of 8-element K groups, sbo = of 8-row groups.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr >> 4) & 0x3FFF);
@@ -69,15 +81,17 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
   return d;
 }
 
-// kind::f16, D f32, A and B bf16, both K-major, N = 16, M = 128
+// kind::f16, D f32, A and B bf16, N = 16, M = 128; K-major operands, or both MN-major (bits 15, 16)
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(16 >> 3) << 17) |
                             ((uint32_t)(128 >> 4) << 24);
+constexpr uint32_t kIdescMN = kIdesc | (1u << 15) | (1u << 16);
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                         uint32_t accumulate) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate));
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
@@ -107,283 +121,404 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-template <int MODE>
-__device__ __forceinline__ float tf(float v) {
-  if (MODE == 1) return fmaxf(v, 0.f);
-  if (MODE == 2) return fmaxf(-v, 0.f);
-  return v;
-}
-
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols));
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
 }
 
-// out[p][c][co] = sum_{tap, ci} W[tap][ci][co] tf(in[p + tap][c][ci]); w2g = W in the canonical bf16
-// operand layout (nn_tc_w2_layout); pairs c >= k and pixels outside the grid read as 0.
-template <int MODE>
-__global__ void __launch_bounds__(kThreads) k_tc_conv16(int nx, int ny, int ldk, int k, int tiles_x,
-                                                        const uint8_t* __restrict__ w2g, const float* __restrict__ in,
-                                                        float* __restrict__ out, int* __restrict__ err) {
-  extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t* A = smem;
-  uint8_t* W = smem + kConvA;
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(W + kConvW);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int tx = blockIdx.x % tiles_x, ty = blockIdx.x / tiles_x;
-  const int x0 = tx * TW, y0 = ty * TR, c0 = blockIdx.y * PB;
-
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
-  if (warp == 0) tmem_alloc(tmem_slot, kConvTmem);
-  for (int t = tid; t < kConvW / 16; t += kThreads)
-    *reinterpret_cast<uint4*>(W + 16 * t) = __ldg(reinterpret_cast<const uint4*>(w2g) + t);
-  // input tile: thread item = (pixel, pair, channel half): 8 floats (32 contiguous bytes; two
-  // consecutive threads read the two halves of one (pixel, pair)) -> 8 bf16, one 16-byte row of
-  // the half's plane.  The planes are kConvPlane + 64 bytes apart, so the two halves that one
-  // group of 8 threads stores fall on different banks.
-  for (int t = tid; t < IR * IW * PB * 2; t += kThreads) {
-    const int half = t & 1, pp = t >> 1;
-    const int q = pp % PB, pix = pp / PB;
-    const int col = pix % IW, row = pix / IW;
-    const int x = x0 - 1 + col, y = y0 - 1 + row, c = c0 + q;
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (x >= 0 && x < nx && y >= 0 && y < ny && c < k) {
-      const float4* src = reinterpret_cast<const float4*>(in + (((int64_t)y * nx + x) * ldk + c) * 16 + half * 8);
-      a = __ldg(src);
-      b = __ldg(src + 1);
+// 8 pairs of a [pixel][ldk] float32 grid vector on a tile (height x width pixels from (x0, y0)), zero
+// outside the grid and for pairs c >= k: asynchronous 16-byte copies where all 8 pairs are real.
+__device__ __forceinline__ void load_tile(const float* __restrict__ src, int nx, int ny, int ldk, int k, int x0,
+                                          int y0, int c0, int height, int width, float* dst) {
+  if (c0 + PB <= k) {
+    for (int t = threadIdx.x; t < height * width * 2; t += kThreads) {
+      const int hlf = t & 1, col = (t >> 1) % width, row = (t >> 1) / width;
+      const int x = x0 + col, y = y0 + row;
+      const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+      const float* s = in ? src + ((int64_t)y * nx + x) * ldk + c0 + 4 * hlf : src;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst + (row * width + col) * PB + 4 * hlf)),
+                   "l"(s), "r"(in ? 16 : 0));
     }
-    __align__(16) __nv_bfloat162 v[4];
-    v[0] = __floats2bfloat162_rn(tf<MODE>(a.x), tf<MODE>(a.y));
-    v[1] = __floats2bfloat162_rn(tf<MODE>(a.z), tf<MODE>(a.w));
-    v[2] = __floats2bfloat162_rn(tf<MODE>(b.x), tf<MODE>(b.y));
-    v[3] = __floats2bfloat162_rn(tf<MODE>(b.z), tf<MODE>(b.w));
-    *reinterpret_cast<uint4*>(A + half * kConvHalf + pp * 16) = *reinterpret_cast<uint4*>(v);
+  } else {
+    for (int t = threadIdx.x; t < height * width * PB; t += kThreads) {
+      const int q = t % PB, col = (t / PB) % width, row = t / (PB * width);
+      const int x = x0 + col, y = y0 + row, c = c0 + q;
+      float v = 0.f;
+      if (x >= 0 && x < nx && y >= 0 && y < ny && c < k) v = src[((int64_t)y * nx + x) * ldk + c];
+      dst[t] = v;
+    }
   }
-  asm volatile("fence.proxy.async.shared::cta;");
+}
+
+// acc[tap] += v[p] w[p + s (tap - centre)] over this thread's pixels of the tile: v = h or gz1
+// ([pixel][pair][16], thread = one channel and pair), w a scalar tile `ww` wide whose pixel (off, off)
+// is the tile's first.  Thread group g takes every kGroups-th run of 7 pixels; the 3 x 3 window of w
+// slides along the run.
+template <int S>
+__device__ __forceinline__ void tap_sums(const float* v, const float* w, int ww, int off, int c, int q, int g,
+                                         float (&acc)[9]) {
+  for (int seg = g; seg < TR * 2; seg += kGroups) {
+    const int i = seg >> 1, j0 = (seg & 1) * (TW / 2);
+    const float* wr = w + ((off + i - 1) * ww + off + j0 - 1) * PB + q;
+    float win[3][3];
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+      for (int dx = 0; dx < 2; ++dx) win[dy][dx + 1] = wr[(dy * ww + dx) * PB];
+#pragma unroll
+    for (int j = 0; j < TW / 2; ++j) {
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy) {
+        win[dy][0] = win[dy][1];
+        win[dy][1] = win[dy][2];
+        win[dy][2] = wr[(dy * ww + j + 2) * PB];
+      }
+      const float x = v[((i * TW + j0 + j) * PB + q) * 16 + c];
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const int tap = S > 0 ? dy * 3 + dx : 8 - (dy * 3 + dx);
+          acc[tap] = fmaf(x, win[dy][dx], acc[tap]);
+        }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    k_tc_back(int nx, int ny, int ldk, int k, int tiles_x, int tiles_xy, int n_tiles, const float* __restrict__ W,
+              const uint8_t* __restrict__ w2f, const uint8_t* __restrict__ w2t, const float* __restrict__ R,
+              const float* __restrict__ gD, float* __restrict__ partial, int* __restrict__ err) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint8_t* sa = smem;                                        // a+-
+  uint8_t* sg = sa + kABytes;                                // g+-
+  float* sf = reinterpret_cast<float*>(sg + kGBytes);        // h, then gz1
+  float* sr = sf + kFBytes / 4;
+  float* sd = sr + kRBytes / 4;
+  uint8_t* sw2f = reinterpret_cast<uint8_t*>(sd + kDBytes / 4);
+  uint8_t* sw2t = sw2f + kW2Bytes;
+  float* sw1 = reinterpret_cast<float*>(sw2t + kW2Bytes);    // [tap][16]
+  float* sw3 = sw1 + 144;                                    // [tap][16]
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sw3 + 144);   // z2, ga, gW2
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 3);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  if (tid == 0) {
+    for (int b = 0; b < 3; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + b)));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
+  for (int t = tid; t < kW2Bytes / 16; t += kThreads) {
+    reinterpret_cast<uint4*>(sw2f)[t] = __ldg(reinterpret_cast<const uint4*>(w2f) + t);
+    reinterpret_cast<uint4*>(sw2t)[t] = __ldg(reinterpret_cast<const uint4*>(w2t) + t);
+  }
+  for (int t = tid; t < 288; t += kThreads) sw1[t] = __ldg(W + (t < 144 ? t : t + 2304));
+  for (int t = tid; t < 2 * kPix / 16; t += kThreads)
+    reinterpret_cast<uint4*>(sg + 2 * kGBranch)[t] = make_uint4(0, 0, 0, 0);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
-  if (tid == 0) {
-    const uint64_t a0 = smem_desc(smem_u32(A), kConvHalf, PB * 16);
-    const uint64_t b0 = smem_desc(smem_u32(W), 128, 256);
-    for (int i = 0; i < TR; ++i) {
-      const uint64_t ai = a0 + (uint64_t)((i * IW * PB * 16) >> 4);
+
+  // epilogue mapping: TMEM lane m = pixel j x 8 + pair q of a row; rows i = rowgrp, rowgrp + 4
+  const int quarter = warp & 3, rowgrp = warp >> 2;
+  const int m = quarter * 32 + lane, ej = m / PB, eq = m % PB;
+  const uint32_t lanebase = tmem + ((uint32_t)(quarter * 32) << 16);
+  // weight-gradient mapping of layers 1 and 3: channel, pair, pixel group
+  const int wc = tid & 15, wq = (tid >> 4) & 7, wg = tid >> 7;
+  float acc1[9], acc3[9];
+#pragma unroll
+  for (int t = 0; t < 9; ++t) acc1[t] = acc3[t] = 0.f;
+
+  bool ok = true;
+  uint32_t walked = 0, phase = 0;
+  int pending = 0;   // barriers with MMAs in flight
+  for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x, ++walked) {
+    phase = walked & 1u;
+    const int txy = tile % tiles_xy, c0 = (tile / tiles_xy) * PB;
+    const int x0 = (txy % tiles_x) * TW, y0 = (txy / tiles_x) * TR;
+    load_tile(R, nx, ny, ldk, k, x0 - 3, y0 - 3, c0, RR, RW, sr);
+    load_tile(gD, nx, ny, ldk, k, x0 - 2, y0 - 2, c0, AR, AW, sd);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // layer 1: a+- as bf16 on the tile + 2, zero outside the grid
+    for (int t = tid; t < AR * AW * PB; t += kThreads) {
+      const int q = t % PB, pix = t / PB, col = pix % AW, row = pix / AW;
+      const int x = x0 - 2 + col, y = y0 - 2 + row;
+      float z[16];
+#pragma unroll
+      for (int o = 0; o < 16; ++o) z[o] = 0.f;
+      if (x >= 0 && x < nx && y >= 0 && y < ny) {
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          const float v = sr[((row + tap / 3) * RW + (col + tap % 3)) * PB + q];
+          const float4* w = reinterpret_cast<const float4*>(sw1 + tap * 16);
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            const float4 w4 = w[o];
+            z[4 * o + 0] = fmaf(w4.x, v, z[4 * o + 0]);
+            z[4 * o + 1] = fmaf(w4.y, v, z[4 * o + 1]);
+            z[4 * o + 2] = fmaf(w4.z, v, z[4 * o + 2]);
+            z[4 * o + 3] = fmaf(w4.w, v, z[4 * o + 3]);
+          }
+        }
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        __align__(16) __nv_bfloat162 vp[4], vm[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const float za = z[half * 8 + 2 * o], zb = z[half * 8 + 2 * o + 1];
+          vp[o] = __floats2bfloat162_rn(fmaxf(za, 0.f), fmaxf(zb, 0.f));
+          vm[o] = __floats2bfloat162_rn(fmaxf(-za, 0.f), fmaxf(-zb, 0.f));
+        }
+        uint8_t* dst = sa + pix * kPix + half * 128 + q * 16;
+        *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<uint4*>(vp);
+        *reinterpret_cast<uint4*>(dst + kABranch) = *reinterpret_cast<uint4*>(vm);
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (tid == 0) {
+      const uint64_t a0 = smem_desc(smem_u32(sa), 128, kPix);
+      const uint64_t b0 = smem_desc(smem_u32(sw2f), 128, 256);
+      for (int i = 0; i < HR; ++i)
+        for (int b = 0; b < 2; ++b) {
+          const uint64_t ai = a0 + (uint64_t)((b * kABranch + i * AW * kPix) >> 4);
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap)
+            mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), ai + (uint64_t)(((tap / 3 * AW + tap % 3) * kPix) >> 4),
+                     b0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
+        }
+      mma_commit(mbar);
+    }
+    pending = 1;
+    // gh for this thread's two rows while the MMAs run: (W3^T * gD), float32
+    float gh[2][16];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int i = rowgrp + 4 * e;
+#pragma unroll
+      for (int o = 0; o < 16; ++o) gh[e][o] = 0.f;
 #pragma unroll
       for (int tap = 0; tap < 9; ++tap) {
-        const int dy = tap / 3, dx = tap % 3;
-        mma_bf16(tmem + (uint32_t)(i * 16), ai + (uint64_t)(((dy * IW + dx) * PB * 16) >> 4),
-                 b0 + (uint64_t)(tap * 512 >> 4), tap > 0 ? 1u : 0u);
+        const float v = sd[((i + tap / 3) * AW + (ej + tap % 3)) * PB + eq];
+        const float4* w = reinterpret_cast<const float4*>(sw3 + (8 - tap) * 16);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          const float4 w4 = w[o];
+          gh[e][4 * o + 0] = fmaf(w4.x, v, gh[e][4 * o + 0]);
+          gh[e][4 * o + 1] = fmaf(w4.y, v, gh[e][4 * o + 1]);
+          gh[e][4 * o + 2] = fmaf(w4.z, v, gh[e][4 * o + 2]);
+          gh[e][4 * o + 3] = fmaf(w4.w, v, gh[e][4 * o + 3]);
+        }
       }
     }
-    mma_commit(mbar);
-  }
-  const bool done = mbar_wait(mbar, 0);
-  if (!done && tid == 0) atomicAdd(err, 1);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (done) {
-    // TMEM lane m = pixel j * 8 + pair q of an output row; warp w reads lane quarter w % 4,
-    // rows i = w / 4, w / 4 + 2, ...
-    const int quarter = warp & 3;
-    const int m = quarter * 32 + lane;
-    const int j = m / PB, q = m % PB;
-    for (int i = warp >> 2; i < TR; i += kThreads / 128) {
-      float v[16];
-      tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(i * 16), v);
-      asm volatile("tcgen05.wait::ld.sync.aligned;");
-      const int x = x0 + j, y = y0 + i, c = c0 + q;
-      if (x < nx && y < ny && c < ldk) {
-        float4* dst = reinterpret_cast<float4*>(out + (((int64_t)y * nx + x) * ldk + c) * 16);
-        const bool real = c < k;
+    ok = mbar_wait(mbar, phase);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (ok) {
 #pragma unroll
-        for (int o = 0; o < 4; ++o)
-          dst[o] = real ? make_float4(v[4 * o], v[4 * o + 1], v[4 * o + 2], v[4 * o + 3])
-                        : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kConvTmem));
-}
-
-// Stage one (pixel, channel) row of 8 pairs of a [pixel][pair][16] float32 tensor as 8 bf16
-// values at dst (pixel-major, [c/8][c%8][pair]); MODE as tf; 0 outside the grid or past k.
-template <int MODE>
-__device__ __forceinline__ void stage_row(const float* __restrict__ src, int nx, int ny, int ldk, int k, int x,
-                                          int y, int c0, int ch, uint8_t* dst) {
-  float v[8];
+      for (int e = 0; e < 2; ++e) {
+        const int i = rowgrp + 4 * e;
+        float vp[16], vm[16];
+        tmem_ld16(lanebase + (uint32_t)((i * 2 + 0) * 16), vp);
+        tmem_ld16(lanebase + (uint32_t)((i * 2 + 1) * 16), vm);
+        asm volatile("tcgen05.wait::ld.sync.aligned;");
+        const int x = x0 - 1 + ej, y = y0 - 1 + i;
+        const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
+        if (i >= 1 && i <= TR && ej >= 1 && ej <= TW) {   // h on the tile's own pixels
+          float4* dst = reinterpret_cast<float4*>(sf + (((i - 1) * TW + ej - 1) * PB + eq) * 16);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = 0.f;
-  if (x >= 0 && x < nx && y >= 0 && y < ny) {
-    const float* p = src + (((int64_t)y * nx + x) * ldk + c0) * 16 + ch;
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (c0 + q < k) v[q] = tf<MODE>(__ldg(p + q * 16));
-  }
-  __align__(16) __nv_bfloat162 b[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) b[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-  *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<uint4*>(b);
-}
-
-// Partial weight gradient of layer 2, both branches, by a persistent CTA that walks the
-// (16 x 8 pixel, 8 pair) tiles blockIdx.x, blockIdx.x + gridDim.x, ... and accumulates in TMEM:
-// partial[cta][tap][ci][co] = sum over its tiles of a+[p+tap][ci] gp[p][co] + a-[p+tap][ci] gm[p][co],
-// a+- = bf16(relu(+-z1)), g+- = bf16(gp / gm).  The tile order per CTA is fixed, so the sums
-// are deterministic for a given grid.
-__global__ void __launch_bounds__(kThreads) k_tc_wgrad16(int nx, int ny, int ldk, int k, int tiles_x,
-                                                         int tiles_xy, int n_tiles, const float* __restrict__ z1,
-                                                         const float* __restrict__ gp, const float* __restrict__ gm,
-                                                         float* __restrict__ partial, int* __restrict__ err) {
-  extern __shared__ __align__(1024) uint8_t smem[];
-  uint8_t* Aa = smem;              // a on the halo tile
-  uint8_t* Bg = smem + kWgArr;     // g on the same pixel indexing
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + 2 * kWgArr);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
-  if (warp == 0) tmem_alloc(tmem_slot, kWgTmem);
-  // the slack pixels past the tile are read only by the unused rows: zero them once
-  for (int t = tid; t < kSlackPix * 256 / 16; t += kThreads) {
-    reinterpret_cast<uint4*>(Aa + kPix * 256)[t] = make_uint4(0, 0, 0, 0);
-    reinterpret_cast<uint4*>(Bg + kPix * 256)[t] = make_uint4(0, 0, 0, 0);
-  }
-  bool ok = true;
-  uint32_t commits = 0;
-  for (int tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
-    const int txy = tile % tiles_xy, cb = tile / tiles_xy;
-    const int x0 = (txy % tiles_x) * TW, y0 = (txy / tiles_x) * TR, c0 = cb * PB;
-    for (int br = 0; br < 2 && ok; ++br) {
-      // stage a (halo tile) and g (interior) of this branch
-      for (int t = tid; t < kPix * 16; t += kThreads) {
-        const int ch = t & 15, pix = t >> 4;
-        const int col = pix % IW, row = pix / IW;
-        const int x = x0 - 1 + col, y = y0 - 1 + row;
-        uint8_t* da = Aa + pix * 256 + (ch >> 3) * 128 + (ch & 7) * 16;
-        if (br == 0) stage_row<1>(z1, nx, ny, ldk, k, x, y, c0, ch, da);
-        else stage_row<2>(z1, nx, ny, ldk, k, x, y, c0, ch, da);
-        uint8_t* dg = Bg + pix * 256 + (ch >> 3) * 128 + (ch & 7) * 16;
-        const bool interior = col >= 1 && col <= TW && row >= 1 && row <= TR;
-        if (interior) stage_row<0>(br == 0 ? gp : gm, nx, ny, ldk, k, x, y, c0, ch, dg);
-        else *reinterpret_cast<uint4*>(dg) = make_uint4(0, 0, 0, 0);
-      }
-      asm volatile("fence.proxy.async.shared::cta;");
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      __syncthreads();
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      if (tid == 0) {
-        const uint32_t tmem = *tmem_slot;
-        // K chunk = one pixel's 8 pairs (16 B per row); an MMA (K = 16) takes two adjacent pixels
-        const uint64_t a0 = smem_desc(smem_u32(Aa), 256, 128);
-        const uint64_t g0 = smem_desc(smem_u32(Bg), 256, 128);
-        for (int i = 0; i < TR; ++i)
-          for (int jj = 0; jj < TW; jj += 2) {
-            const int P = (i + 1) * IW + (jj + 1);   // g pixel of this K step
-#pragma unroll
-            for (int tap = 0; tap < 9; ++tap) {
-              const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-              const int Pa = P + dy * IW + dx;
-              mma_bf16(tmem + (uint32_t)(tap * 16), a0 + (uint64_t)((Pa * 256) >> 4),
-                       g0 + (uint64_t)((P * 256) >> 4), (commits > 0 || i > 0 || jj > 0) ? 1u : 0u);
-            }
+          for (int o = 0; o < 4; ++o) {
+            float4 h4;
+            h4.x = in ? 0.5f * (fmaxf(vp[4 * o], 0.f) - fmaxf(vm[4 * o], 0.f)) : 0.f;
+            h4.y = in ? 0.5f * (fmaxf(vp[4 * o + 1], 0.f) - fmaxf(vm[4 * o + 1], 0.f)) : 0.f;
+            h4.z = in ? 0.5f * (fmaxf(vp[4 * o + 2], 0.f) - fmaxf(vm[4 * o + 2], 0.f)) : 0.f;
+            h4.w = in ? 0.5f * (fmaxf(vp[4 * o + 3], 0.f) - fmaxf(vm[4 * o + 3], 0.f)) : 0.f;
+            dst[o] = h4;
           }
-        mma_commit(mbar);
+        }
+        uint8_t* dg = sg + (i * HW + ej) * kPix + eq * 16;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+          __align__(16) __nv_bfloat162 gp[4], gm[4];
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            const int u = half * 8 + 2 * o;
+            gp[o] = __floats2bfloat162_rn(in && vp[u] > 0.f ? 0.5f * gh[e][u] : 0.f,
+                                          in && vp[u + 1] > 0.f ? 0.5f * gh[e][u + 1] : 0.f);
+            gm[o] = __floats2bfloat162_rn(in && vm[u] > 0.f ? -0.5f * gh[e][u] : 0.f,
+                                          in && vm[u + 1] > 0.f ? -0.5f * gh[e][u + 1] : 0.f);
+          }
+          *reinterpret_cast<uint4*>(dg + half * 128) = *reinterpret_cast<uint4*>(gp);
+          *reinterpret_cast<uint4*>(dg + half * 128 + kGBranch) = *reinterpret_cast<uint4*>(gm);
+        }
       }
-      ok = mbar_wait(mbar, commits & 1u);
-      ++commits;
-      if (!ok && tid == 0) atomicAdd(err, 1);
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      __syncthreads();   // the next staging overwrites the operands
     }
+    asm volatile("fence.proxy.async.shared::cta;");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    ok = __syncthreads_and(ok);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (!ok) break;
+    pending = 6;
+    if (tid == 0) {
+      // input gradients ga+- of the tile's rows (outputs 14, 15 of a row are not used)
+      const uint64_t g0 = smem_desc(smem_u32(sg), 128, kPix);
+      const uint64_t t0 = smem_desc(smem_u32(sw2t), 128, 256);
+      for (int i = 0; i < TR; ++i)
+        for (int b = 0; b < 2; ++b) {
+          const uint64_t gi = g0 + (uint64_t)((b * kGBranch + i * HW * kPix) >> 4);
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap)
+            mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), gi + (uint64_t)(((tap / 3 * HW + tap % 3) * kPix) >> 4),
+                     t0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
+        }
+      mma_commit(mbar + 1);
+      // weight gradient: K = two pixels of the tile a step; rows = 16 channels of the pixels dx = 0..7
+      const uint64_t am = smem_desc(smem_u32(sa), kPix, 128);
+      const uint64_t gm = smem_desc(smem_u32(sg), kPix, 128);
+      for (int i = 0; i < TR; ++i)
+        for (int j = 0; j < TW; j += 2)
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            const uint64_t gj = gm + (uint64_t)((b * kGBranch + ((i + 1) * HW + j + 1) * kPix) >> 4);
+            const uint64_t aj = am + (uint64_t)((b * kABranch + ((i + 1) * AW + j + 1) * kPix) >> 4);
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy)
+              mma_bf16(tmem + kTmemW + (uint32_t)(dy * 16), aj + (uint64_t)((dy * AW * kPix) >> 4), gj, kIdescMN,
+                       (walked > 0 || i > 0 || j > 0 || b > 0) ? 1u : 0u);
+          }
+      mma_commit(mbar + 2);
+    }
+    tap_sums<-1>(sf, sd, AW, 2, wc, wq, wg, acc3);
+    __syncthreads();   // h is read: gz1 takes its place
+    ok = mbar_wait(mbar + 1, phase);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (ok) {
+      for (int i = rowgrp; i < TR; i += 4) {
+        float vp[16], vm[16];
+        tmem_ld16(lanebase + (uint32_t)((i * 2 + 0) * 16), vp);
+        tmem_ld16(lanebase + (uint32_t)((i * 2 + 1) * 16), vm);
+        asm volatile("tcgen05.wait::ld.sync.aligned;");
+        if (ej < TW) {
+          const bool in = x0 + ej < nx && y0 + i < ny;
+          const uint8_t* pa = sa + ((i + 2) * AW + ej + 2) * kPix + eq * 16;
+          float4* dst = reinterpret_cast<float4*>(sf + ((i * TW + ej) * PB + eq) * 16);
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            // the sign of z1: a+ > 0 or a- > 0 (never both)
+            const uint4 up = *reinterpret_cast<const uint4*>(pa + half * 128);
+            const uint4 um = *reinterpret_cast<const uint4*>(pa + half * 128 + kABranch);
+            const uint32_t p4[4] = {up.x, up.y, up.z, up.w}, m4[4] = {um.x, um.y, um.z, um.w};
+            float g8[8];
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+              const uint32_t mask = o & 1 ? 0xFFFF0000u : 0xFFFFu;
+              const int u = half * 8 + o;
+              g8[o] = in ? ((p4[o / 2] & mask) ? vp[u] : 0.f) - ((m4[o / 2] & mask) ? vm[u] : 0.f) : 0.f;
+            }
+            dst[half * 2] = make_float4(g8[0], g8[1], g8[2], g8[3]);
+            dst[half * 2 + 1] = make_float4(g8[4], g8[5], g8[6], g8[7]);
+          }
+        }
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    ok = __syncthreads_and(ok);
+    tap_sums<1>(sf, sr, RW, 3, wc, wq, wg, acc1);
+    // the next tile overwrites the operands
+    const bool fin = mbar_wait(mbar + 2, phase);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    ok = __syncthreads_and(ok && fin);
   }
-  const uint32_t tmem = *tmem_slot;
-  if (warp == 0) {
-    // rows 0..15 of the accumulators (TMEM lanes 0..15) hold gW[tap][ci = lane][co]; a CTA
-    // without tiles or with a failed wait contributes zeros
-    const bool have = ok && commits > 0;
+  if (!ok && tid == 0) {
+    atomicAdd(err, 1);
+    // MMAs that a wait gave up on still read shared memory: wait (bounded) before it is reused
+    for (int b = 0; b < 3; ++b)
+      if (pending >> b & 1) mbar_wait(mbar + b, phase);
+  }
+  __syncthreads();
+  // this CTA's row of partial sums, in the order of the weights; zeros without tiles or after an error
+  float* out = partial + (size_t)blockIdx.x * kNNWeights;
+  const bool have = ok && walked > 0;
+  if (warp < 2) {
+    // accumulator row dx * 16 + ci (rows 48.. unused), columns dy * 16 + co
 #pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
+    for (int dy = 0; dy < 3; ++dy) {
       float v[16];
       if (have) {
-        tmem_ld16(tmem + (uint32_t)(tap * 16), v);
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + kTmemW + (uint32_t)(dy * 16), v);
         asm volatile("tcgen05.wait::ld.sync.aligned;");
       } else {
 #pragma unroll
         for (int o = 0; o < 16; ++o) v[o] = 0.f;
       }
-      if (lane < 16) {
-        float4* dst = reinterpret_cast<float4*>(partial + (size_t)blockIdx.x * 2304 + (tap * 16 + lane) * 16);
+      const int row = warp * 32 + lane, dx = row >> 4, ci = row & 15;
+      if (dx < 3) {
+        float4* dst = reinterpret_cast<float4*>(out + 144 + ((dy * 3 + dx) * 16 + ci) * 16);
 #pragma unroll
         for (int o = 0; o < 4; ++o) dst[o] = make_float4(v[4 * o], v[4 * o + 1], v[4 * o + 2], v[4 * o + 3]);
       }
     }
   }
+  // layers 1 and 3: over the 8 pairs and the pixel groups, in a fixed order
+  float* red = reinterpret_cast<float*>(smem);   // [kThreads / 16][9][16]
+  for (int pass = 0; pass < 2; ++pass) {
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < 9; ++t) red[((tid >> 4) * 9 + t) * 16 + wc] = have ? (pass ? acc3[t] : acc1[t]) : 0.f;
+    __syncthreads();
+    if (tid < 144) {
+      float s = 0.f;
+      for (int r = 0; r < kThreads / 16; ++r) s += red[r * 144 + tid];
+      out[(pass ? 144 + 2304 : 0) + tid] = s;
+    }
+  }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kWgTmem));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 
 // Layer 2's kernel W[tap][ci][co] (float32, device) in the canonical bf16 operand layout of the
 // B matrix (row n = output channel, k = input channel, per tap two 8 x 8 core matrices along n,
-// 256 B apart, and two along k, 128 B apart); flip: the kernel of the input gradient,
-// Wt[tap][co][ci] = W[8 - tap][ci][co] (output and input channels exchanged).
-__global__ void k_tc_w2_layout(const float* __restrict__ W, int flip, uint16_t* __restrict__ out) {
+// 256 B apart, and two along k, 128 B apart), and the kernel of the input gradient,
+// Wt[tap][co][ci] = W[8 - tap][ci][co] (output and input channels exchanged), in the same layout.
+__global__ void k_tc_w2_layout(const float* __restrict__ W, uint16_t* __restrict__ fwd, uint16_t* __restrict__ flip) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2304) return;
   const int tap = t / 256, ci = (t / 16) % 16, co = t % 16;   // W index t = [tap][ci][co]
-  int otap = tap, n = co, kk = ci;
-  if (flip) { otap = 8 - tap; n = ci; kk = co; }
-  const int off = otap * 512 + (n % 8) * 16 + (n / 8) * 256 + (kk / 8) * 128 + (kk % 8) * 2;
   const __nv_bfloat16 b = __float2bfloat16_rn(W[t]);
-  out[off / 2] = *reinterpret_cast<const uint16_t*>(&b);
+  const uint16_t bits = *reinterpret_cast<const uint16_t*>(&b);
+  fwd[(tap * 512 + (co % 8) * 16 + (co / 8) * 256 + (ci / 8) * 128 + (ci % 8) * 2) / 2] = bits;
+  flip[((8 - tap) * 512 + (ci % 8) * 16 + (ci / 8) * 256 + (co / 8) * 128 + (co % 8) * 2) / 2] = bits;
 }
 
 }  // namespace
 
 cudaError_t nn_tc_train_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(k_tc_conv16<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_conv16<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_conv16<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tc_wgrad16, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
-  return e;
+  return cudaFuncSetAttribute(k_tc_back, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
 }
 
-int nn_tc_wgrad_ctas(const NNGrid& g) {
-  const int n_tiles = ((g.nx + TW - 1) / TW) * ((g.ny + TR - 1) / TR) * (g.ldk / PB);
-  return n_tiles < kWgradCtas ? n_tiles : kWgradCtas;
-}
-
-void nn_tc_w2_layout(const Launch& L, const float* W2, bool flip, uint16_t* out) {
-  L.begin(KC_NN, 2304 * 6.0, 0);
-  k_tc_w2_layout<<<(2304 + 255) / 256, 256, 0, L.s>>>(W2, flip ? 1 : 0, out);
+void nn_tc_w2_layout(const Launch& L, const float* W2, uint16_t* fwd, uint16_t* flip) {
+  L.begin(KC_NN, 2304 * 8.0, 0);
+  k_tc_w2_layout<<<(2304 + 255) / 256, 256, 0, L.s>>>(W2, fwd, flip);
   L.bump();
 }
 
-void nn_tc_conv16(const Launch& L, const NNGrid& g, int mode, const uint16_t* w2, const float* in, float* out,
-                  int* err) {
-  const int tiles_x = (g.nx + TW - 1) / TW, tiles_y = (g.ny + TR - 1) / TR;
-  dim3 grid(tiles_x * tiles_y, g.ldk / PB);
-  const double pp = (double)g.nx * g.ny * g.ldk;
-  L.begin(KC_NN, pp * 16 * 4.0 * 2, pp * 2.0 * 9 * 256);
-  const uint8_t* w = reinterpret_cast<const uint8_t*>(w2);
-  if (mode == 1) k_tc_conv16<1><<<grid, kThreads, kConvSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, w, in, out, err);
-  else if (mode == 2) k_tc_conv16<2><<<grid, kThreads, kConvSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, w, in, out, err);
-  else k_tc_conv16<0><<<grid, kThreads, kConvSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, w, in, out, err);
-  L.bump();
-}
-
-void nn_tc_wgrad16(const Launch& L, const NNGrid& g, const float* z1, const float* gp, const float* gm,
-                   float* partial, int* err) {
+int nn_backward_tc(const Launch& L, const NNGrid& g, const float* W, const uint16_t* w2f, const uint16_t* w2t,
+                   const float* R, const float* gD, float* partial, int* err) {
   const int tiles_x = (g.nx + TW - 1) / TW, tiles_y = (g.ny + TR - 1) / TR;
   const int n_tiles = tiles_x * tiles_y * (g.ldk / PB);
+  const int ctas = n_tiles < kCtas ? n_tiles : kCtas;
   const double pp = (double)g.nx * g.ny * g.ldk;
-  L.begin(KC_NN, pp * 16 * 4.0 * 3, pp * 2.0 * 2 * 9 * 256);
-  k_tc_wgrad16<<<nn_tc_wgrad_ctas(g), kThreads, kWgSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, tiles_x * tiles_y,
-                                                                 n_tiles, z1, gp, gm, partial, err);
+  L.begin(KC_NN, pp * 8.0, pp * 2.0 * (3 * 2 * 9 * 256 + 4 * 9 * 16));
+  k_tc_back<<<ctas, kThreads, kSmem, L.s>>>(g.nx, g.ny, g.ldk, g.k, tiles_x, tiles_x * tiles_y, n_tiles, W,
+                                            reinterpret_cast<const uint8_t*>(w2f), reinterpret_cast<const uint8_t*>(w2t),
+                                            R, gD, partial, err);
   L.bump();
+  return ctas;
 }
 
 }  // namespace pasm
