@@ -353,6 +353,41 @@ __device__ __forceinline__ Cand block_best(Cand c, Cand* buf) {
   return r;
 }
 
+// Sum of v over the threads before this one; total = over all of them.
+__device__ __forceinline__ int block_exclusive(int v, int* buf, int& total) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (l >= o) x += y;
+  }
+  __syncthreads();
+  if (l == 31) buf[w] = x;
+  __syncthreads();
+  int before = 0;
+  total = 0;
+  for (int q = 0; q < kSecWarps; ++q) {
+    if (q < w) before += buf[q];
+    total += buf[q];
+  }
+  __syncthreads();
+  return before + x - v;
+}
+
+__device__ __forceinline__ int block_max(int v, int* buf) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __syncthreads();
+  if (l == 0) buf[w] = v;
+  __syncthreads();
+  int r = buf[0];
+  for (int q = 1; q < kSecWarps; ++q) r = max(r, buf[q]);
+  __syncthreads();
+  return r;
+}
+
 __device__ __forceinline__ int block_min(int v, int* buf) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -381,7 +416,10 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
   const bool lead = rank == 0;  // the CTA that writes the pair's results
   const int NH = a.NH, ldk = a.ldk;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int gwarp = rank * kSecWarps + warp, nwarps = cs * kSecWarps;  // warps of the cluster
+  // warps of the cluster, neighbours on different CTAs: the 8 roots of the first window then run on
+  // 8 / cs warps of every SM's float64 pipe instead of 8 of one (216 -> 87 us at N_H = 361, k = 37 with
+  // the block-wide pole lists below)
+  const int gwarp = warp * cs + rank, nwarps = cs * kSecWarps;
   if (!a.active[i]) {
     if (tid == 0 && lead) a.upd[i] = 0;
     return;
@@ -426,55 +464,77 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
   const double scale = fmax(fmax(fabs(S.d[NH - 1]), fabs(rho)), sqrt(zz));
   const double tolz = 8.0 * DBL_EPSILON * scale;
   const double lam_prev = a.lam[i];
-  if (tid == 0) {
-    // poles: indices with |z_j| > tolz.  Two poles closer than told (an exact
-    // coarse degeneracy) are merged by a rotation in their plane: the second
-    // carries the weight z_a^2 + z_b^2, and the first becomes a deflated root at
-    // the same lambda with eigenvector (z_b e_a - z_a e_b) / r.
-    const double told = 64.0 * DBL_EPSILON * fabs(S.d[NH - 1]);
-    int nJ = 0, nK = 0, m0 = 0;
-    bool last_merged = false;
-    double zj2 = 0.0, dmin = 0.0, dmax = 0.0;
-    for (int j = 0; j < NH; ++j) {
+  // poles: indices with |z_j| > tolz.  Two neighbouring poles closer than told (an exact coarse
+  // degeneracy) are merged by a rotation in their plane: the second carries the weight z_a^2 + z_b^2,
+  // and the first becomes a deflated root at the same lambda with eigenvector (z_b e_a - z_a e_b) / r.
+  // In a chain of close poles every second one merges with its predecessor, so a pole merges if its
+  // distance from the chain's start is odd; the lists K and J are compacted by block scans (one
+  // thread walking the N_H indices took a quarter of the kernel).
+  const double told = 64.0 * DBL_EPSILON * fabs(S.d[NH - 1]);
+  int nK_all, nJ_all;
+  {
+    const int per = (NH + kSecThreads - 1) / kSecThreads, j0 = tid * per, j1 = min(NH, j0 + per);
+    int cnt = 0;
+    double zj2 = 0.0;
+    for (int j = j0; j < j1; ++j) {
       S.rot[j] = -1;
       S.pole[j] = j;
-      if (!(fabs(S.z[j]) > tolz)) continue;
-      const double wj = S.z[j] * S.z[j];
-      if (nJ > 0 && !last_merged && S.d[j] - S.d[S.J[nJ - 1]] <= told) {
-        const int pj = S.J[nJ - 1];
+      if (fabs(S.z[j]) > tolz) {
+        S.w[j] = S.z[j] * S.z[j];
+        zj2 += S.w[j];
+        ++cnt;
+      }
+    }
+    int at = block_exclusive(cnt, s_imin, nK_all);
+    for (int j = j0; j < j1; ++j)
+      if (fabs(S.z[j]) > tolz) S.K[at++] = j;
+    zj2 = block_sum(zj2, red);   // its barriers also order K before the reads below
+    const int t0 = tid * per, t1 = min(nK_all, t0 + per);
+    auto close = [&](int t) { return t > 0 && S.d[S.K[t]] - S.d[S.K[t - 1]] <= told; };
+    auto merged = [&](int t) {
+      int s = t;
+      while (close(s)) --s;
+      return ((t - s) & 1) != 0;
+    };
+    int nm = 0;
+    for (int t = t0; t < t1; ++t) nm += merged(t) ? 1 : 0;
+    int total;
+    int mb = block_exclusive(nm, s_imin, total);   // merged poles before t0
+    nJ_all = nK_all - total;
+    // weights of merged poles from the squares, read before any is replaced by a merged weight (a
+    // merged pole's predecessor is never merged itself)
+    int below = 0;
+    for (int t = t0; t < t1; ++t) {
+      const int j = S.K[t];
+      if (merged(t)) {
+        const int pj = S.K[t - 1];
         S.rot[pj] = j;
         S.pole[pj] = j;
-        S.w[j] = S.w[pj] + wj;
-        S.J[nJ - 1] = j;
-        last_merged = true;
-      } else {
-        S.w[j] = wj;
-        S.J[nJ++] = j;
-        last_merged = false;
+        S.w[j] = S.w[pj] + S.z[j] * S.z[j];
+        ++mb;
       }
-      S.K[nK++] = j;
-      zj2 += wj;
+      if (!(t + 1 < nK_all && merged(t + 1))) {   // a pole of the secular equation
+        S.J[t - mb] = j;
+        if (S.d[j] < lam_prev) below = t - mb + 1;
+      }
     }
-    for (int t = 0; t < nJ; ++t) {
-      const double dj = S.d[S.J[t]];
-      if (t == 0) dmin = dj;
-      dmax = dj;
-      if (dj < lam_prev) m0 = t + 1;
+    below = block_max(below, s_imin);
+    if (tid == 0) {
+      const int nJ = nJ_all, m0 = below;
+      const double zn = sqrt(zj2);
+      s_nJ = nJ;
+      s_nK = nK_all;
+      s_m0 = m0;
+      s_lower = (nJ ? fmin(S.d[S.J[0]], rho) : rho) - zn;
+      s_upper = (nJ ? fmax(S.d[S.J[nJ - 1]], rho) : rho) + zn;
+      // phase-1 list: root 0 and a window around the root holding lambda^(l)
+      int nl = 0;
+      s_list[nl++] = 0;
+      const int w = a.window;
+      for (int m = max(1, m0 - w); m <= min(nJ, m0 + w); ++m) s_list[nl++] = m;
+      s_nlist = nl;
+      if (lead) a.steps[i] += 1;
     }
-    const double zn = sqrt(zj2);
-    s_nJ = nJ;
-    s_nK = nK;
-    s_m0 = m0;
-    s_lower = (nJ ? fmin(dmin, rho) : rho) - zn;
-    s_upper = (nJ ? fmax(dmax, rho) : rho) + zn;
-    // phase-1 list: root 0 and a window around the root holding lambda^(l)
-    int nl = 0;
-    s_list[nl++] = 0;
-    const int w = a.window;
-    for (int m = max(1, m0 - w); m <= min(nJ, m0 + w); ++m) s_list[nl++] = m;
-    if (nl == 1 && nJ == 0) nl = 1;
-    s_nlist = nl;
-    if (lead) a.steps[i] += 1;
   }
   for (int m = tid; m <= NH; m += kSecThreads) S.solved[m] = 0;
   // every CTA of the cluster is running and initialised before any writes into its shared memory
