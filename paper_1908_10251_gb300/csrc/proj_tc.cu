@@ -24,7 +24,7 @@
 // GB300 runs float64 at 1/64 of the float32 rate, so everything around the
 // MMAs is integer work: B's exponents come from its bit fields, its digits from
 // shifts of its significands.  Grid: (16-column tiles) x (128-row tiles) x
-// (32-wide chunks of the inner dimension); 128 threads, one per TMEM lane /
+// (32-wide chunks of the inner dimension); 256 threads, two per TMEM lane /
 // output row.  A's digit planes are split once at setup, stored in the
 // canonical K-major no-swizzle operand layout, and the chunk's planes are
 // brought into shared memory by bulk asynchronous copies (cp.async.bulk,
@@ -43,13 +43,16 @@ namespace {
 constexpr int kM = 128;          // rows per tile (TMEM lanes)
 constexpr int kN = 16;           // output columns per tile (MMA N)
 constexpr int kKC = 32;          // inner-dimension chunk per CTA
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;          // two warps per TMEM lane quarter
 constexpr int kDigitBits = 7, kDigits = 8;   // 56 bits per operand
 constexpr int kGroups = kDigits;             // weights d = 2 .. S + 1
 constexpr uint32_t kTmemCols = 128;          // kGroups x kN
 constexpr int kAPlaneBytes = (kKC / 8) * 2048;           // one digit plane of a 128 x 32 A chunk
 constexpr int kBPlaneBytes = (kKC / 8) * (kN / 8) * 128;  // one digit plane of a 16 x 32 B chunk
-constexpr int kSmem = kDigits * (kAPlaneBytes + kBPlaneBytes) + 1024;
+constexpr int kStageRow = kN * 16 + 16;   // folded sums of a row, 16 bytes a column (padded against bank conflicts)
+constexpr int kTileWords = kM * kN * 2;   // 64-bit words of a tile's integer sums
+constexpr int kSmem = kDigits * (kAPlaneBytes + kBPlaneBytes) + 2048;
+static_assert(kM * kStageRow <= kDigits * kAPlaneBytes, "the folded sums reuse A's planes");
 constexpr int kWaitLimit = 1 << 22;
 static_assert(kGroups * kN <= (int)kTmemCols, "accumulators must fit in TMEM");
 static_assert((uint64_t)kGroups * kKC * 127 * 127 < (1u << 24), "group sums must be exact in float32");
@@ -75,15 +78,13 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Bounded wait for phase `parity` of an mbarrier (at most `limit` polls); true when it completed.
@@ -113,12 +114,6 @@ __device__ __forceinline__ void red_add(unsigned long long* p, long long v) {
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)v) : "memory");
 }
 
-// Exponent e with |v| < 2^e for a finite nonzero v, from its bit fields.
-__device__ __forceinline__ int bound_exponent(uint64_t bits) {
-  const int ex = (int)((bits >> 52) & 0x7FF);
-  return (ex > 0 ? ex : 1) - 1022;
-}
-
 // floor(|v| / 2^e * 2^T) for |v| < 2^e, T <= 62, from the significand of v.
 __device__ __forceinline__ uint64_t scaled_magnitude(uint64_t bits, int e, int T) {
   const int ex = (int)((bits >> 52) & 0x7FF);
@@ -128,24 +123,35 @@ __device__ __forceinline__ uint64_t scaled_magnitude(uint64_t bits, int e, int T
   return -sh < 64 ? (mant >> -sh) : 0ull;
 }
 
-// Round a signed 128-bit integer to float64 (to nearest, once) times 2^k.
+// Round a signed 128-bit integer to float64 (to nearest even, once) times 2^k: the bits are assembled
+// with integer operations where the result is a normal number (GB300's float64 pipe would take the
+// conversion, the product and ldexp of 16 outputs per thread one after another), else by ldexp.
 __device__ __forceinline__ double i128_to_double_scaled(__int128 a, int k) {
   if (a == 0) return 0.0;
   const bool neg = a < 0;
   const unsigned __int128 u = neg ? (unsigned __int128)(-a) : (unsigned __int128)a;
-  const uint64_t hi = (uint64_t)(u >> 64);
-  double d;
-  if (hi == 0) {
-    d = (double)(uint64_t)u;
+  const uint64_t hi = (uint64_t)(u >> 64), lo = (uint64_t)u;
+  // top: the leading 64 bits (leading one at bit 63), value = top 2^drop, lower bits in a sticky bit
+  const int lz = hi ? __clzll((long long)hi) : 64 + __clzll((long long)lo);
+  uint64_t top;
+  bool sticky = false;
+  const int drop = 64 - lz;   // > 0: bits below the leading 64
+  if (drop > 0) {
+    top = (uint64_t)(u >> drop);
+    sticky = drop < 64 ? (lo << (64 - drop)) != 0 : lo != 0;
   } else {
-    const int drop = 64 - __clzll((long long)hi);              // bits below the top 64
-    const unsigned __int128 lowmask = (((unsigned __int128)1) << drop) - 1;
-    uint64_t top = (uint64_t)(u >> drop);
-    if ((u & lowmask) != 0) top |= 1ull;                       // sticky bit keeps the rounding exact
-    d = (double)top;
-    k += drop;
+    top = lo << -drop;
   }
-  d = ldexp(d, k);
+  const int e = drop + k + 63;   // |a| 2^k = 1.xxx 2^e
+  if (e > -1000 && e < 1000) {
+    uint64_t m = top >> 11;
+    const uint64_t rest = (top & 0x7FFull) << 1 | (sticky ? 1ull : 0ull);   // 12 bits; half = 0x800
+    if (rest > 0x800ull || (rest == 0x800ull && (m & 1ull))) ++m;           // 2^53 carries into the exponent
+    const uint64_t bits = ((uint64_t)(e + 1022) << 52) + m;
+    return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
+  }
+  if (sticky) top |= 1ull;
+  const double d = ldexp((double)top, k + drop);
   return neg ? -d : d;
 }
 
@@ -212,72 +218,62 @@ __global__ void __launch_bounds__(kThreads)
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
-  // column exponents over the whole inner dimension, from the bit fields:
-  // |B[j][n]| < 2^cexp[n]; a NaN/Inf marks the column.  Loads use clamped
-  // indices (always valid addresses) so that each batch is issued at once.
+  // column exponents over the whole inner dimension: |B[j][n]| < 2^cexp[n] from the largest high
+  // word (an all-zero high word with low bits set is subnormal: key 1); a NaN/Inf marks the column.
+  // Loads use clamped indices (always valid addresses) so that each batch is issued at once.
   {
     const int col = tid % kN, part = tid / kN;
     constexpr int kParts = kThreads / kN;
     const bool cv = n0 + col < ncols;
     const double* cp = bcol(B0, B1, ldk, cv ? n0 + col : 0);
-    int emax = -100000;
-    bool bad = false;
+    uint32_t hmax = 0, lor = 0;
     for (int j0 = part; j0 < K; j0 += 8 * kParts) {
-      uint64_t bits[8];
+      uint2 w[8];   // low, high word
 #pragma unroll
-      for (int q = 0; q < 8; ++q) bits[q] = ld_bits(cp + (size_t)min(j0 + q * kParts, K - 1) * ldk);
+      for (int q = 0; q < 8; ++q)
+        w[q] = __ldg(reinterpret_cast<const uint2*>(cp + (size_t)min(j0 + q * kParts, K - 1) * ldk));
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (!cv || j0 + q * kParts >= K) continue;
-        if (((bits[q] >> 52) & 0x7FF) == 0x7FF) bad = true;
-        else if ((bits[q] << 1) != 0) emax = max(emax, bound_exponent(bits[q]));
+      for (int q = 0; q < 8; ++q) {   // a clamped load repeats the last row
+        hmax = max(hmax, w[q].y & 0x7FFFFFFFu);
+        lor |= w[q].x;
       }
     }
-    red[tid] = bad ? 0x7FFFFFFF : emax;
+    red[tid] = !cv ? 0 : (int)(hmax ? hmax : (lor ? 1u : 0u));
   }
   __syncthreads();
   if (tid < kN) {
-    int emax = -100000;
-    bool bad = false;
-    for (int p = 0; p < kThreads / kN; ++p) {
-      const int v = red[p * kN + tid];
-      if (v == 0x7FFFFFFF) bad = true;
-      else emax = max(emax, v);
-    }
-    cexp[tid] = (bad || emax == -100000) ? 0 : emax;
+    int key = 0;
+    for (int p = 0; p < kThreads / kN; ++p) key = max(key, red[p * kN + tid]);
+    const bool bad = key >= 0x7FF00000;
+    cexp[tid] = (bad || key == 0) ? 0 : max(key >> 20, 1) - 1022;
     cbad[tid] = bad ? 1 : 0;
   }
   __syncthreads();
-  // B's digit planes for this chunk: item (kc8, n) slices 8 consecutive entries of column n
+  // B's digit planes for this chunk: item (kc2, n) slices 2 consecutive entries of column n
   const uint64_t dmask = (1ull << kDigitBits) - 1;
-  for (int it = tid; it < (kw / 8) * kN; it += kThreads) {
-    const int n = it % kN, kc8 = it / kN;
+  for (int it = tid; it < (kw / 2) * kN; it += kThreads) {
+    const int n = it % kN, k2 = it / kN;
     const int e = cexp[n];
     const bool cv = n0 + n < ncols && !cbad[n];
     const double* cp = bcol(B0, B1, ldk, n0 + n < ncols ? n0 + n : 0);
-    uint64_t raw[8], mag[8];
-    uint32_t neg = 0;
+    uint64_t raw[2], mag[2];
+    bool neg[2];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) raw[q] = ld_bits(cp + (size_t)min(kc0 + kc8 * 8 + q, K - 1) * ldk);
+    for (int q = 0; q < 2; ++q) raw[q] = ld_bits(cp + (size_t)min(kc0 + k2 * 2 + q, K - 1) * ldk);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint64_t bits = (cv && kc0 + kc8 * 8 + q < K) ? raw[q] : 0ull;
+    for (int q = 0; q < 2; ++q) {
+      const uint64_t bits = (cv && kc0 + k2 * 2 + q < K) ? raw[q] : 0ull;
       mag[q] = (bits << 1) ? scaled_magnitude(bits, e, T) : 0ull;
-      neg |= (uint32_t)(bits >> 63) << q;
+      neg[q] = (bits >> 63) != 0;
     }
-    const int off = kc8 * (kN / 8) * 128 + (n / 8) * 128 + (n % 8) * 16;
+    const int off = (k2 / 4) * (kN / 8) * 128 + (n / 8) * 128 + (n % 8) * 16 + (k2 % 4) * 4;
 #pragma unroll
     for (int t = 0; t < S; ++t) {
       const int sh = T - kDigitBits * (t + 1);
-      uint32_t w[4];
-#pragma unroll
-      for (int q = 0; q < 8; q += 2) {
-        int d0 = (int)((mag[q] >> sh) & dmask), d1 = (int)((mag[q + 1] >> sh) & dmask);
-        if (neg >> q & 1u) d0 = -d0;
-        if (neg >> (q + 1) & 1u) d1 = -d1;
-        w[q / 2] = bf16_bits_of_int(d0) | (bf16_bits_of_int(d1) << 16);
-      }
-      *reinterpret_cast<uint4*>(sB + t * kBPlaneBytes + off) = make_uint4(w[0], w[1], w[2], w[3]);
+      int d0 = (int)((mag[0] >> sh) & dmask), d1 = (int)((mag[1] >> sh) & dmask);
+      if (neg[0]) d0 = -d0;
+      if (neg[1]) d1 = -d1;
+      *reinterpret_cast<uint32_t*>(sB + t * kBPlaneBytes + off) = bf16_bits_of_int(d0) | (bf16_bits_of_int(d1) << 16);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;");
@@ -323,35 +319,42 @@ __global__ void __launch_bounds__(kThreads)
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  const int i = mt * kM + warp * 32 + lane;
-  if (!flag[0]) {
-    // fold the weight groups of this row exactly: H (d <= 5), L (d >= 6)
-    long long H[kN], L[kN];
+  // The tile's integer sums are [row][column][H, L], contiguous: every CTA stages its folded rows in
+  // shared memory (A's planes are read) and adds them in that order, a warp 256 contiguous bytes,
+  // and the last one reads them back the same way.  (One thread per row, 16 columns each, scattered
+  // every access over 32 rows: 18 of 40 us at N_H = 361, k = 64 were this read-back and its float64
+  // conversions, 6 us the additions.)
+  uint8_t* stage = sA;
+  unsigned long long* sums = hl + (size_t)(mt * gridDim.x + blockIdx.x) * kTileWords;
+  const bool good = !flag[0];
+  if (good) {
+    // fold the weight groups of this row exactly, 8 columns a warp: H (d <= 5), L (d >= 6)
+    const int row = (warp & 3) * 32 + lane, nb = (warp >> 2) * 8;
+    long long H[8], L[8];
 #pragma unroll
-    for (int n = 0; n < kN; ++n) H[n] = L[n] = 0;
-    const uint32_t lanebase = tmem + ((uint32_t)(warp * 32) << 16);
+    for (int n = 0; n < 8; ++n) H[n] = L[n] = 0;
+    const uint32_t lanebase = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)nb;
 #pragma unroll
     for (int g = 0; g < kGroups; ++g) {
-      float v[16];
-      tmem_ld16(lanebase + (uint32_t)(g * kN), v);
+      float v[8];
+      tmem_ld8(lanebase + (uint32_t)(g * kN), v);
       asm volatile("tcgen05.wait::ld.sync.aligned;");
       const int d = g + 2;
 #pragma unroll
-      for (int n = 0; n < kN; ++n) {
+      for (int n = 0; n < 8; ++n) {
         const long long x = (long long)__float2int_rn(v[n]);
         if (d <= 5) H[n] += x << (kDigitBits * (5 - d));
         else L[n] += x << (kDigitBits * (9 - d));
       }
     }
-    if (i < m) {
 #pragma unroll
-      for (int n = 0; n < kN; ++n) {
-        const int col = n0 + n;
-        if (col >= ncols) continue;
-        unsigned long long* q = hl + ((size_t)i * ncols + col) * 2;
-        red_add(q, H[n]);
-        red_add(q + 1, L[n]);
-      }
+    for (int n = 0; n < 8; ++n)
+      *reinterpret_cast<longlong2*>(stage + row * kStageRow + (nb + n) * 16) = make_longlong2(H[n], L[n]);
+    __syncthreads();
+    const int rows = min(kM, m - mt * kM);
+    for (int t = tid; t < rows * kN * 2; t += kThreads) {
+      const int w = t % (kN * 2);
+      if (n0 + w / 2 < ncols) red_add(sums + t, *reinterpret_cast<const long long*>(stage + (t / (kN * 2)) * kStageRow + w * 8));
     }
   }
   // the last CTA of this output tile rounds, writes and clears
@@ -364,27 +367,27 @@ __global__ void __launch_bounds__(kThreads)
   __syncthreads();
   if (flag[1]) {
     __threadfence();
-    if (i < m) {
-      const int kbase = rexp[i] - kDigitBits * (S + 1);
-      unsigned long long* row = hl + (size_t)i * ncols * 2;
-      long long h[kN], l[kN];
+    constexpr int kItems = kM * kN / kThreads;
+    ulonglong2* s2 = reinterpret_cast<ulonglong2*>(sums);
+    ulonglong2 v[kItems];
+    int re[kItems];
+    const int col = tid % kN, gc = n0 + col;   // kThreads is a multiple of kN
 #pragma unroll
-      for (int n = 0; n < kN; ++n) {
-        const int col = min(n0 + n, ncols - 1);
-        h[n] = (long long)__ldcg(row + col * 2);
-        l[n] = (long long)__ldcg(row + col * 2 + 1);
-      }
+    for (int q = 0; q < kItems; ++q) {
+      const int row = mt * kM + (tid + q * kThreads) / kN;
+      v[q] = __ldcg(s2 + tid + q * kThreads);
+      re[q] = __ldg(rexp + min(row, m - 1));
+    }
 #pragma unroll
-      for (int n = 0; n < kN; ++n) {
-        const int col = n0 + n;
-        if (col >= ncols) continue;
-        row[col * 2] = 0ull;
-        row[col * 2 + 1] = 0ull;
-        const double r = cbad[n] ? __longlong_as_double(0x7ff8000000000000LL)
-                                 : i128_to_double_scaled(((__int128)h[n] << 28) + (__int128)l[n], kbase + cexp[n]);
-        if (col < ldk) C0[(size_t)i * ldk + col] = r;
-        else C1[(size_t)i * ldk + (col - ldk)] = r;
-      }
+    for (int q = 0; q < kItems; ++q) {
+      const int row = mt * kM + (tid + q * kThreads) / kN;
+      if (row >= m || gc >= ncols) continue;
+      s2[tid + q * kThreads] = make_ulonglong2(0ull, 0ull);
+      const double r = cbad[col] ? __longlong_as_double(0x7ff8000000000000LL)
+                                 : i128_to_double_scaled(((__int128)(long long)v[q].x << 28) + (__int128)(long long)v[q].y,
+                                                         re[q] - kDigitBits * (S + 1) + cexp[col]);
+      if (gc < ldk) C0[(size_t)row * ldk + gc] = r;
+      else C1[(size_t)row * ldk + (gc - ldk)] = r;
     }
     if (tid == 0) tickets[blockIdx.y * gridDim.x + blockIdx.x] = 0u;
   }
@@ -434,8 +437,8 @@ void proj_split_host(const double* A, int m, int K, const ProjPlan& plan, int& K
   }
 }
 
-size_t proj_scratch_words(int m, int ncols_max) { return (size_t)m * ncols_max * 2; }
 size_t proj_tickets(int m, int ncols_max) { return (size_t)((m + kM - 1) / kM) * ((ncols_max + kN - 1) / kN); }
+size_t proj_scratch_words(int m, int ncols_max) { return proj_tickets(m, ncols_max) * kTileWords; }
 
 cudaError_t proj_tc_prepare() { return allow_dynamic_smem((const void*)k_proj_tc, (size_t)kSmem); }
 
