@@ -225,7 +225,9 @@ int pasm_project(pasm_ctx* ctx, const double* b, const double* c, double* bq, do
  * restriction; prolongation + sweep) on this level, which then runs instead.
  * PASM_TILE_RESTRICT_FIRST is above 0 only where the autotuner timed the
  * restriction-first form of the coarse residual, R f - (R A) e with R A formed
- * at setup, faster than both forms of R (f - A e); it then runs instead.
+ * at setup, faster than both forms of R (f - A e); it then runs instead.  It
+ * also runs where neither it nor PASM_TILE_RESID_RESTRICT has a shape (both 0:
+ * levels the autotuner leaves out, and autotune = 0), in mixed precision.
  * Errors: PASM_EINVAL. */
 int pasm_tiles(pasm_ctx* ctx, int level, int* chunks_per_thread);
 

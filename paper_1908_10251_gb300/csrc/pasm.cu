@@ -388,7 +388,12 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
   }
   bool restricted = false;
   if constexpr (std::is_same<T, float>::value) {
-    if (fuse && v.RA.rp && c->geo[(size_t)l][PASM_TILE_RESTRICT_FIRST] > 0) {
+    // restriction first where the autotuner timed it fastest, and on levels without a tuned shape (few
+    // rows, or no autotuner): there every kernel is a chain of dependent loads, and the fused form's
+    // is the longest (a fine row's index, its entries, their vectors, for each of 7 or 15 fine rows)
+    const auto& g = c->geo[(size_t)l];
+    const bool untuned = g[PASM_TILE_RESTRICT_FIRST] == 0 && g[PASM_TILE_RESID_RESTRICT] == 0;
+    if (fuse && v.RA.rp && (g[PASM_TILE_RESTRICT_FIRST] > 0 || untuned)) {
       restrict_first(launcher(c, l, PASM_TILE_RESTRICT_FIRST), v.R, v.RA, cur, F, (float*)c->lv[l - 1].vF, ldk);
       restricted = true;
     }
