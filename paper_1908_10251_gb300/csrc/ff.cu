@@ -3,7 +3,8 @@
 // (Algorithm 1 step 1), the bordering products (the bordered matrix form of
 // Section 3.1), the transfer chains and the update.  Vectors that are gathered
 // through a sparse matrix are kept as (hi, lo) float pairs ("ff", 8 bytes per
-// entry like float64): the multigrid iterate u~, its products A u~ and M u~,
+// entry like float64; two columns make one 16-byte chunk hi, hi, lo, lo, the
+// operands of the packed float32 instructions): the multigrid iterate u~, its products A u~ and M u~,
 // the intermediate levels of the transfer chains, and the state U itself
 // between steps (its float64 form is rebuilt when read).  Matrix values are
 // split once at setup; a matrix whose values are all float32 skips the
@@ -58,16 +59,19 @@ static int ff_rows(const Launch& L) { return L.rpt > 0 ? L.rpt : 1; }
   }
 
 // Two consecutive entries (columns col, col + 1) of row i of a block vector,
-// as (hi, lo) pairs: from float pairs directly, from float64 by splitting.
+// as packed hi and lo parts: from a pair chunk directly, from float64 by splitting.
 template <bool FF>
-__device__ __forceinline__ void load_pair(const double* __restrict__ X, size_t off, float (&h)[2], float (&l)[2]) {
+__device__ __forceinline__ void load_pair(const double* __restrict__ X, size_t off, ff2& h, ff2& l) {
   if (FF) {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(X + off));
-    h[0] = t.x; l[0] = t.y; h[1] = t.z; l[1] = t.w;
+    const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(X + off));
+    h = t.x; l = t.y;
   } else {
     const double2 t = __ldg(reinterpret_cast<const double2*>(X + off));
-    ff_split(t.x, h[0], l[0]);
-    ff_split(t.y, h[1], l[1]);
+    float h0, l0, h1, l1;
+    ff_split(t.x, h0, l0);
+    ff_split(t.y, h1, l1);
+    h = ff2_pack(h0, h1);
+    l = ff2_pack(l0, l1);
   }
 }
 
@@ -76,7 +80,7 @@ __device__ __forceinline__ void load_pair(const double* __restrict__ X, size_t o
 template <int CH, int N, bool FFIN, bool EX>
 __device__ __forceinline__ void gather_group_ff(const int* __restrict__ ci, const float2* __restrict__ av,
                                                 const double* __restrict__ X, int p, int lane, int tpr, int ldk,
-                                                float (&hi)[CH][2], float (&lo)[CH][2]) {
+                                                ff2 (&hi)[CH], ff2 (&lo)[CH]) {
   int j[N];
   float2 a[N];
 #pragma unroll
@@ -84,20 +88,20 @@ __device__ __forceinline__ void gather_group_ff(const int* __restrict__ ci, cons
     j[u] = __ldg(ci + p + u);
     a[u] = __ldg(av + p + u);
   }
-  float xh[N][CH][2], xl[N][CH][2];
+  ff2 xh[N][CH], xl[N][CH];
 #pragma unroll
   for (int u = 0; u < N; ++u)
 #pragma unroll
     for (int c = 0; c < CH; ++c) load_pair<FFIN>(X, (size_t)j[u] * ldk + (c * tpr + lane) * 2, xh[u][c], xl[u][c]);
 #pragma unroll
-  for (int u = 0; u < N; ++u)
+  for (int u = 0; u < N; ++u) {
+    const ff2 ah = ff2_pack(a[u].x, a[u].x), na = ff2_pack(-a[u].x, -a[u].x), al = ff2_pack(a[u].y, a[u].y);
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        if (EX) ff_mac_exact(hi[c][v], lo[c][v], a[u].x, xh[u][c][v], xl[u][c][v]);
-        else ff_mac(hi[c][v], lo[c][v], a[u].x, a[u].y, xh[u][c][v], xl[u][c][v]);
-      }
+    for (int c = 0; c < CH; ++c) {
+      if (EX) ff2_mac_exact(hi[c], lo[c], ah, na, xh[u][c], xl[u][c]);
+      else ff2_mac(hi[c], lo[c], ah, na, al, xh[u][c], xl[u][c]);
+    }
+  }
 }
 
 // One row of S X in double-float (groups of 4 entries, then an exact remainder group);
@@ -105,9 +109,9 @@ __device__ __forceinline__ void gather_group_ff(const int* __restrict__ ci, cons
 template <int CH, bool FFIN, bool EX = false>
 __device__ __forceinline__ void gather_row_ff(const int* __restrict__ rp, const int* __restrict__ ci,
                                               const float2* __restrict__ av, const double* __restrict__ X, int row,
-                                              int lane, int tpr, int ldk, float (&hi)[CH][2], float (&lo)[CH][2]) {
+                                              int lane, int tpr, int ldk, ff2 (&hi)[CH], ff2 (&lo)[CH]) {
 #pragma unroll
-  for (int c = 0; c < CH; ++c) hi[c][0] = hi[c][1] = lo[c][0] = lo[c][1] = 0.f;
+  for (int c = 0; c < CH; ++c) hi[c] = lo[c] = 0;
   int p = __ldg(rp + row);
   const int p1 = __ldg(rp + row + 1);
   for (; p + 4 <= p1; p += 4) gather_group_ff<CH, 4, FFIN, EX>(ci, av, X, p, lane, tpr, ldk, hi, lo);
@@ -116,10 +120,7 @@ __device__ __forceinline__ void gather_row_ff(const int* __restrict__ rp, const 
   else if (rem == 2) gather_group_ff<CH, 2, FFIN, EX>(ci, av, X, p, lane, tpr, ldk, hi, lo);
   else if (rem == 1) gather_group_ff<CH, 1, FFIN, EX>(ci, av, X, p, lane, tpr, ldk, hi, lo);
 #pragma unroll
-  for (int c = 0; c < CH; ++c) {
-    ff_norm(hi[c][0], lo[c][0]);
-    ff_norm(hi[c][1], lo[c][1]);
-  }
+  for (int c = 0; c < CH; ++c) ff2_norm(hi[c], lo[c]);
 }
 
 // A X and M X together over M's pattern (am: A's and M's split values per
@@ -129,8 +130,7 @@ __device__ __forceinline__ void gather_row_ff(const int* __restrict__ rp, const 
 template <int CH, int N, bool FFIN, bool AEX>
 __device__ __forceinline__ void gather_group_am(const int* __restrict__ ci, const float4* __restrict__ am,
                                                 const double* __restrict__ X, int p, int lane, int tpr, int ldk,
-                                                float (&ah)[CH][2], float (&al)[CH][2], float (&mh)[CH][2],
-                                                float (&ml)[CH][2]) {
+                                                ff2 (&ah)[CH], ff2 (&al)[CH], ff2 (&mh)[CH], ff2 (&ml)[CH]) {
   int j[N];
   float4 w[N];
 #pragma unroll
@@ -138,36 +138,36 @@ __device__ __forceinline__ void gather_group_am(const int* __restrict__ ci, cons
     j[u] = __ldg(ci + p + u);
     w[u] = __ldg(am + p + u);
   }
-  float xh[N][CH][2], xl[N][CH][2];
+  ff2 xh[N][CH], xl[N][CH];
 #pragma unroll
   for (int u = 0; u < N; ++u)
 #pragma unroll
     for (int c = 0; c < CH; ++c) load_pair<FFIN>(X, (size_t)j[u] * ldk + (c * tpr + lane) * 2, xh[u][c], xl[u][c]);
 #pragma unroll
   for (int u = 0; u < N; ++u) {
-    const bool has_a = w[u].x != 0.f;
+    {
+      const ff2 w0 = ff2_pack(w[u].z, w[u].z), wn = ff2_pack(-w[u].z, -w[u].z), w1 = ff2_pack(w[u].w, w[u].w);
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
+      for (int c = 0; c < CH; ++c) ff2_mac(mh[c], ml[c], w0, wn, w1, xh[u][c], xl[u][c]);
+    }
+    if (w[u].x != 0.f) {
+      const ff2 w0 = ff2_pack(w[u].x, w[u].x), wn = ff2_pack(-w[u].x, -w[u].x), w1 = ff2_pack(w[u].y, w[u].y);
 #pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        ff_mac(mh[c][v], ml[c][v], w[u].z, w[u].w, xh[u][c][v], xl[u][c][v]);
-        if (has_a) {
-          if (AEX) ff_mac_exact(ah[c][v], al[c][v], w[u].x, xh[u][c][v], xl[u][c][v]);
-          else ff_mac(ah[c][v], al[c][v], w[u].x, w[u].y, xh[u][c][v], xl[u][c][v]);
-        }
+      for (int c = 0; c < CH; ++c) {
+        if (AEX) ff2_mac_exact(ah[c], al[c], w0, wn, xh[u][c], xl[u][c]);
+        else ff2_mac(ah[c], al[c], w0, wn, w1, xh[u][c], xl[u][c]);
       }
+    }
   }
 }
 
 template <int CH, bool FFIN, bool AEX>
 __device__ __forceinline__ void gather_row_am(const int* __restrict__ rp, const int* __restrict__ ci,
                                               const float4* __restrict__ am, const double* __restrict__ X, int row,
-                                              int lane, int tpr, int ldk, float (&ah)[CH][2], float (&al)[CH][2],
-                                              float (&mh)[CH][2], float (&ml)[CH][2]) {
+                                              int lane, int tpr, int ldk, ff2 (&ah)[CH], ff2 (&al)[CH],
+                                              ff2 (&mh)[CH], ff2 (&ml)[CH]) {
 #pragma unroll
-  for (int c = 0; c < CH; ++c)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) ah[c][v] = al[c][v] = mh[c][v] = ml[c][v] = 0.f;
+  for (int c = 0; c < CH; ++c) ah[c] = al[c] = mh[c] = ml[c] = 0;
   int p = __ldg(rp + row);
   const int p1 = __ldg(rp + row + 1);
   for (; p + 4 <= p1; p += 4) gather_group_am<CH, 4, FFIN, AEX>(ci, am, X, p, lane, tpr, ldk, ah, al, mh, ml);
@@ -176,20 +176,23 @@ __device__ __forceinline__ void gather_row_am(const int* __restrict__ rp, const 
   else if (rem == 2) gather_group_am<CH, 2, FFIN, AEX>(ci, am, X, p, lane, tpr, ldk, ah, al, mh, ml);
   else if (rem == 1) gather_group_am<CH, 1, FFIN, AEX>(ci, am, X, p, lane, tpr, ldk, ah, al, mh, ml);
 #pragma unroll
-  for (int c = 0; c < CH; ++c)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      ff_norm(ah[c][v], al[c][v]);
-      ff_norm(mh[c][v], ml[c][v]);
-    }
+  for (int c = 0; c < CH; ++c) {
+    ff2_norm(ah[c], al[c]);
+    ff2_norm(mh[c], ml[c]);
+  }
 }
 
-// Store two entries as float pairs or, rounded, as float64.
+// Store two entries as a pair chunk or, rounded, as float64.
 template <bool FF>
-__device__ __forceinline__ void store_pair(double* __restrict__ out, size_t off, const float (&h)[2],
-                                           const float (&l)[2]) {
-  if (FF) *reinterpret_cast<float4*>(out + off) = make_float4(h[0], l[0], h[1], l[1]);
-  else *reinterpret_cast<double2*>(out + off) = make_double2(ff_to_double(h[0], l[0]), ff_to_double(h[1], l[1]));
+__device__ __forceinline__ void store_pair(double* __restrict__ out, size_t off, ff2 h, ff2 l) {
+  if (FF) {
+    *reinterpret_cast<ulonglong2*>(out + off) = make_ulonglong2(h, l);
+  } else {
+    float h0, h1, l0, l1;
+    ff2_unpack(h, h0, h1);
+    ff2_unpack(l, l0, l1);
+    *reinterpret_cast<double2*>(out + off) = make_double2(ff_to_double(h0, l0), ff_to_double(h1, l1));
+  }
 }
 
 // Fd = lam .* (M U) stored as (hi, lo) float pairs, R = Fd - A U as float32
@@ -200,16 +203,16 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
                        const int* __restrict__ mrp, const int* __restrict__ mci, const float2* __restrict__ mval,
                        const double* __restrict__ lam, const double* __restrict__ U, float2* __restrict__ Fd,
                        float* __restrict__ R, int ldk, int tpr, int rpt) {
-  // the eigenvalues as (hi, lo) pairs, split once per block rather than once per entry
-  extern __shared__ float2 lsp[];  // [ldk]
-  for (int t = threadIdx.x; t < ldk; t += blockDim.x) ff_split(__ldg(lam + t), lsp[t].x, lsp[t].y);
+  // the eigenvalues as pair chunks, split once per block rather than once per entry
+  extern __shared__ ulonglong2 lsp[];  // [ldk / 2]
+  for (int t = threadIdx.x; t < ldk / 2; t += blockDim.x) load_pair<false>(lam, 2 * t, lsp[t].x, lsp[t].y);
   __syncthreads();
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
-  float muh[CH][2], mul[CH][2], auh[CH][2], aul[CH][2];
+  ff2 muh[CH], mul[CH], auh[CH], aul[CH];
   // two separate gathers: the one-gather form (as in the bordering kernel) needs more registers
   // than the four blocks per SM this kernel runs at, and was slower (0.57 -> 0.63 ms)
   gather_row_ff<CH, true>(mrp, mci, mval, U, row, lane, tpr, ldk, muh, mul);
@@ -218,15 +221,12 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    float f[2][2], r[2];
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const float2 l = lsp[col + v];
-      ff_mul(l.x, l.y, muh[c][v], mul[c][v], f[v][0], f[v][1]);
-      r[v] = __fadd_rn(__fsub_rn(f[v][0], auh[c][v]), __fsub_rn(f[v][1], aul[c][v]));
-    }
-    *reinterpret_cast<float4*>(Fd + base + col) = make_float4(f[0][0], f[0][1], f[1][0], f[1][1]);
-    *reinterpret_cast<float2*>(R + base + col) = make_float2(r[0], r[1]);
+    const ulonglong2 l = lsp[col / 2];
+    ff2 fh, fl;
+    ff2_mul(l.x, l.y, muh[c], mul[c], fh, fl);
+    const ff2 r = ff2_addrn(ff2_subrn(fh, auh[c]), ff2_subrn(fl, aul[c]));
+    *reinterpret_cast<ulonglong2*>(Fd + base + col) = make_ulonglong2(fh, fl);
+    *reinterpret_cast<ff2*>(R + base + col) = r;
   }
   }
 }
@@ -242,16 +242,14 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
-  float axh[CH][2], axl[CH][2];
+  ff2 axh[CH], axl[CH];
   gather_row_ff<CH, true, AEX>(arp, aci, aval, X, row, lane, tpr, ldk, axh, axl);
   const size_t base = (size_t)row * ldk;
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    const float4 f = __ldg(reinterpret_cast<const float4*>(Fd + base + col));
-    const float r0 = __fadd_rn(__fsub_rn(f.x, axh[c][0]), __fsub_rn(f.y, axl[c][0]));
-    const float r1 = __fadd_rn(__fsub_rn(f.z, axh[c][1]), __fsub_rn(f.w, axl[c][1]));
-    *reinterpret_cast<float2*>(R + base + col) = make_float2(r0, r1);
+    const ulonglong2 f = __ldg(reinterpret_cast<const ulonglong2*>(Fd + base + col));
+    *reinterpret_cast<ff2*>(R + base + col) = ff2_addrn(ff2_subrn(f.x, axh[c]), ff2_subrn(f.y, axl[c]));
   }
   }
 }
@@ -264,17 +262,15 @@ __global__ void __launch_bounds__(kBlock)
                 const int* __restrict__ mrp, const int* __restrict__ mci, const float2* __restrict__ mval,
                 const double* __restrict__ X, double* __restrict__ YA, double* __restrict__ YM,
                 double* __restrict__ partials, int ldk, int tpr, const float4* __restrict__ am) {
-  extern __shared__ double red[];  // [rpb][2][ldk]
+  extern __shared__ __align__(16) double red[];  // [rpb][2][ldk]
   const int rpb = kBlock / tpr;
   const int grp = threadIdx.x / tpr;
   const int lane = threadIdx.x % tpr;
-  float sAh[CH][2], sAl[CH][2], sMh[CH][2], sMl[CH][2];
+  ff2 sAh[CH], sAl[CH], sMh[CH], sMl[CH];
 #pragma unroll
-  for (int c = 0; c < CH; ++c)
-#pragma unroll
-    for (int v = 0; v < 2; ++v) sAh[c][v] = sAl[c][v] = sMh[c][v] = sMl[c][v] = 0.f;
+  for (int c = 0; c < CH; ++c) sAh[c] = sAl[c] = sMh[c] = sMl[c] = 0;
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
-    float yah[CH][2], yal[CH][2], ymh[CH][2], yml[CH][2];
+    ff2 yah[CH], yal[CH], ymh[CH], yml[CH];
     if (MERGED) {
       gather_row_am<CH, true, AEX>(mrp, mci, am, X, row, lane, tpr, ldk, yah, yal, ymh, yml);
     } else {
@@ -285,25 +281,20 @@ __global__ void __launch_bounds__(kBlock)
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       const size_t off = base + (c * tpr + lane) * 2;
-      float xh[2], xl[2];
+      ff2 xh, xl;
       load_pair<true>(X, off, xh, xl);
       store_pair<true>(YA, off, yah[c], yal[c]);
       store_pair<true>(YM, off, ymh[c], yml[c]);
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        ff_mac(sAh[c][v], sAl[c][v], xh[v], xl[v], yah[c][v], yal[c][v]);
-        ff_mac(sMh[c][v], sMl[c][v], xh[v], xl[v], ymh[c][v], yml[c][v]);
-      }
+      const ff2 nx = ff2_neg(xh);
+      ff2_mac(sAh[c], sAl[c], xh, nx, xl, yah[c], yal[c]);
+      ff2_mac(sMh[c], sMl[c], xh, nx, xl, ymh[c], yml[c]);
     }
   }
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      red[(grp * 2 + 0) * ldk + col + v] = ff_to_double(sAh[c][v], sAl[c][v]);
-      red[(grp * 2 + 1) * ldk + col + v] = ff_to_double(sMh[c][v], sMl[c][v]);
-    }
+    store_pair<false>(red, (grp * 2 + 0) * ldk + col, sAh[c], sAl[c]);
+    store_pair<false>(red, (grp * 2 + 1) * ldk + col, sMh[c], sMl[c]);
   }
   __syncthreads();
   for (int t = threadIdx.x; t < 2 * ldk; t += blockDim.x) {
@@ -323,7 +314,7 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm_ff(int n, con
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
-  float yh[CH][2], yl[CH][2];
+  ff2 yh[CH], yl[CH];
   gather_row_ff<CH, FFIN, EX>(rp, ci, av, X, row, lane, tpr, ldk, yh, yl);
   const size_t base = (size_t)row * ldk;
 #pragma unroll
@@ -337,8 +328,8 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm_ff(int n, con
 template <int CH, int N, bool FFIN, bool EX>
 __device__ __forceinline__ void gather_group_ff2(const int* __restrict__ ci, const float2* __restrict__ av,
                                                  const double* __restrict__ XA, const double* __restrict__ XM,
-                                                 int p, int lane, int tpr, int ldk, float (&ah)[CH][2],
-                                                 float (&al)[CH][2], float (&mh)[CH][2], float (&ml)[CH][2]) {
+                                                 int p, int lane, int tpr, int ldk, ff2 (&ah)[CH], ff2 (&al)[CH],
+                                                 ff2 (&mh)[CH], ff2 (&ml)[CH]) {
   int j[N];
   float2 a[N];
 #pragma unroll
@@ -346,7 +337,7 @@ __device__ __forceinline__ void gather_group_ff2(const int* __restrict__ ci, con
     j[u] = __ldg(ci + p + u);
     a[u] = __ldg(av + p + u);
   }
-  float xh[N][CH][2], xl[N][CH][2], yh[N][CH][2], yl[N][CH][2];
+  ff2 xh[N][CH], xl[N][CH], yh[N][CH], yl[N][CH];
 #pragma unroll
   for (int u = 0; u < N; ++u)
 #pragma unroll
@@ -356,19 +347,19 @@ __device__ __forceinline__ void gather_group_ff2(const int* __restrict__ ci, con
       load_pair<FFIN>(XM, off, yh[u][c], yl[u][c]);
     }
 #pragma unroll
-  for (int u = 0; u < N; ++u)
+  for (int u = 0; u < N; ++u) {
+    const ff2 w0 = ff2_pack(a[u].x, a[u].x), wn = ff2_pack(-a[u].x, -a[u].x), w1 = ff2_pack(a[u].y, a[u].y);
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        if (EX) {
-          ff_mac_exact(ah[c][v], al[c][v], a[u].x, xh[u][c][v], xl[u][c][v]);
-          ff_mac_exact(mh[c][v], ml[c][v], a[u].x, yh[u][c][v], yl[u][c][v]);
-        } else {
-          ff_mac(ah[c][v], al[c][v], a[u].x, a[u].y, xh[u][c][v], xl[u][c][v]);
-          ff_mac(mh[c][v], ml[c][v], a[u].x, a[u].y, yh[u][c][v], yl[u][c][v]);
-        }
+    for (int c = 0; c < CH; ++c) {
+      if (EX) {
+        ff2_mac_exact(ah[c], al[c], w0, wn, xh[u][c], xl[u][c]);
+        ff2_mac_exact(mh[c], ml[c], w0, wn, yh[u][c], yl[u][c]);
+      } else {
+        ff2_mac(ah[c], al[c], w0, wn, w1, xh[u][c], xl[u][c]);
+        ff2_mac(mh[c], ml[c], w0, wn, w1, yh[u][c], yl[u][c]);
       }
+    }
+  }
 }
 
 template <int CH, bool FFIN, bool FFOUT, bool EX>
@@ -385,11 +376,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm2_ff(int n, co
   for (int rr = 0; rr < rpt; ++rr) {
     const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
     if (row >= n) return;
-    float ah[CH][2], al[CH][2], mh[CH][2], ml[CH][2];
+    ff2 ah[CH], al[CH], mh[CH], ml[CH];
 #pragma unroll
-    for (int c = 0; c < CH; ++c)
-#pragma unroll
-      for (int v = 0; v < 2; ++v) ah[c][v] = al[c][v] = mh[c][v] = ml[c][v] = 0.f;
+    for (int c = 0; c < CH; ++c) ah[c] = al[c] = mh[c] = ml[c] = 0;
     int p = __ldg(rp + row);
     const int p1 = __ldg(rp + row + 1);
     for (; p + 4 <= p1; p += 4) gather_group_ff2<CH, 4, FFIN, EX>(ci, av, XA, XM, p, lane, tpr, ldk, ah, al, mh, ml);
@@ -400,11 +389,8 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm2_ff(int n, co
     const size_t base = (size_t)row * ldk;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        ff_norm(ah[c][v], al[c][v]);
-        ff_norm(mh[c][v], ml[c][v]);
-      }
+      ff2_norm(ah[c], al[c]);
+      ff2_norm(mh[c], ml[c]);
       store_pair<FFOUT>(outA, base + (c * tpr + lane) * 2, ah[c], al[c]);
       store_pair<FFOUT>(outM, base + (c * tpr + lane) * 2, mh[c], ml[c]);
     }
@@ -417,18 +403,10 @@ template <bool BFF>
 __global__ void k_axpy_ff(int64_t total, const double* B, const float* __restrict__ E, double* X) {
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
-    float bh[2], bl[2];
+    ff2 bh, bl;
     load_pair<BFF>(B, 2 * i, bh, bl);
-    const float2 e = __ldg(reinterpret_cast<const float2*>(E + 2 * i));
-    const float ev[2] = {e.x, e.y};
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      float h = bh[v], l = bl[v];
-      ff_mac(h, l, ev[v], 0.f, 1.f, 0.f);
-      ff_norm(h, l);
-      bh[v] = h;
-      bl[v] = l;
-    }
+    ff2_add(bh, bl, __ldg(reinterpret_cast<const ff2*>(E + 2 * i)));
+    ff2_norm(bh, bl);
     store_pair<true>(X, 2 * i, bh, bl);
   }
 }
@@ -438,7 +416,7 @@ __global__ void k_axpy_ff(int64_t total, const double* B, const float* __restric
 __global__ void k_to_ff(int64_t total, const double* in, double* out) {
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
-    float h[2], l[2];
+    ff2 h, l;
     load_pair<false>(in, 2 * i, h, l);
     store_pair<true>(out, 2 * i, h, l);
   }
@@ -446,7 +424,7 @@ __global__ void k_to_ff(int64_t total, const double* in, double* out) {
 __global__ void k_from_ff(int64_t total, const double* __restrict__ in, double* __restrict__ out) {
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
-    float h[2], l[2];
+    ff2 h, l;
     load_pair<true>(in, 2 * i, h, l);
     store_pair<false>(out, 2 * i, h, l);
   }
@@ -464,15 +442,15 @@ __global__ void __launch_bounds__(kBlock)
                 const double* __restrict__ W, const double* __restrict__ X, const double* __restrict__ alpha,
                 const int* __restrict__ upd, double* __restrict__ U, double* __restrict__ Usplit, int ldk, int tpr,
                 int identity, int rpt) {
-  extern __shared__ float2 asp[];  // [ldk]: alpha as (hi, lo) pairs, split once per block
-  for (int t = threadIdx.x; t < ldk; t += blockDim.x) ff_split(__ldg(alpha + t), asp[t].x, asp[t].y);
+  extern __shared__ ulonglong2 asp[];  // [ldk / 2]: alpha as pair chunks, split once per block
+  for (int t = threadIdx.x; t < ldk / 2; t += blockDim.x) load_pair<false>(alpha, 2 * t, asp[t].x, asp[t].y);
   __syncthreads();
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
-  float wh[CH][2], wl[CH][2];
+  ff2 wh[CH], wl[CH];
   const size_t base = (size_t)row * ldk;
   if (identity) {
 #pragma unroll
@@ -486,37 +464,35 @@ __global__ void __launch_bounds__(kBlock)
     const size_t off = base + col;
     const int u0 = upd[col], u1 = upd[col + 1];
     if (!u0 && !u1) continue;  // both pairs frozen: U and its split copy stay as they are
-    float xh[2], xl[2];
+    ff2 xh, xl;
     load_pair<true>(X, off, xh, xl);
-    float h[2], l[2];
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const float2 a = asp[col + v];
-      h[v] = wh[c][v];
-      l[v] = wl[c][v];
-      ff_mac(h[v], l[v], a.x, a.y, xh[v], xl[v]);
-      ff_norm(h[v], l[v]);
-    }
+    const ulonglong2 a = asp[col / 2];
+    ff2 h = wh[c], l = wl[c];
+    ff2_mac(h, l, a.x, ff2_neg(a.x), a.y, xh, xl);
+    ff2_norm(h, l);
     if (!U) {  // the state lives in pairs only: write the updated pairs, keep the frozen one
       if (!(u0 && u1)) {
-        float oh[2], ol[2];
+        ff2 oh, ol;
         load_pair<true>(Usplit, off, oh, ol);
-        if (!u0) { h[0] = oh[0]; l[0] = ol[0]; }
-        if (!u1) { h[1] = oh[1]; l[1] = ol[1]; }
+        const ff2 keep = u0 ? 0xFFFFFFFF00000000ull : 0x00000000FFFFFFFFull;
+        h = (h & ~keep) | (oh & keep);
+        l = (l & ~keep) | (ol & keep);
       }
       store_pair<true>(Usplit, off, h, l);
       continue;
     }
     double2 u;
     if (!(u0 && u1)) u = *reinterpret_cast<const double2*>(U + off);
-    if (u0) u.x = ff_to_double(h[0], l[0]);
-    if (u1) u.y = ff_to_double(h[1], l[1]);
+    float h0, h1, l0, l1;
+    ff2_unpack(h, h0, h1);
+    ff2_unpack(l, l0, l1);
+    if (u0) u.x = ff_to_double(h0, l0);
+    if (u1) u.y = ff_to_double(h1, l1);
     *reinterpret_cast<double2*>(U + off) = u;
     if (Usplit) {  // the (hi, lo) copy of U the next step's gathers read
-      float uh[2], ul[2];
-      ff_split(u.x, uh[0], ul[0]);
-      ff_split(u.y, uh[1], ul[1]);
-      store_pair<true>(Usplit, off, uh, ul);
+      ff_split(u.x, h0, l0);
+      ff_split(u.y, h1, l1);
+      store_pair<true>(Usplit, off, ff2_pack(h0, h1), ff2_pack(l0, l1));
     }
   }
   }

@@ -41,46 +41,84 @@ __device__ __forceinline__ double ff_f2d(float f) {
 // hi + lo rounded to float64 (one float64 addition).
 __device__ __forceinline__ double ff_to_double(float hi, float lo) { return __dadd_rn(ff_f2d(hi), ff_f2d(lo)); }
 
-// (hi, lo) += (ah + al) * (xh + xl): exact product error by FMA, two-sum of
-// the leading parts; the low-order cross terms and errors collect in lo.
-__device__ __forceinline__ void ff_mac(float& hi, float& lo, float ah, float al, float xh, float xl) {
-  const float p = __fmul_rn(ah, xh);
-  float e = __fmaf_rn(ah, xh, -p);
-  e = __fmaf_rn(ah, xl, e);
-  e = __fmaf_rn(al, xh, e);
-  const float s = __fadd_rn(hi, p);
-  const float bb = __fsub_rn(s, hi);
-  const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(t, e));
-}
+// ----------------------------------------------------------------------------------------------
+// The arithmetic, on two values at once: the packed float32 instructions of sm_100 and later (f32x2)
+// take one issue slot for two lanes' worth of work.  The float32 pipe's rate is the same and so are the
+// results; the kernels of ff.cu were bound by issue (65 % of the slots at h = 1/320, k = 37).  A block vector "in pairs" stores two columns as one
+// 16-byte chunk (hi0, hi1, lo0, lo1), so that a 16-byte load gives both packed operands.
+typedef unsigned long long ff2;  // two float32
 
-// ff_mac for a float32 coefficient a (no low part): one FMA fewer.
-__device__ __forceinline__ void ff_mac_exact(float& hi, float& lo, float a, float xh, float xl) {
-  const float p = __fmul_rn(a, xh);
-  float e = __fmaf_rn(a, xh, -p);
-  e = __fmaf_rn(a, xl, e);
-  const float s = __fadd_rn(hi, p);
-  const float bb = __fsub_rn(s, hi);
-  const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-  hi = s;
-  lo = __fadd_rn(lo, __fadd_rn(t, e));
+__device__ __forceinline__ ff2 ff2_pack(float a, float b) {
+  ff2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
 }
+__device__ __forceinline__ void ff2_unpack(ff2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ ff2 ff2_addrn(ff2 a, ff2 b) {
+  ff2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ff2 ff2_subrn(ff2 a, ff2 b) {
+  ff2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ff2 ff2_mulrn(ff2 a, ff2 b) {
+  ff2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ ff2 ff2_fmarn(ff2 a, ff2 b, ff2 c) {
+  ff2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ ff2 ff2_neg(ff2 a) { return a ^ 0x8000000080000000ull; }
 
-// Renormalise so that |lo| <= ulp(hi) / 2.
-__device__ __forceinline__ void ff_norm(float& hi, float& lo) {
-  const float s = __fadd_rn(hi, lo);
-  lo = __fsub_rn(lo, __fsub_rn(s, hi));
+// (hi, lo) += -n + e for the product -n with exact error e (two-sum of hi and -n)
+__device__ __forceinline__ void ff2_accumulate(ff2& hi, ff2& lo, ff2 n, ff2 e) {
+  const ff2 s = ff2_subrn(hi, n);
+  const ff2 bb = ff2_subrn(s, hi);
+  const ff2 t = ff2_subrn(ff2_subrn(hi, ff2_subrn(s, bb)), ff2_addrn(n, bb));
+  hi = s;
+  lo = ff2_addrn(lo, ff2_addrn(t, e));
+}
+// (hi, lo) += (ah + al) * (xh + xl); na = -ah
+__device__ __forceinline__ void ff2_mac(ff2& hi, ff2& lo, ff2 ah, ff2 na, ff2 al, ff2 xh, ff2 xl) {
+  const ff2 n = ff2_mulrn(na, xh);
+  ff2 e = ff2_fmarn(ah, xh, n);
+  e = ff2_fmarn(ah, xl, e);
+  e = ff2_fmarn(al, xh, e);
+  ff2_accumulate(hi, lo, n, e);
+}
+// ff2_mac for a float32 coefficient a (no low part)
+__device__ __forceinline__ void ff2_mac_exact(ff2& hi, ff2& lo, ff2 a, ff2 na, ff2 xh, ff2 xl) {
+  const ff2 n = ff2_mulrn(na, xh);
+  ff2 e = ff2_fmarn(a, xh, n);
+  e = ff2_fmarn(a, xl, e);
+  ff2_accumulate(hi, lo, n, e);
+}
+// (hi, lo) += v
+__device__ __forceinline__ void ff2_add(ff2& hi, ff2& lo, ff2 v) {
+  const ff2 s = ff2_addrn(hi, v);
+  const ff2 bb = ff2_subrn(s, hi);
+  const ff2 t = ff2_addrn(ff2_subrn(hi, ff2_subrn(s, bb)), ff2_subrn(v, bb));
+  hi = s;
+  lo = ff2_addrn(lo, t);
+}
+__device__ __forceinline__ void ff2_norm(ff2& hi, ff2& lo) {
+  const ff2 s = ff2_addrn(hi, lo);
+  lo = ff2_subrn(lo, ff2_subrn(s, hi));
   hi = s;
 }
-
-// (hi, lo) = (ah + al) * (bh + bl), renormalised.
-__device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& hi, float& lo) {
-  const float p = __fmul_rn(ah, bh);
-  float e = __fmaf_rn(ah, bh, -p);
-  e = __fmaf_rn(ah, bl, e);
-  e = __fmaf_rn(al, bh, e);
-  hi = p;
-  lo = e;
-  ff_norm(hi, lo);
+// (hi, lo) = (ah + al) * (bh + bl), renormalised
+__device__ __forceinline__ void ff2_mul(ff2 ah, ff2 al, ff2 bh, ff2 bl, ff2& hi, ff2& lo) {
+  hi = ff2_mulrn(ah, bh);
+  ff2 e = ff2_fmarn(ah, bh, ff2_neg(hi));
+  e = ff2_fmarn(ah, bl, e);
+  lo = ff2_fmarn(al, bh, e);
+  ff2_norm(hi, lo);
 }

@@ -736,8 +736,8 @@ __global__ void __launch_bounds__(kBlock) k_residual_partials(int n, int ldk, co
       if (FF) {
         const float4 f = *reinterpret_cast<const float4*>(Fd + off);
         const float4 u = *reinterpret_cast<const float4*>(U + off);
-        m0 = (double)f.x + (double)f.y; m1 = (double)f.z + (double)f.w;
-        u0 = (double)u.x + (double)u.y; u1 = (double)u.z + (double)u.w;
+        m0 = (double)f.x + (double)f.z; m1 = (double)f.y + (double)f.w;   // chunk = hi, hi, lo, lo
+        u0 = (double)u.x + (double)u.z; u1 = (double)u.y + (double)u.w;
       } else {
         m0 = Fd[off]; m1 = Fd[off + 1];
         u0 = U[off]; u1 = U[off + 1];
@@ -972,24 +972,30 @@ __global__ void __launch_bounds__(kBlock)
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const size_t off = base + (c * tpr + lane) * V;
-    float h[V], l[V];
-    if (BFF) {
-      const float4 b0 = *reinterpret_cast<const float4*>(B + off);
-      const float4 b1 = *reinterpret_cast<const float4*>(B + off + 2);
-      h[0] = b0.x; l[0] = b0.y; h[1] = b0.z; l[1] = b0.w; h[2] = b1.x; l[2] = b1.y; h[3] = b1.z; l[3] = b1.w;
-    } else {
-      const double2 b0 = *reinterpret_cast<const double2*>(B + off);
-      const double2 b1 = *reinterpret_cast<const double2*>(B + off + 2);
-      ff_split(b0.x, h[0], l[0]); ff_split(b0.y, h[1], l[1]); ff_split(b1.x, h[2], l[2]); ff_split(b1.y, h[3], l[3]);
-    }
+    ff2 h[2], l[2];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float e = fmaf(w, y[c][v] - acc[c][v], z[c][v]);
-      ff_mac(h[v], l[v], e, 0.f, 1.f, 0.f);
-      ff_norm(h[v], l[v]);
+    for (int q = 0; q < 2; ++q) {
+      if (BFF) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(B + off + 2 * q);
+        h[q] = t.x; l[q] = t.y;
+      } else {
+        const double2 t = *reinterpret_cast<const double2*>(B + off + 2 * q);
+        float h0, l0, h1, l1;
+        ff_split(t.x, h0, l0);
+        ff_split(t.y, h1, l1);
+        h[q] = ff2_pack(h0, h1);
+        l[q] = ff2_pack(l0, l1);
+      }
     }
-    *reinterpret_cast<float4*>(X + off) = make_float4(h[0], l[0], h[1], l[1]);
-    *reinterpret_cast<float4*>(X + off + 2) = make_float4(h[2], l[2], h[3], l[3]);
+    float e[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) e[v] = fmaf(w, y[c][v] - acc[c][v], z[c][v]);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      ff2_add(h[q], l[q], ff2_pack(e[2 * q], e[2 * q + 1]));
+      ff2_norm(h[q], l[q]);
+      *reinterpret_cast<ulonglong2*>(X + off + 2 * q) = make_ulonglong2(h[q], l[q]);
+    }
   }
   }
 }
