@@ -63,16 +63,27 @@ static int ff_rows(const Launch& L) { return L.rpt > 0 ? L.rpt : 1; }
 template <bool FF>
 __device__ __forceinline__ void load_pair(const double* __restrict__ X, size_t off, ff2& h, ff2& l) {
   if (FF) {
-    const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2*>(X + off));
-    h = t.x; l = t.y;
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(h), "=l"(l) : "l"(X + off));
   } else {
-    const double2 t = __ldg(reinterpret_cast<const double2*>(X + off));
+    double t[2];
+    ldg16<double>(X + off, t);
     float h0, l0, h1, l1;
-    ff_split(t.x, h0, l0);
-    ff_split(t.y, h1, l1);
+    ff_split(t[0], h0, l0);
+    ff_split(t[1], h1, l1);
     h = ff2_pack(h0, h1);
     l = ff2_pack(l0, l1);
   }
+}
+
+// The first row of a row group, before pdl_wait: its entries on their way to the SM.
+template <typename VT>
+__device__ __forceinline__ void prefetch_row(const int* __restrict__ rp, const int* __restrict__ ci,
+                                             const VT* __restrict__ av, int row, int n) {
+  if (row >= n) return;
+  const int p = __ldg(rp + row);
+  if (p >= __ldg(rp + row + 1)) return;
+  prefetch_line(ci + p);
+  prefetch_line(av + p);
 }
 
 // acc += a_p X[ci_p, cols] for the N entries p .. p+N-1: index and value loads,
@@ -203,6 +214,10 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
                        const int* __restrict__ mrp, const int* __restrict__ mci, const float2* __restrict__ mval,
                        const double* __restrict__ lam, const double* __restrict__ U, float2* __restrict__ Fd,
                        float* __restrict__ R, int ldk, int tpr, int rpt) {
+  pdl_trigger();
+  prefetch_row(mrp, mci, mval, blockIdx.x * rpt * (kBlock / tpr) + threadIdx.x / tpr, n);
+  prefetch_row(arp, aci, aval, blockIdx.x * rpt * (kBlock / tpr) + threadIdx.x / tpr, n);
+  pdl_wait();
   // the eigenvalues as pair chunks, split once per block rather than once per entry
   extern __shared__ ulonglong2 lsp[];  // [ldk / 2]
   for (int t = threadIdx.x; t < ldk / 2; t += blockDim.x) load_pair<false>(lam, 2 * t, lsp[t].x, lsp[t].y);
@@ -239,6 +254,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
                    int tpr, int rpt) {
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(arp, aci, aval, blockIdx.x * rpt * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
@@ -248,8 +266,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    const ulonglong2 f = __ldg(reinterpret_cast<const ulonglong2*>(Fd + base + col));
-    *reinterpret_cast<ff2*>(R + base + col) = ff2_addrn(ff2_subrn(f.x, axh[c]), ff2_subrn(f.y, axl[c]));
+    ff2 fh, fl;
+    load_pair<true>(reinterpret_cast<const double*>(Fd), base + col, fh, fl);
+    *reinterpret_cast<ff2*>(R + base + col) = ff2_addrn(ff2_subrn(fh, axh[c]), ff2_subrn(fl, axl[c]));
   }
   }
 }
@@ -269,6 +288,14 @@ __global__ void __launch_bounds__(kBlock)
   ff2 sAh[CH], sAl[CH], sMh[CH], sMl[CH];
 #pragma unroll
   for (int c = 0; c < CH; ++c) sAh[c] = sAl[c] = sMh[c] = sMl[c] = 0;
+  pdl_trigger();
+  if (MERGED) {
+    prefetch_row(mrp, mci, am, blockIdx.x * rpb + grp, n);
+  } else {
+    prefetch_row(mrp, mci, mval, blockIdx.x * rpb + grp, n);
+    prefetch_row(arp, aci, aval, blockIdx.x * rpb + grp, n);
+  }
+  pdl_wait();
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
     ff2 yah[CH], yal[CH], ymh[CH], yml[CH];
     if (MERGED) {
@@ -311,6 +338,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm_ff(int n, con
                                                      double* __restrict__ out, int ldk, int tpr, int rpt) {
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * rpt * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
@@ -373,6 +403,9 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm2_ff(int n, co
                                                                      int rpt) {
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * rpt * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < rpt; ++rr) {
     const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
     if (row >= n) return;
@@ -400,12 +433,16 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather) k_spmm2_ff(int n, co
 // X = B + E with E float32, X as float pairs; B as float pairs (may alias X)
 // or float64.
 template <bool BFF>
-__global__ void k_axpy_ff(int64_t total, const double* B, const float* __restrict__ E, double* X) {
+__global__ void k_axpy_ff(int64_t total, const double* B, const float* E, double* X) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
     ff2 bh, bl;
     load_pair<BFF>(B, 2 * i, bh, bl);
-    ff2_add(bh, bl, __ldg(reinterpret_cast<const ff2*>(E + 2 * i)));
+    ff2 e;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(e) : "l"(E + 2 * i));
+    ff2_add(bh, bl, e);
     ff2_norm(bh, bl);
     store_pair<true>(X, 2 * i, bh, bl);
   }
@@ -414,6 +451,8 @@ __global__ void k_axpy_ff(int64_t total, const double* B, const float* __restric
 // Elementwise format conversions of block vectors.
 // in may equal out: each thread reads its two entries before writing them.
 __global__ void k_to_ff(int64_t total, const double* in, double* out) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
     ff2 h, l;
@@ -421,7 +460,9 @@ __global__ void k_to_ff(int64_t total, const double* in, double* out) {
     store_pair<true>(out, 2 * i, h, l);
   }
 }
-__global__ void k_from_ff(int64_t total, const double* __restrict__ in, double* __restrict__ out) {
+__global__ void k_from_ff(int64_t total, const double* in, double* out) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
     ff2 h, l;
@@ -436,12 +477,18 @@ __global__ void k_from_ff(int64_t total, const double* __restrict__ in, double* 
 // pair array Usplit alone (the finest-level state of the mixed-precision step;
 // its float64 copy is made on demand), else U is written in float64 and, if
 // Usplit is given, also split into pairs.
-template <int CH, bool WFF, bool EX>
-__global__ void __launch_bounds__(kBlock)
+// STATE: the finest-level update of a step (U null, P given), on its own so that it fits 32 registers
+// for one chunk per thread (8 blocks per SM; at 40 it took 298 us instead of UPD1 at h = 1/1024, k = 64).
+template <int CH, bool STATE> struct UpdateMinBlocks { static constexpr int v = STATE && CH == 1 ? 8 : 0; };
+template <int CH, bool WFF, bool EX, bool STATE>
+__global__ void __launch_bounds__(kBlock, (UpdateMinBlocks<CH, STATE>::v))
     k_update_ff(int n, const int* __restrict__ rp, const int* __restrict__ ci, const float2* __restrict__ pv,
                 const double* __restrict__ W, const double* __restrict__ X, const double* __restrict__ alpha,
                 const int* __restrict__ upd, double* __restrict__ U, double* __restrict__ Usplit, int ldk, int tpr,
                 int identity, int rpt) {
+  pdl_trigger();
+  if (STATE || !identity) prefetch_row(rp, ci, pv, blockIdx.x * rpt * (kBlock / tpr) + threadIdx.x / tpr, n);
+  pdl_wait();
   extern __shared__ ulonglong2 asp[];  // [ldk / 2]: alpha as pair chunks, split once per block
   for (int t = threadIdx.x; t < ldk / 2; t += blockDim.x) load_pair<false>(alpha, 2 * t, asp[t].x, asp[t].y);
   __syncthreads();
@@ -452,7 +499,7 @@ __global__ void __launch_bounds__(kBlock)
   if (row >= n) return;
   ff2 wh[CH], wl[CH];
   const size_t base = (size_t)row * ldk;
-  if (identity) {
+  if (!STATE && identity) {
 #pragma unroll
     for (int c = 0; c < CH; ++c) load_pair<WFF>(W, base + (c * tpr + lane) * 2, wh[c], wl[c]);
   } else {
@@ -462,7 +509,7 @@ __global__ void __launch_bounds__(kBlock)
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
     const size_t off = base + col;
-    const int u0 = upd[col], u1 = upd[col + 1];
+    const int u0 = ld1(upd + col), u1 = ld1(upd + col + 1);
     if (!u0 && !u1) continue;  // both pairs frozen: U and its split copy stay as they are
     ff2 xh, xl;
     load_pair<true>(X, off, xh, xl);
@@ -470,7 +517,7 @@ __global__ void __launch_bounds__(kBlock)
     ff2 h = wh[c], l = wl[c];
     ff2_mac(h, l, a.x, ff2_neg(a.x), a.y, xh, xl);
     ff2_norm(h, l);
-    if (!U) {  // the state lives in pairs only: write the updated pairs, keep the frozen one
+    if (STATE || !U) {  // the state lives in pairs only: write the updated pairs, keep the frozen one
       if (!(u0 && u1)) {
         ff2 oh, ol;
         load_pair<true>(Usplit, off, oh, ol);
@@ -511,7 +558,7 @@ void outer_rhs_residual_ff(const Launch& L, const DCsr& A, const DCsr& M, const 
     L.begin(KC_OUTER_RHS, nnz * 12.0 + 2 * (n + 1) * 4.0 + n * ldk * (16.0 + 4.0), 2.0 * nnz * ldk + 2.0 * n * ldk);
   }
 #define PASM_FF_RHS(AEX)                                                                      \
-  PASM_FF_DISPATCH(g.ch, k_outer_rhs_res_ff<CH, AEX><<<grid, kBlock, ldk * sizeof(float2), L.s>>>( \
+  PASM_FF_DISPATCH(g.ch, launch(L, k_outer_rhs_res_ff<CH, AEX>, grid, kBlock, ldk * sizeof(float2), \
                              A.n_rows, A.rp, A.ci, A.vff, M.rp, M.ci, M.vff, lam, U,            \
                              reinterpret_cast<float2*>(Fd), R, ldk, g.tpr, rpt))
   if (A.exact32) { PASM_FF_RHS(true); } else { PASM_FF_RHS(false); }
@@ -529,11 +576,9 @@ void outer_residual_ff(const Launch& L, const DCsr& A, const double* Fd, const d
     L.begin(KC_OUTER_RES, nnz * 12.0 + (n + 1) * 4.0 + n * ldk * (16.0 + 4.0), 2.0 * nnz * ldk + n * ldk);
   }
   if (A.exact32) {
-    PASM_FF_DISPATCH(g.ch, k_outer_res_ff<CH, true><<<grid, kBlock, 0, L.s>>>(
-                               A.n_rows, A.rp, A.ci, A.vff, reinterpret_cast<const float2*>(Fd), X, R, ldk, g.tpr, rpt));
+    PASM_FF_DISPATCH(g.ch, launch(L, k_outer_res_ff<CH, true>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.vff, reinterpret_cast<const float2*>(Fd), X, R, ldk, g.tpr, rpt));
   } else {
-    PASM_FF_DISPATCH(g.ch, k_outer_res_ff<CH, false><<<grid, kBlock, 0, L.s>>>(
-                               A.n_rows, A.rp, A.ci, A.vff, reinterpret_cast<const float2*>(Fd), X, R, ldk, g.tpr, rpt));
+    PASM_FF_DISPATCH(g.ch, launch(L, k_outer_res_ff<CH, false>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.vff, reinterpret_cast<const float2*>(Fd), X, R, ldk, g.tpr, rpt));
   }
   L.bump();
 }
@@ -554,7 +599,7 @@ int border_products_ff(const Launch& L, const DCsr& A, const DCsr& M, const doub
     L.begin(KC_BORDER, nnz * 12.0 + 2 * (n + 1) * 4.0 + 3.0 * n * ldk * 8.0, 2.0 * nnz * ldk + 4.0 * n * ldk);
   }
 #define PASM_FF_BORDER(AEX, MG)                                                                \
-  PASM_FF_DISPATCH(g.ch, k_border_ff<CH, AEX, MG><<<grid, kBlock, smem, L.s>>>(                 \
+  PASM_FF_DISPATCH(g.ch, launch(L, k_border_ff<CH, AEX, MG>, grid, kBlock, smem, \
                              A.n_rows, A.rp, A.ci, A.vff, M.rp, M.ci, M.vff, X, YA, YM, partials, ldk, g.tpr, M.am))
   if (M.am) {
     if (A.exact32) { PASM_FF_BORDER(true, true); } else { PASM_FF_BORDER(false, true); }
@@ -578,10 +623,10 @@ void spmm_ff(const Launch& L, const DCsr& S, const double* X, bool x_ff, double*
   }
 #define PASM_FF_SPMM(FI, FO)                                                                                   \
   if (S.exact32) {                                                                                             \
-    PASM_FF_DISPATCH(g.ch, k_spmm_ff<CH, FI, FO, true><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, S.vff, X, \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_spmm_ff<CH, FI, FO, true>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, S.vff, X, \
                                                                                   out, ldk, g.tpr, rpt));           \
   } else {                                                                                                     \
-    PASM_FF_DISPATCH(g.ch, k_spmm_ff<CH, FI, FO, false><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, S.vff, \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_spmm_ff<CH, FI, FO, false>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, S.vff, \
                                                                                    X, out, ldk, g.tpr, rpt));       \
   }
   if (x_ff && out_ff) { PASM_FF_SPMM(true, true); }
@@ -605,10 +650,10 @@ void spmm2_ff(const Launch& L, const DCsr& S, const double* XA, const double* XM
   }
 #define PASM_FF_SPMM2(FI, FO)                                                                                    \
   if (S.exact32) {                                                                                               \
-    PASM_FF_DISPATCH(g.ch, k_spmm2_ff<CH, FI, FO, true><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, S.vff, XA,  \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_spmm2_ff<CH, FI, FO, true>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, S.vff, XA,  \
                                                                                    XM, outA, outM, ldk, g.tpr, rpt)); \
   } else {                                                                                                       \
-    PASM_FF_DISPATCH(g.ch, k_spmm2_ff<CH, FI, FO, false><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, S.vff, XA, \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_spmm2_ff<CH, FI, FO, false>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, S.vff, XA, \
                                                                                     XM, outA, outM, ldk, g.tpr, rpt)); \
   }
   if (x_ff && out_ff) { PASM_FF_SPMM2(true, true); }
@@ -624,20 +669,20 @@ static int stream_grid(int64_t total) { return (int)std::min<int64_t>((total / 2
 void axpy_ff(const Launch& L, int n, const double* B, bool b_ff, const float* E, double* X, int ldk) {
   const int64_t total = (int64_t)n * ldk;
   L.begin(KC_AXPY, (double)total * (16.0 + 4.0), (double)total);
-  if (b_ff) k_axpy_ff<true><<<stream_grid(total), kBlock, 0, L.s>>>(total, B, E, X);
-  else k_axpy_ff<false><<<stream_grid(total), kBlock, 0, L.s>>>(total, B, E, X);
+  if (b_ff) launch(L, k_axpy_ff<true>, stream_grid(total), kBlock, 0, total, B, E, X);
+  else launch(L, k_axpy_ff<false>, stream_grid(total), kBlock, 0, total, B, E, X);
   L.bump();
 }
 
 void to_ff(const Launch& L, int64_t total, const double* in, double* out) {
   L.begin(KC_CAST, (double)total * 16.0, 0.0);
-  k_to_ff<<<stream_grid(total), kBlock, 0, L.s>>>(total, in, out);
+  launch(L, k_to_ff, stream_grid(total), kBlock, 0, total, in, out);
   L.bump();
 }
 
 void from_ff(const Launch& L, int64_t total, const double* in, double* out) {
   L.begin(KC_CAST, (double)total * 16.0, (double)total);
-  k_from_ff<<<stream_grid(total), kBlock, 0, L.s>>>(total, in, out);
+  launch(L, k_from_ff, stream_grid(total), kBlock, 0, total, in, out);
   L.bump();
 }
 
@@ -656,10 +701,14 @@ void update_pairs_ff(const Launch& L, const DCsr* P, int n, const double* W, boo
   const int* ci = P ? P->ci : nullptr;
   const float2* pv = P ? P->vff : nullptr;
   const bool ex = P ? P->exact32 : true;
-#define PASM_FF_UPD(WF, EXV)                                                                                  \
-  PASM_FF_DISPATCH(g.ch, k_update_ff<CH, WF, EXV><<<grid, kBlock, ldk * sizeof(float2), L.s>>>(                \
-                             n, rp, ci, pv, W, X, alpha, upd, U,                                                \
-                                                                           Usplit, ldk, g.tpr, identity, rpt))
+#define PASM_FF_UPD(WF, EXV)                                                                                     \
+  if (P && !U) {                                                                                                 \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_update_ff<CH, WF, EXV, true>, grid, kBlock, ldk * sizeof(float2), \
+                               n, rp, ci, pv, W, X, alpha, upd, nullptr, Usplit, ldk, g.tpr, 0, rpt));            \
+  } else {                                                                                                       \
+    PASM_FF_DISPATCH(g.ch, launch(L, k_update_ff<CH, WF, EXV, false>, grid, kBlock, ldk * sizeof(float2), \
+                               n, rp, ci, pv, W, X, alpha, upd, U, Usplit, ldk, g.tpr, identity, rpt));           \
+  }
   if (w_ff) {
     if (ex) { PASM_FF_UPD(true, true); } else { PASM_FF_UPD(true, false); }
   } else {

@@ -94,6 +94,17 @@ __device__ __forceinline__ void gather_rows(const int* __restrict__ ci, const T*
   else if (rem == 1) gather_group<T, CH, 1>(ci, av, dscale, omega, X, p, lane, tpr, ldk, acc);
 }
 
+// The first row of a row group, before pdl_wait: its entries on their way to the SM.
+template <typename VT>
+__device__ __forceinline__ void prefetch_row(const int* __restrict__ rp, const int* __restrict__ ci,
+                                             const VT* __restrict__ av, int row, int n) {
+  if (row >= n) return;
+  const int p = __ldg(rp + row);
+  if (p >= __ldg(rp + row + 1)) return;
+  prefetch_line(ci + p);
+  prefetch_line(av + p);
+}
+
 // ----------------------------------------------------------------------------------------------
 // Row blocks per block: a block may walk `rpt` consecutive row blocks, so that fewer blocks are
 // launched and the neighbour rows one row block gathers are still in L1 for the next.  The
@@ -119,6 +130,9 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int 
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * RowBlocks<T>::of(rpt) * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < RowBlocks<T>::of(rpt); ++rr) {
   const int row = (blockIdx.x * RowBlocks<T>::of(rpt) + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
@@ -133,12 +147,12 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int 
   T w = T(0);
   if (OP != OP_SPMM) {
 #pragma unroll
-    for (int c = 0; c < CH; ++c) Vec16<T>::load(Y + base + (c * tpr + lane) * V, y[c]);
+    for (int c = 0; c < CH; ++c) ldg16<T>(Y + base + (c * tpr + lane) * V, y[c]);
   }
   if (OP == OP_JACOBI) {
     w = omega * dinv[row];
 #pragma unroll
-    for (int c = 0; c < CH; ++c) Vec16<T>::load(Z + base + (c * tpr + lane) * V, z[c]);
+    for (int c = 0; c < CH; ++c) ldg16<T>(Z + base + (c * tpr + lane) * V, z[c]);
   }
   gather_rows<T, CH>(ci, av, nullptr, T(0), X, rp[row], rp[row + 1], lane, tpr, ldk, acc);
 #pragma unroll
@@ -179,10 +193,10 @@ void rowop(const Launch& L, RowOp op, const DCsr& S, const T* X, const T* Y, con
   }
   PASM_DISPATCH_CH(g.ch,
     switch (op) {
-      case OP_JACOBI: k_rowop<T, CH, OP_JACOBI><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_RESID: k_rowop<T, CH, OP_RESID><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_SPMM: k_rowop<T, CH, OP_SPMM><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_SPMM_ADD: k_rowop<T, CH, OP_SPMM_ADD><<<grid, kBlock, 0, L.s>>>(S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
+      case OP_JACOBI: launch(L, k_rowop<T, CH, OP_JACOBI>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
+      case OP_RESID: launch(L, k_rowop<T, CH, OP_RESID>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
+      case OP_SPMM: launch(L, k_rowop<T, CH, OP_SPMM>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
+      case OP_SPMM_ADD: launch(L, k_rowop<T, CH, OP_SPMM_ADD>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
     });
   L.bump();
 }
@@ -210,12 +224,15 @@ __global__ void __launch_bounds__(kBlock) k_prolong_jacobi(int n, const int* __r
   const int rpb = kBlock / tpr;
   const int row = blockIdx.x * rpb + threadIdx.x / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(arp, aci, av, row, n);
+  pdl_wait();
   if (row >= n) return;
   const size_t base = (size_t)row * ldk;
   float y[CH][V], z[CH][V], acc[CH][V];
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
-    Vec16<float>::load(F + base + (c * tpr + lane) * V, y[c]);
+    ldg16<float>(F + base + (c * tpr + lane) * V, y[c]);
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[c][v] = z[c][v] = 0.f;
   }
@@ -275,7 +292,7 @@ void prolong_jacobi(const Launch& L, const DCsr& A, const DCsr& P, const float* 
     L.rows(A.n_rows);
     L.begin(KC_JACOBI, bytes, 2.0 * (nnz + pnnz) * ldk + 4.0 * rows * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_prolong_jacobi<CH><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, A.v32, P.rp, P.ci,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_prolong_jacobi<CH>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.v32, P.rp, P.ci,
                                                                           P.v32, X, Ec, F, dinv, omega, out, ldk,
                                                                           g.tpr));
   L.bump();
@@ -286,13 +303,15 @@ template <typename T>
 __global__ void k_jacobi_zero(int64_t total, int ldk, const T* __restrict__ dinv, T omega, const T* __restrict__ F,
                               T* __restrict__ out) {
   constexpr int V = Vec16<T>::N;
+  pdl_trigger();
+  pdl_wait();
   const int64_t nv = total / V;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nv; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = i * V;
     const int64_t row = e / ldk;
     const T w = omega * dinv[row];
     T f[V], r[V];
-    Vec16<T>::load(F + e, f);
+    ldg16<T>(F + e, f);
 #pragma unroll
     for (int v = 0; v < V; ++v) r[v] = w * f[v];
     Vec16<T>::store(out + e, r);
@@ -306,7 +325,7 @@ void jacobi_zero(const Launch& L, int n, const T* dinv, T omega, const T* F, T* 
   const int64_t nv = total / Vec16<T>::N;
   int grid = (int)std::min<int64_t>((nv + kBlock - 1) / kBlock, 152 * 16);
   L.begin(KC_JACOBI0, (2.0 * total + n) * sizeof(T), 2.0 * total);
-  k_jacobi_zero<T><<<grid, kBlock, 0, L.s>>>(total, ldk, dinv, omega, F, out);
+  launch(L, k_jacobi_zero<T>, grid, kBlock, 0, total, ldk, dinv, omega, F, out);
   L.bump();
 }
 template void jacobi_zero<double>(const Launch&, int, const double*, double, const double*, double*, int);
@@ -334,6 +353,9 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<T>::gather) k_jacobi2_zero(i
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * RowBlocks<T>::of(rpt) * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < RowBlocks<T>::of(rpt); ++rr) {
   const int row = (blockIdx.x * RowBlocks<T>::of(rpt) + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
@@ -372,6 +394,9 @@ __global__ void __launch_bounds__(kBlock, MinBlocks<T>::gather) k_resid_restrict
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rrp, rci, rv, blockIdx.x * RowBlocks<T>::of(rpt) * rpb + threadIdx.x / tpr, nc);
+  pdl_wait();
   for (int rr = 0; rr < RowBlocks<T>::of(rpt); ++rr) {
   const int row = (blockIdx.x * RowBlocks<T>::of(rpt) + rr) * rpb + threadIdx.x / tpr;
   if (row >= nc) return;
@@ -417,7 +442,7 @@ void jacobi2_zero(const Launch& L, const DCsr& A, const T* dinv, T omega, const 
             3.0 * nnz * ldk + 2.0 * rows * ldk);
   }
   const T* ws = scaled_vals<T>(A);
-  PASM_DISPATCH_CH(g.ch, k_jacobi2_zero<T, CH><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, ws ? ws : vals<T>(A),
+  PASM_DISPATCH_CH(g.ch, launch(L, k_jacobi2_zero<T, CH>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, ws ? ws : vals<T>(A),
                                                                           dinv, omega, F, out, ldk, g.tpr,
                                                                           ws ? 1 : 0, rpt));
   L.bump();
@@ -437,7 +462,7 @@ void resid_restrict(const Launch& L, const DCsr& R, const DCsr& A, const T* E, c
                           nc * ldk * sz,
             2.0 * (double)(A.nnz + R.nnz) * ldk + nf * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_resid_restrict<T, CH><<<grid, kBlock, 0, L.s>>>(R.n_rows, R.rp, R.ci, vals<T>(R), A.rp,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_resid_restrict<T, CH>, grid, kBlock, 0, R.n_rows, R.rp, R.ci, vals<T>(R), A.rp,
                                                                             A.ci, vals<T>(A), E, F, out, ldk, g.tpr, rpt));
   L.bump();
 }
@@ -454,6 +479,10 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<float, CH>::v)) k_restri
   constexpr int V = 4;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rrp, rci, rv, blockIdx.x * rpt * rpb + threadIdx.x / tpr, nc);
+  prefetch_row(qrp, qci, qv, blockIdx.x * rpt * rpb + threadIdx.x / tpr, nc);
+  pdl_wait();
   for (int rr = 0; rr < rpt; ++rr) {
     const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
     if (row >= nc) return;
@@ -488,7 +517,7 @@ void restrict_first(const Launch& L, const DCsr& R, const DCsr& RA, const float*
     L.begin(KC_RESID, (double)(R.nnz + RA.nnz) * 8.0 + 2.0 * (nc + 1) * 4.0 + 2.0 * nf * ldk * 4.0 + nc * ldk * 4.0,
             2.0 * (double)(R.nnz + RA.nnz) * ldk + nc * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_restrict_first<CH><<<grid, kBlock, 0, L.s>>>(R.n_rows, R.rp, R.ci, R.v32, RA.rp, RA.ci,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_restrict_first<CH>, grid, kBlock, 0, R.n_rows, R.rp, R.ci, R.v32, RA.rp, RA.ci,
                                                                          RA.v32, E, F, out, ldk, g.tpr, rpt));
   L.bump();
 }
@@ -535,6 +564,10 @@ __global__ void __launch_bounds__(kBlock) k_outer_rhs_res(int n, const int* __re
   const int rpb = kBlock / tpr;
   const int row = blockIdx.x * rpb + threadIdx.x / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(mrp, mci, mval, row, n);
+  prefetch_row(arp, aci, aval, row, n);
+  pdl_wait();
   if (row >= n) return;
   double mu[CH][2], au[CH][2];
   gather_row64<CH>(mrp, mci, mval, U, row, lane, tpr, ldk, mu);
@@ -543,7 +576,9 @@ __global__ void __launch_bounds__(kBlock) k_outer_rhs_res(int n, const int* __re
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    const double f0 = lam[col] * mu[c][0], f1 = lam[col + 1] * mu[c][1];
+    double l[2];
+    ldg16<double>(lam + col, l);
+    const double f0 = l[0] * mu[c][0], f1 = l[1] * mu[c][1];
     *reinterpret_cast<double2*>(Fd + base + col) = make_double2(f0, f1);
     store_vec2<TV>(R + base + col, f0 - au[c][0], f1 - au[c][1]);
   }
@@ -556,6 +591,9 @@ __global__ void __launch_bounds__(kBlock) k_outer_res(int n, const int* __restri
   const int rpb = kBlock / tpr;
   const int row = blockIdx.x * rpb + threadIdx.x / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(arp, aci, aval, row, n);
+  pdl_wait();
   if (row >= n) return;
   double ax[CH][2];
   gather_row64<CH>(arp, aci, aval, X, row, lane, tpr, ldk, ax);
@@ -563,13 +601,16 @@ __global__ void __launch_bounds__(kBlock) k_outer_res(int n, const int* __restri
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    double2 f = *reinterpret_cast<const double2*>(Fd + base + col);
-    store_vec2<TV>(R + base + col, f.x - ax[c][0], f.y - ax[c][1]);
+    double f[2];
+    ldg16<double>(Fd + base + col, f);
+    store_vec2<TV>(R + base + col, f[0] - ax[c][0], f[1] - ax[c][1]);
   }
 }
 
 template <typename TV>
-__global__ void k_outer_axpy(int64_t total, const double* B, const TV* __restrict__ E, double* X) {
+__global__ void k_outer_axpy(int64_t total, const double* B, const TV* E, double* X) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t np = total / 2;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < np; i += (int64_t)gridDim.x * blockDim.x) {
     double e[2];
@@ -593,7 +634,7 @@ void outer_rhs_residual(const Launch& L, const DCsr& A, const DCsr& M, const dou
     L.begin(KC_OUTER_RHS, nnz * 12.0 + 2 * (n + 1) * 4.0 + n * ldk * (16.0 + sizeof(TV)),
             2.0 * nnz * ldk + 2.0 * n * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_outer_rhs_res<TV, CH><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, A.v64, M.rp, M.ci,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_outer_rhs_res<TV, CH>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.v64, M.rp, M.ci,
                                                                             M.v64, lam, U, Fd, R, ldk, g.tpr));
   L.bump();
 }
@@ -607,7 +648,7 @@ void outer_residual(const Launch& L, const DCsr& A, const double* Fd, const doub
     L.rows(A.n_rows);
     L.begin(KC_OUTER_RES, nnz * 12.0 + (n + 1) * 4.0 + n * ldk * (16.0 + sizeof(TV)), 2.0 * nnz * ldk + n * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_outer_res<TV, CH><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, A.v64, Fd, X, R, ldk,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_outer_res<TV, CH>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.v64, Fd, X, R, ldk,
                                                                         g.tpr));
   L.bump();
 }
@@ -616,7 +657,7 @@ void outer_axpy(const Launch& L, int n, const double* B, const TV* E, double* X,
   const int64_t total = (int64_t)n * ldk;
   int grid = (int)std::min<int64_t>((total / 2 + kBlock - 1) / kBlock, 152 * 16);
   L.begin(KC_AXPY, (double)total * (16.0 + sizeof(TV)), (double)total);
-  k_outer_axpy<TV><<<grid, kBlock, 0, L.s>>>(total, B, E, X);
+  launch(L, k_outer_axpy<TV>, grid, kBlock, 0, total, B, E, X);
   L.bump();
 }
 template void outer_rhs_residual<double>(const Launch&, const DCsr&, const DCsr&, const double*, const double*,
@@ -645,6 +686,10 @@ __global__ void __launch_bounds__(kBlock) k_border(int n, const int* __restrict_
   double sA[CH][2], sM[CH][2];
 #pragma unroll
   for (int c = 0; c < CH; ++c) sA[c][0] = sA[c][1] = sM[c][0] = sM[c][1] = 0.0;
+  pdl_trigger();
+  prefetch_row(arp, aci, aval, blockIdx.x * rpb + grp, n);
+  prefetch_row(mrp, mci, mval, blockIdx.x * rpb + grp, n);
+  pdl_wait();
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
     double ya[CH][2], ym[CH][2];
     gather_row64<CH>(arp, aci, aval, X, row, lane, tpr, ldk, ya);
@@ -653,13 +698,14 @@ __global__ void __launch_bounds__(kBlock) k_border(int n, const int* __restrict_
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       const int col = (c * tpr + lane) * 2;
-      double2 x = *reinterpret_cast<const double2*>(X + base + col);
+      double x[2];
+      ldg16<double>(X + base + col, x);
       *reinterpret_cast<double2*>(YA + base + col) = make_double2(ya[c][0], ya[c][1]);
       *reinterpret_cast<double2*>(YM + base + col) = make_double2(ym[c][0], ym[c][1]);
-      sA[c][0] = fma(x.x, ya[c][0], sA[c][0]);
-      sA[c][1] = fma(x.y, ya[c][1], sA[c][1]);
-      sM[c][0] = fma(x.x, ym[c][0], sM[c][0]);
-      sM[c][1] = fma(x.y, ym[c][1], sM[c][1]);
+      sA[c][0] = fma(x[0], ya[c][0], sA[c][0]);
+      sA[c][1] = fma(x[1], ya[c][1], sA[c][1]);
+      sM[c][0] = fma(x[0], ym[c][0], sM[c][0]);
+      sM[c][1] = fma(x[1], ym[c][1], sM[c][1]);
     }
   }
 #pragma unroll
@@ -693,7 +739,7 @@ int border_products(const Launch& L, const DCsr& A, const DCsr& M, const double*
     L.rows(A.n_rows);
     L.begin(KC_BORDER, nnz * 12.0 + 2 * (n + 1) * 4.0 + 3.0 * n * ldk * 8.0, 2.0 * nnz * ldk + 4.0 * n * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_border<CH><<<grid, kBlock, smem, L.s>>>(A.n_rows, A.rp, A.ci, A.v64, M.rp, M.ci, M.v64, X,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_border<CH>, grid, kBlock, smem, A.n_rows, A.rp, A.ci, A.v64, M.rp, M.ci, M.v64, X,
                                                                     YA, YM, partials, ldk, g.tpr));
   L.bump();
   return grid;
@@ -704,9 +750,11 @@ int border_products(const Launch& L, const DCsr& A, const DCsr& M, const double*
 __global__ void __launch_bounds__(128) k_colsum(const double* __restrict__ partials, int nblk, int width,
                                                 double* __restrict__ out) {
   __shared__ double red[4];
+  pdl_trigger();
+  pdl_wait();
   const int t = blockIdx.x;
   double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += 128) s += partials[(size_t)b * width + t];
+  for (int b = threadIdx.x; b < nblk; b += 128) s += ld1(partials + (size_t)b * width + t);
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
@@ -725,22 +773,25 @@ __global__ void __launch_bounds__(kBlock) k_residual_partials(int n, int ldk, co
                                                               const double* __restrict__ U,
                                                               double* __restrict__ partials) {
   __shared__ double red[kBlock * 4];
+  pdl_trigger();
+  pdl_wait();
   const int cpairs = ldk / 2, rpb = kBlock / cpairs;
   const int cp = threadIdx.x % cpairs, ro = threadIdx.x / cpairs;
   double rr0 = 0.0, rr1 = 0.0, um0 = 0.0, um1 = 0.0;
   if (ro < rpb) {
     for (int row = blockIdx.x * rpb + ro; row < n; row += gridDim.x * rpb) {
       const size_t off = (size_t)row * ldk + 2 * cp;
-      const double r0 = (double)R[off], r1 = (double)R[off + 1];
+      const double r0 = (double)ld1(R + off), r1 = (double)ld1(R + off + 1);
       double m0, m1, u0, u1;
       if (FF) {
-        const float4 f = *reinterpret_cast<const float4*>(Fd + off);
-        const float4 u = *reinterpret_cast<const float4*>(U + off);
-        m0 = (double)f.x + (double)f.z; m1 = (double)f.y + (double)f.w;   // chunk = hi, hi, lo, lo
-        u0 = (double)u.x + (double)u.z; u1 = (double)u.y + (double)u.w;
+        float f[4], u[4];   // chunk = hi, hi, lo, lo
+        ldg16<float>(reinterpret_cast<const float*>(Fd + off), f);
+        ldg16<float>(reinterpret_cast<const float*>(U + off), u);
+        m0 = (double)f[0] + (double)f[2]; m1 = (double)f[1] + (double)f[3];
+        u0 = (double)u[0] + (double)u[2]; u1 = (double)u[1] + (double)u[3];
       } else {
-        m0 = Fd[off]; m1 = Fd[off + 1];
-        u0 = U[off]; u1 = U[off + 1];
+        m0 = ld1(Fd + off); m1 = ld1(Fd + off + 1);
+        u0 = ld1(U + off); u1 = ld1(U + off + 1);
       }
       rr0 = fma(r0, r0, rr0); rr1 = fma(r1, r1, rr1);
       um0 = fma(u0, m0, um0); um1 = fma(u1, m1, um1);
@@ -765,8 +816,8 @@ int residual_partials(const Launch& L, int n, int ldk, const TR* R, bool ff, con
   const int rpb = kBlock / (ldk / 2);
   const int grid = std::max(1, std::min((n + rpb - 1) / rpb, max_blocks));
   L.begin(KC_COLSUM, (double)n * ldk * (sizeof(TR) + 16.0), 4.0 * n * ldk);
-  if (ff) k_residual_partials<TR, true><<<grid, kBlock, 0, L.s>>>(n, ldk, R, Fd, U, partials);
-  else k_residual_partials<TR, false><<<grid, kBlock, 0, L.s>>>(n, ldk, R, Fd, U, partials);
+  if (ff) launch(L, k_residual_partials<TR, true>, grid, kBlock, 0, n, ldk, R, Fd, U, partials);
+  else launch(L, k_residual_partials<TR, false>, grid, kBlock, 0, n, ldk, R, Fd, U, partials);
   L.bump();
   return grid;
 }
@@ -778,7 +829,7 @@ template int residual_partials<double>(const Launch&, int, int, const double*, b
 void column_sums(const Launch& L, const double* partials, int nblk, int nq, int ldk, double* out) {
   const int width = nq * ldk;
   L.begin(KC_COLSUM, (double)nblk * width * 8.0 + width * 8.0, (double)nblk * width);
-  k_colsum<<<width, 128, 0, L.s>>>(partials, nblk, width, out);
+  launch(L, k_colsum, width, 128, 0, partials, nblk, width, out);
   L.bump();
 }
 
@@ -804,9 +855,11 @@ __global__ void __launch_bounds__(kBlock) k_dense_mm(int m, int p, const T* __re
   T s[kDenseRows];
 #pragma unroll
   for (int r = 0; r < kDenseRows; ++r) s[r] = T(0);
+  pdl_trigger();
+  pdl_wait();
 #pragma unroll 8
   for (int j = part; j < p; j += kDenseParts) {
-    const T b = __ldg(B + (size_t)j * ldk + c);
+    const T b = ld1(B + (size_t)j * ldk + c);
 #pragma unroll
     for (int r = 0; r < kDenseRows; ++r) s[r] = fma(__ldg(d[r] + (size_t)j * dj), b, s[r]);
   }
@@ -828,7 +881,7 @@ void dense_mm(const Launch& L, int m, int p, const T* D, int ldd, bool trans, co
   const int cols = std::min(ldk, 32), rows = kDenseRows * (32 / cols);
   dim3 grid(ldk / cols, (m + rows - 1) / rows);
   L.begin(KC_DENSE, ((double)m * p + (double)p * ldk + (double)m * ldk) * sizeof(T), 2.0 * m * p * ldk);
-  k_dense_mm<T><<<grid, kBlock, 0, L.s>>>(m, p, D, ldd, trans ? 1 : 0, B, C, ldk, cols);
+  launch(L, k_dense_mm<T>, grid, kBlock, 0, m, p, D, ldd, trans ? 1 : 0, B, C, ldk, cols);
   L.bump();
 }
 template void dense_mm<double>(const Launch&, int, int, const double*, int, bool, const double*, double*, int);
@@ -836,6 +889,8 @@ template void dense_mm<float>(const Launch&, int, int, const float*, int, bool, 
 
 __global__ void k_coarse_init(int NH, int k, const double* __restrict__ Q, const double* __restrict__ lamH,
                               double* __restrict__ W0, double* __restrict__ lam, int ldk) {
+  pdl_trigger();
+  pdl_wait();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y;
   if (c >= ldk) return;
@@ -847,7 +902,7 @@ void coarse_init(const Launch& L, int NH, int k, const double* Q, const double* 
                  int ldk) {
   dim3 grid((ldk + 63) / 64, NH);
   L.begin(KC_INIT, (double)NH * ldk * 16.0, 0.0);
-  k_coarse_init<<<grid, 64, 0, L.s>>>(NH, k, Q, lamH, W0, lam, ldk);
+  launch(L, k_coarse_init, grid, 64, 0, NH, k, Q, lamH, W0, lam, ldk);
   L.bump();
 }
 
@@ -863,14 +918,14 @@ __global__ void __launch_bounds__(kBlock) k_update(int n, const int* __restrict_
   const int rpb = kBlock / tpr;
   const int row = blockIdx.x * rpb + threadIdx.x / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  if (!identity) prefetch_row(rp, ci, pv, row, n);
+  pdl_wait();
   if (row >= n) return;
   double pw[CH][2];
   if (identity) {
 #pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      double2 w = *reinterpret_cast<const double2*>(W + (size_t)row * ldk + (c * tpr + lane) * 2);
-      pw[c][0] = w.x; pw[c][1] = w.y;
-    }
+    for (int c = 0; c < CH; ++c) ldg16<double>(W + (size_t)row * ldk + (c * tpr + lane) * 2, pw[c]);
   } else {
     gather_row64<CH>(rp, ci, pv, W, row, lane, tpr, ldk, pw);
   }
@@ -878,11 +933,13 @@ __global__ void __launch_bounds__(kBlock) k_update(int n, const int* __restrict_
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
     const int col = (c * tpr + lane) * 2;
-    double2 x = *reinterpret_cast<const double2*>(X + base + col);
-    double2 u = *reinterpret_cast<const double2*>(U + base + col);
-    if (upd[col]) u.x = fma(alpha[col], x.x, pw[c][0]);
-    if (upd[col + 1]) u.y = fma(alpha[col + 1], x.y, pw[c][1]);
-    *reinterpret_cast<double2*>(U + base + col) = u;
+    double x[2], u[2], a[2];
+    ldg16<double>(X + base + col, x);
+    ldg16<double>(U + base + col, u);
+    ldg16<double>(alpha + col, a);
+    if (ld1(upd + col)) u[0] = fma(a[0], x[0], pw[c][0]);
+    if (ld1(upd + col + 1)) u[1] = fma(a[1], x[1], pw[c][1]);
+    *reinterpret_cast<double2*>(U + base + col) = make_double2(u[0], u[1]);
   }
 }
 
@@ -896,7 +953,7 @@ void update_pairs(const Launch& L, const DCsr& P, const double* W, const double*
     L.begin(KC_UPDATE, nnz * 12.0 + (n + 1) * 4.0 + (double)P.n_cols * ldk * 8.0 + 3.0 * n * ldk * 8.0,
             2.0 * nnz * ldk + 2.0 * n * ldk);
   }
-  PASM_DISPATCH_CH(g.ch, k_update<CH><<<grid, kBlock, 0, L.s>>>(P.n_rows, P.rp, P.ci, P.v64, W, X, alpha, upd, U,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_update<CH>, grid, kBlock, 0, P.n_rows, P.rp, P.ci, P.v64, W, X, alpha, upd, U,
                                                                  ldk, g.tpr, 0));
   L.bump();
 }
@@ -906,24 +963,28 @@ void update_pairs_identity(const Launch& L, int n, const double* W, const double
   const int rpb = kBlock / g.tpr;
   const int grid = (n + rpb - 1) / rpb;
   L.begin(KC_UPDATE, 4.0 * n * ldk * 8.0, 2.0 * n * ldk);
-  PASM_DISPATCH_CH(g.ch, k_update<CH><<<grid, kBlock, 0, L.s>>>(n, nullptr, nullptr, nullptr, W, X, alpha, upd, U,
+  PASM_DISPATCH_CH(g.ch, launch(L, k_update<CH>, grid, kBlock, 0, n, nullptr, nullptr, nullptr, W, X, alpha, upd, U,
                                                                  ldk, g.tpr, 1));
   L.bump();
 }
 
 __global__ void k_count_active(const int* __restrict__ active, int k, int* out) {
+  pdl_trigger();
+  pdl_wait();
   int c = 0;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) c += active[i] != 0;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) c += ld1(active + i) != 0;
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (threadIdx.x == 0) *out = c;
 }
 void count_active(const Launch& L, const int* active, int k, int* out) {
   L.begin(KC_COUNT, k * 4.0, 0.0);
-  k_count_active<<<1, 32, 0, L.s>>>(active, k, out);
+  launch(L, k_count_active, 1, 32, 0, active, k, out);
   L.bump();
 }
 
-__global__ void k_cast_d2f(const double* __restrict__ in, float* __restrict__ out, int64_t count) {
+__global__ void k_cast_d2f(const double* in, float* out, int64_t count) {
+  pdl_trigger();
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
     out[i] = (float)in[i];
 }
@@ -931,7 +992,7 @@ void cast_d2f(const Launch& L, const double* in, float* out, int64_t count) {
   if (count == 0) return;
   int grid = (int)std::min<int64_t>((count + kBlock - 1) / kBlock, 152 * 16);
   L.begin(KC_CAST, count * 12.0, 0.0);
-  k_cast_d2f<<<grid, kBlock, 0, L.s>>>(in, out, count);
+  launch(L, k_cast_d2f, grid, kBlock, 0, in, out, count);
   L.bump();
 }
 
@@ -952,6 +1013,9 @@ __global__ void __launch_bounds__(kBlock)
   constexpr int V = 4;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * rpt * rpb + threadIdx.x / tpr, n);
+  pdl_wait();
   for (int rr = 0; rr < rpt; ++rr) {
   const int row = (blockIdx.x * rpt + rr) * rpb + threadIdx.x / tpr;
   if (row >= n) return;
@@ -964,8 +1028,8 @@ __global__ void __launch_bounds__(kBlock)
   float y[CH][V], z[CH][V];
 #pragma unroll
   for (int c = 0; c < CH; ++c) {
-    Vec16<float>::load(F + base + (c * tpr + lane) * V, y[c]);
-    Vec16<float>::load(E + base + (c * tpr + lane) * V, z[c]);
+    ldg16<float>(F + base + (c * tpr + lane) * V, y[c]);
+    ldg16<float>(E + base + (c * tpr + lane) * V, z[c]);
   }
   const float w = omega * dinv[row];
   gather_rows<float, CH>(ci, av, nullptr, 0.f, E, rp[row], rp[row + 1], lane, tpr, ldk, acc);
@@ -1014,10 +1078,10 @@ void jacobi_axpy_ff(const Launch& L, const DCsr& A, const float* E, const float*
             2.0 * nnz * ldk + 4.0 * rows * ldk);
   }
   if (b_ff) {
-    PASM_DISPATCH_CH(g.ch, k_jacobi_axpy_ff<CH, true><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, A.v32, E, F, dinv,
+    PASM_DISPATCH_CH(g.ch, launch(L, k_jacobi_axpy_ff<CH, true>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.v32, E, F, dinv,
                                                                                  omega, B, X, ldk, g.tpr, rpt));
   } else {
-    PASM_DISPATCH_CH(g.ch, k_jacobi_axpy_ff<CH, false><<<grid, kBlock, 0, L.s>>>(A.n_rows, A.rp, A.ci, A.v32, E, F,
+    PASM_DISPATCH_CH(g.ch, launch(L, k_jacobi_axpy_ff<CH, false>, grid, kBlock, 0, A.n_rows, A.rp, A.ci, A.v32, E, F,
                                                                                   dinv, omega, B, X, ldk, g.tpr, rpt));
   }
   L.bump();

@@ -53,6 +53,8 @@ struct Launch {
   Tracer* tr = nullptr;
   int geo = 0;  // row-group kernels: 16-byte chunks per thread (0 = default; set by the autotuner)
   int rpt = 0;  // float32 row kernels: row blocks each block walks (0 = by size; set by the autotuner)
+  bool pdl = true;  // programmatic dependent launch (see `launch`); off where an operand that is static in a
+                    // context may have been written by the kernel before
   void begin(int cls, double bytes, double flops) const { if (tr) tracer_begin(tr, s, cls, bytes, flops); }
   void rows(int n) const { if (tr) tracer_rows(tr, n); }
   void bump() const {
@@ -60,6 +62,29 @@ struct Launch {
     if (tr) tracer_end(tr, s);
   }
 };
+
+// Programmatic dependent launch: a kernel of the step may start while the one before it in the stream
+// drains.  Every kernel launched through `launch` calls pdl_trigger() first (the next kernel's blocks
+// may take the slots this grid leaves), then reads only what no kernel of a step writes (matrices,
+// index arrays), then pdl_wait() in every thread -- which returns when all earlier kernels have
+// completed and their writes are visible -- before it touches anything else or returns.  Data that
+// other kernels write is loaded through the volatile loads of common.cuh: a load through a const
+// __restrict__ pointer or __ldg is one the compiler may move above the wait.
+// A launch gap between two small kernels costs 1 to 1.5 us; a step has 40 to 80.
+template <typename... P, typename... A>
+inline void launch(const Launch& L, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = L.pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 enum RowOp { OP_JACOBI = 0, OP_RESID = 1, OP_SPMM = 2, OP_SPMM_ADD = 3 };
 

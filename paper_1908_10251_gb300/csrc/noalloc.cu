@@ -74,6 +74,7 @@ extern "C" int pasm_border_noalloc(int n, const int32_t* A_row_ptr, const int32_
   M.rp = const_cast<int*>(M_row_ptr); M.ci = const_cast<int*>(M_col); M.v64 = const_cast<double*>(M_val);
   Launch L;
   L.s = static_cast<cudaStream_t>(stream);
+  L.pdl = false;  // the caller may have written the matrices in the kernel before
   // every scratch entry read below is written earlier in the same call, so no part of it needs clearing
   const int nblk = border_products(L, A, M, X, YA, YM, scratch, k, max_blocks);
   double* sums = scratch + (size_t)nblk * 2 * k;

@@ -1079,7 +1079,7 @@ static int autotune(pasm_ctx* c) {
       // into scratch (YM) instead of U
       CK(cudaMemsetAsync(c->upd, 1, sizeof(int) * (size_t)ldk, c->s));
       pick(l, PASM_TILE_UPDATE, c64, [&](const Launch& L) {
-        update_pairs_ff(L, &v.P, v.n, wsrc, l - 1 >= 1, c->X, c->alpha, c->upd, c->YM, nullptr, ldk);
+        update_pairs_ff(L, &v.P, v.n, wsrc, l - 1 >= 1, c->X, c->alpha, c->upd, nullptr, c->YM, ldk);
       }, true);
       CK(cudaMemsetAsync(c->upd, 0, sizeof(int) * (size_t)ldk, c->s));
     } else {

@@ -108,7 +108,7 @@ __device__ __forceinline__ const double* bcol(const double* B0, const double* B1
   return n < ldk ? B0 + n : B1 + (n - ldk);
 }
 
-__device__ __forceinline__ uint64_t ld_bits(const double* p) { return (uint64_t)__double_as_longlong(__ldg(p)); }
+__device__ __forceinline__ uint64_t ld_bits(const double* p) { return (uint64_t)__double_as_longlong(ld1(p)); }
 
 __device__ __forceinline__ void red_add(unsigned long long* p, long long v) {
   asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"((unsigned long long)v) : "memory");
@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kThreads)
   const int n0 = blockIdx.x * kN, mt = blockIdx.y, ch = blockIdx.z;
   const int kc0 = ch * kKC, kw = min(kKC, Kpad - kc0);
   const uint32_t bar_load = smem_u32(mbar), bar_mma = smem_u32(mbar + 1);
+  pdl_trigger();
 
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_load));
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(kThreads)
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
+  pdl_wait();   // A's planes are static and on their way
   // column exponents over the whole inner dimension: |B[j][n]| < 2^cexp[n] from the largest high
   // word (an all-zero high word with low bits set is subnormal: key 1); a NaN/Inf marks the column.
   // Loads use clamped indices (always valid addresses) so that each batch is issued at once.
@@ -231,7 +233,9 @@ __global__ void __launch_bounds__(kThreads)
       uint2 w[8];   // low, high word
 #pragma unroll
       for (int q = 0; q < 8; ++q)
-        w[q] = __ldg(reinterpret_cast<const uint2*>(cp + (size_t)min(j0 + q * kParts, K - 1) * ldk));
+        asm volatile("ld.global.v2.u32 {%0, %1}, [%2];"
+                     : "=r"(w[q].x), "=r"(w[q].y)
+                     : "l"(cp + (size_t)min(j0 + q * kParts, K - 1) * ldk));
 #pragma unroll
       for (int q = 0; q < 8; ++q) {   // a clamped load repeats the last row
         hmax = max(hmax, w[q].y & 0x7FFFFFFFu);
@@ -448,7 +452,7 @@ void proj_tc(const Launch& L, const SplitMat& A, const double* B0, const double*
   dim3 grid((ncols + kN - 1) / kN, A.mtiles, (A.Kpad + kKC - 1) / kKC);
   const double m = A.m, K = A.K, n = ncols;
   L.begin(KC_PROJ, (m * K + K * n + m * n) * 8.0, 2.0 * m * K * n);
-  k_proj_tc<<<grid, kThreads, kSmem, L.s>>>(A.m, A.K, A.Kpad, A.planes, A.rexp, B0, B1, C0, C1, ldk, ncols, hl,
+  launch(L, k_proj_tc, grid, kThreads, kSmem, A.m, A.K, A.Kpad, A.planes, A.rexp, B0, B1, C0, C1, ldk, ncols, hl,
                                             tickets, err, wait_limit > 0 ? wait_limit : kWaitLimit, skip_mma);
   L.bump();
 }

@@ -420,6 +420,8 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
   // 8 / cs warps of every SM's float64 pipe instead of 8 of one (216 -> 87 us at N_H = 361, k = 37 with
   // the block-wide pole lists below)
   const int gwarp = warp * cs + rank, nwarps = cs * kSecWarps;
+  pdl_trigger();
+  pdl_wait();
   if (!a.active[i]) {
     if (tid == 0 && lead) a.upd[i] = 0;
     return;
@@ -743,13 +745,15 @@ void secular_select(const Launch& L, const SecularArgs& a0) {
   cfg.blockDim = dim3(kSecThreads);
   cfg.dynamicSmemBytes = secular_smem(a.NH);
   cfg.stream = L.s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)a.cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = L.pdl ? 2 : 1;
   cudaLaunchKernelEx(&cfg, k_secular, a);
   L.bump();
 }
