@@ -1111,15 +1111,17 @@ __device__ __forceinline__ void block_column_partials(const T (&s)[CH][Vec16<T>:
   }
 }
 
-// r = f - A x (x == nullptr: r = f), p = r, partial sums of r.r
+// R = F - A X, partial sums of r.r
 template <typename T, int CH>
 __global__ void __launch_bounds__(kBlock) k_cg_start(int n, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                      const T* __restrict__ av, const T* __restrict__ X,
-                                                      const T* __restrict__ F, T* __restrict__ R, T* __restrict__ P,
-                                                      double* __restrict__ partial, int ldk, int tpr) {
+                                                      const T* __restrict__ av, const T* X, const T* F, T* R,
+                                                      double* partial, int ldk, int tpr) {
   extern __shared__ double red[];
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr, grp = threadIdx.x / tpr, lane = threadIdx.x % tpr;
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * rpb + grp, n);
+  pdl_wait();
   T s[CH][V];
 #pragma unroll
   for (int c = 0; c < CH; ++c)
@@ -1131,7 +1133,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_start(int n, const int* __restric
     for (int c = 0; c < CH; ++c)
 #pragma unroll
       for (int v = 0; v < V; ++v) acc[c][v] = T(0);
-    if (X) gather_rows<T, CH>(ci, av, nullptr, T(0), X, rp[row], rp[row + 1], lane, tpr, ldk, acc);
+    gather_rows<T, CH>(ci, av, nullptr, T(0), X, rp[row], rp[row + 1], lane, tpr, ldk, acc);
     const size_t base = (size_t)row * ldk;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
@@ -1144,26 +1146,28 @@ __global__ void __launch_bounds__(kBlock) k_cg_start(int n, const int* __restric
         s[c][v] = fma(r[v], r[v], s[c][v]);
       }
       Vec16<T>::store(R + off, r);
-      Vec16<T>::store(P + off, r);
     }
   }
   block_column_partials<T, CH>(s, red, grp, lane, tpr, rpb, ldk, partial);
 }
 
-// q = A p, partial sums of p.q
-template <typename T, int CH>
+// q = A p, partial sums of p.q; QOUT: q is stored (not needed in the last step); RR: also of p.p, in
+// partial2 (the first step, whose p is the residual)
+template <typename T, int CH, bool QOUT, bool RR>
 __global__ void __launch_bounds__(kBlock) k_cg_dir(int n, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                    const T* __restrict__ av, const T* __restrict__ P,
-                                                    T* __restrict__ Q, double* __restrict__ partial, int ldk,
-                                                    int tpr) {
+                                                    const T* __restrict__ av, const T* P, T* Q, double* partial,
+                                                    double* partial2, int ldk, int tpr) {
   extern __shared__ double red[];
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr, grp = threadIdx.x / tpr, lane = threadIdx.x % tpr;
-  T s[CH][V];
+  pdl_trigger();
+  prefetch_row(rp, ci, av, blockIdx.x * rpb + grp, n);
+  pdl_wait();
+  T s[CH][V], s2[CH][V];
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
-    for (int v = 0; v < V; ++v) s[c][v] = T(0);
+    for (int v = 0; v < V; ++v) s[c][v] = s2[c][v] = T(0);
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
     T acc[CH][V];
 #pragma unroll
@@ -1178,92 +1182,163 @@ __global__ void __launch_bounds__(kBlock) k_cg_dir(int n, const int* __restrict_
       T p[V];
       ldg16<T>(P + off, p);
 #pragma unroll
-      for (int v = 0; v < V; ++v) s[c][v] = fma(p[v], acc[c][v], s[c][v]);
-      Vec16<T>::store(Q + off, acc[c]);
+      for (int v = 0; v < V; ++v) {
+        s[c][v] = fma(p[v], acc[c][v], s[c][v]);
+        if (RR) s2[c][v] = fma(p[v], p[v], s2[c][v]);
+      }
+      if (QOUT) Vec16<T>::store(Q + off, acc[c]);
     }
   }
   block_column_partials<T, CH>(s, red, grp, lane, tpr, rpb, ldk, partial);
+  if (RR) {
+    __syncthreads();
+    block_column_partials<T, CH>(s2, red, grp, lane, tpr, rpb, ldk, partial2);
+  }
 }
 
-// x = (x_zero ? 0 : x) + alpha p, r -= alpha q, partial sums of r.r
+// Rn = R - alpha Q (Rn may be R), partial sums of the new r.r
 template <typename T, int CH>
-__global__ void __launch_bounds__(kBlock) k_cg_update(int n, T* __restrict__ X, T* __restrict__ R,
-                                                       const T* __restrict__ P, const T* __restrict__ Q,
-                                                       const double* __restrict__ alpha, double* __restrict__ partial,
-                                                       int ldk, int tpr, int x_zero) {
+__global__ void __launch_bounds__(kBlock) k_cg_resid(int n, const T* R, const T* Q, T* Rn, const double* alpha,
+                                                      double* partial, int ldk, int tpr) {
   extern __shared__ double red[];
   constexpr int V = Vec16<T>::N;
   const int rpb = kBlock / tpr, grp = threadIdx.x / tpr, lane = threadIdx.x % tpr;
+  pdl_trigger();
+  pdl_wait();
   T s[CH][V], a[CH][V];
 #pragma unroll
   for (int c = 0; c < CH; ++c)
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       s[c][v] = T(0);
-      a[c][v] = (T)alpha[(c * tpr + lane) * V + v];
+      a[c][v] = (T)ld1(alpha + (c * tpr + lane) * V + v);
     }
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
     const size_t base = (size_t)row * ldk;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       const size_t off = base + (c * tpr + lane) * V;
-      T x[V], r[V], p[V], q[V];
-      if (x_zero) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) x[v] = T(0);
-      } else {
-        Vec16<T>::load(X + off, x);
-      }
-      Vec16<T>::load(R + off, r);
-      ldg16<T>(P + off, p);
+      T r[V], q[V];
+      ldg16<T>(R + off, r);
       ldg16<T>(Q + off, q);
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        x[v] = fma(a[c][v], p[v], x[v]);
         r[v] = fma(-a[c][v], q[v], r[v]);
         s[c][v] = fma(r[v], r[v], s[c][v]);
       }
-      Vec16<T>::store(X + off, x);
-      Vec16<T>::store(R + off, r);
+      Vec16<T>::store(Rn + off, r);
     }
   }
   block_column_partials<T, CH>(s, red, grp, lane, tpr, rpb, ldk, partial);
 }
 
-// p = r + beta p
+// The coefficients of one 16-byte chunk of columns.
 template <typename T>
-__global__ void k_cg_pupdate(int64_t total, int ldk, const T* __restrict__ R, T* __restrict__ P,
-                             const double* __restrict__ beta) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x)
-    P[i] = fma((T)beta[i % ldk], P[i], R[i]);
+__device__ __forceinline__ void chunk_coef(const double* a, T (&o)[Vec16<T>::N]) {
+#pragma unroll
+  for (int v = 0; v < Vec16<T>::N; v += 2) {
+    double t[2];
+    ldg16<double>(a + v, t);
+    o[v] = (T)t[0];
+    o[v + 1] = (T)t[1];
+  }
+}
+
+// Pn = R + beta P (Pn may be R or P), and X += alpha P with XM = 2, X = alpha P with XM = 1
+template <typename T, int XM>
+__global__ void __launch_bounds__(kBlock) k_cg_pstep(int64_t total, int ldk, const T* R, const T* P, T* Pn,
+                                                      const double* beta, T* X, const double* alpha) {
+  constexpr int V = Vec16<T>::N;
+  pdl_trigger();
+  pdl_wait();
+  for (int64_t i = blockIdx.x * (int64_t)kBlock + threadIdx.x; i < total / V; i += (int64_t)gridDim.x * kBlock) {
+    const int c = (int)(i * V % ldk);
+    T r[V], p[V], x[V], o[V], b[V], al[V];
+    chunk_coef<T>(beta + c, b);
+    if (XM) chunk_coef<T>(alpha + c, al);
+    ldg16<T>(R + i * V, r);
+    ldg16<T>(P + i * V, p);
+    if (XM == 2) ldg16<T>(X + i * V, x);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      o[v] = fma(b[v], p[v], r[v]);
+      if (XM) x[v] = fma(al[v], p[v], XM == 2 ? x[v] : T(0));
+    }
+    Vec16<T>::store(Pn + i * V, o);
+    if (XM) Vec16<T>::store(X + i * V, x);
+  }
+}
+
+// X = (XZ ? 0 : X) + alpha0 P0 (P0 given) + alpha1 P1
+template <typename T, bool XZ>
+__global__ void __launch_bounds__(kBlock) k_cg_final(int64_t total, int ldk, T* X, const T* P0, const double* alpha0,
+                                                      const T* P1, const double* alpha1) {
+  constexpr int V = Vec16<T>::N;
+  pdl_trigger();
+  pdl_wait();
+  for (int64_t i = blockIdx.x * (int64_t)kBlock + threadIdx.x; i < total / V; i += (int64_t)gridDim.x * kBlock) {
+    const int c = (int)(i * V % ldk);
+    T x[V], p[V], q[V], a0[V], a1[V];
+    if (P0) chunk_coef<T>(alpha0 + c, a0);
+    chunk_coef<T>(alpha1 + c, a1);
+    if (XZ) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) x[v] = T(0);
+    } else {
+      ldg16<T>(X + i * V, x);
+    }
+    if (P0) ldg16<T>(P0 + i * V, p);
+    ldg16<T>(P1 + i * V, q);
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (P0) x[v] = fma(a0[v], p[v], x[v]);
+      x[v] = fma(a1[v], q[v], x[v]);
+    }
+    Vec16<T>::store(X + i * V, x);
+  }
 }
 
 // One block per column: s = sum of the partials; mode 0: rr = s; mode 1: alpha = rr / s
-// (0 if s <= 0); mode 2: beta = s / rr (0 if rr <= 0), rr = s.
-__global__ void __launch_bounds__(128) k_cg_scalar(const double* __restrict__ partial, int nblk, int ldk, int mode,
-                                                   double* __restrict__ rr, double* __restrict__ coef) {
-  __shared__ double w[4];
+// (0 if s <= 0); mode 2: beta = s / rr (0 if rr <= 0), rr = s; mode 3: rr = sum of partial2, then mode 1.
+__global__ void __launch_bounds__(128) k_cg_scalar(const double* partial, const double* partial2, int nblk, int ldk,
+                                                   int mode, double* rr, double* coef) {
+  __shared__ double w[4], w2[4];
+  pdl_trigger();
+  pdl_wait();
   const int c = blockIdx.x;
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += 128) s += partial[(size_t)b * ldk + c];
+  double s = 0.0, s2 = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nblk; b += 128) s += ld1(partial + (size_t)b * ldk + c);
+  if (mode == 3) {
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nblk; b += 128) s2 += ld1(partial2 + (size_t)b * ldk + c);
+  }
   s = warp_sum(s);
-  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = s;
+  s2 = warp_sum(s2);
+  if ((threadIdx.x & 31) == 0) { w[threadIdx.x >> 5] = s; w2[threadIdx.x >> 5] = s2; }
   __syncthreads();
   if (threadIdx.x == 0) {
     s = (w[0] + w[1]) + (w[2] + w[3]);
+    if (mode == 3) rr[c] = (w2[0] + w2[1]) + (w2[2] + w2[3]);
     if (mode == 0) {
       rr[c] = s;
-    } else if (mode == 1) {
-      coef[c] = s > 0.0 ? rr[c] / s : 0.0;
-    } else {
+    } else if (mode == 2) {
       coef[c] = rr[c] > 0.0 ? s / rr[c] : 0.0;
       rr[c] = s;
+    } else {
+      coef[c] = s > 0.0 ? rr[c] / s : 0.0;
     }
   }
 }
 
 }  // namespace
 
+// nu CG steps.  The first direction is the residual itself (F for a zero start: no copy is made), the
+// last step forms neither its image nor the residual that nothing reads, and with the usual two steps
+// x takes both of its updates in one pass: 16 passes over vectors (12 from zero) instead of 23 (21).
+// Longer runs update x beside the directions.  Every element goes through the operations of the
+// recurrence in their order.  The scalars are a launch of their own: a last-block sum of up to 1216
+// partial rows would be a longer chain than the launch.
 template <typename T>
 void cg_smooth(const Launch& L, const DCsr& A, const T* F, T* X, bool x_zero, T* R, T* P, T* Q, const CgWork& w,
                int ldk, int nu) {
@@ -1274,39 +1349,76 @@ void cg_smooth(const Launch& L, const DCsr& A, const T* F, T* X, bool x_zero, T*
   const size_t smem = (size_t)rpb * ldk * sizeof(double);
   const double sz = sizeof(T), rows = A.n_rows, nnz = (double)A.nnz, vec = rows * ldk * sz;
   const double mat = nnz * (4.0 + sz) + (rows + 1) * 4.0;
+  const int64_t total = (int64_t)A.n_rows * ldk;
+  const int sgrid = (int)std::min<int64_t>((total / Vec16<T>::N + kBlock - 1) / kBlock, 152 * 16);
   const T* av = vals<T>(A);
+  double* partial2 = w.partial + (size_t)w.max_blocks * ldk;
   auto scalars = [&](int mode, double* coef) {
     L.begin(KC_CG, (double)grid * ldk * 8.0, (double)grid * ldk);
-    k_cg_scalar<<<ldk, 128, 0, L.s>>>(w.partial, grid, ldk, mode, w.rr, coef);
+    launch(L, k_cg_scalar, ldk, 128, 0, w.partial, partial2, grid, ldk, mode, w.rr, coef);
     L.bump();
   };
-  L.rows(A.n_rows);
-  L.begin(KC_CG, (x_zero ? 0.0 : mat + vec) + 3.0 * vec, x_zero ? 2.0 * rows * ldk : 2.0 * nnz * ldk + 3.0 * rows * ldk);
-  PASM_DISPATCH_CH(g.ch, k_cg_start<T, CH><<<grid, kBlock, smem, L.s>>>(A.n_rows, A.rp, A.ci, av, x_zero ? nullptr : X,
-                                                                         F, R, P, w.partial, ldk, g.tpr));
-  L.bump();
-  scalars(0, nullptr);
+  const T* r = F;   // the residual, and the first direction
+  if (!x_zero) {
+    L.rows(A.n_rows);
+    L.begin(KC_CG, mat + 3.0 * vec, 2.0 * nnz * ldk + 3.0 * rows * ldk);
+    PASM_DISPATCH_CH(g.ch, launch(L, k_cg_start<T, CH>, grid, kBlock, smem, A.n_rows, A.rp, A.ci, av, X, F, R, w.partial,
+                                  ldk, g.tpr));
+    L.bump();
+    scalars(0, nullptr);
+    r = R;
+  }
+  const T* p = r;
+  const T* p0 = nullptr;      // two steps: the first direction, whose update of x waits for the second
+  double* alpha[2] = {w.alpha, w.alpha2};
   for (int it = 0; it < nu; ++it) {
+    const bool last = it + 1 == nu, rr = x_zero && it == 0;
     L.rows(A.n_rows);
-    L.begin(KC_CG, mat + 2.0 * vec, 2.0 * nnz * ldk + 2.0 * rows * ldk);
-    PASM_DISPATCH_CH(g.ch, k_cg_dir<T, CH><<<grid, kBlock, smem, L.s>>>(A.n_rows, A.rp, A.ci, av, P, Q, w.partial,
-                                                                         ldk, g.tpr));
-    L.bump();
-    scalars(1, w.alpha);
-    const bool xz = x_zero && it == 0;
-    L.rows(A.n_rows);
-    L.begin(KC_CG, (xz ? 5.0 : 6.0) * vec, 6.0 * rows * ldk);
-    PASM_DISPATCH_CH(g.ch, k_cg_update<T, CH><<<grid, kBlock, smem, L.s>>>(A.n_rows, X, R, P, Q, w.alpha, w.partial,
-                                                                            ldk, g.tpr, xz ? 1 : 0));
-    L.bump();
-    if (it + 1 < nu) {
-      scalars(2, w.beta);
-      const int64_t total = (int64_t)A.n_rows * ldk;
-      L.begin(KC_CG, 3.0 * vec, 2.0 * rows * ldk);
-      k_cg_pupdate<T><<<(int)std::min<int64_t>((total + kBlock - 1) / kBlock, 152 * 16), kBlock, 0, L.s>>>(
-          total, ldk, R, P, w.beta);
-      L.bump();
+    L.begin(KC_CG, mat + (last ? 1.0 : 2.0) * vec, 2.0 * nnz * ldk + 2.0 * rows * ldk);
+#define PASM_CG_DIR(QO, RRV)                                                                                     \
+  PASM_DISPATCH_CH(g.ch, launch(L, k_cg_dir<T, CH, QO, RRV>, grid, kBlock, smem, A.n_rows, A.rp, A.ci, av, p, Q,    \
+                                w.partial, partial2, ldk, g.tpr))
+    if (last) {
+      if (rr) { PASM_CG_DIR(false, true); } else { PASM_CG_DIR(false, false); }
+    } else {
+      if (rr) { PASM_CG_DIR(true, true); } else { PASM_CG_DIR(true, false); }
     }
+#undef PASM_CG_DIR
+    L.bump();
+    scalars(rr ? 3 : 1, alpha[it & 1]);
+    if (last) {
+      const bool xz = x_zero && (it == 0 || p0);   // x has taken no update yet
+      L.rows(A.n_rows);
+      L.begin(KC_CG, ((xz ? 2.0 : 3.0) + (p0 ? 1.0 : 0.0)) * vec, 4.0 * rows * ldk);
+      if (xz) launch(L, k_cg_final<T, true>, sgrid, kBlock, 0, total, ldk, X, p0, alpha[(it + 1) & 1], p, alpha[it & 1]);
+      else launch(L, k_cg_final<T, false>, sgrid, kBlock, 0, total, ldk, X, p0, alpha[(it + 1) & 1], p, alpha[it & 1]);
+      L.bump();
+      return;
+    }
+    // the new residual: beside the first direction (kept, as F or in R), later in place
+    T* rn = it > 0 ? const_cast<T*>(r) : (r == R ? P : R);
+    L.rows(A.n_rows);
+    L.begin(KC_CG, 3.0 * vec, 4.0 * rows * ldk);
+    PASM_DISPATCH_CH(g.ch, launch(L, k_cg_resid<T, CH>, grid, kBlock, smem, A.n_rows, r, Q, rn, alpha[it & 1], w.partial,
+                                  ldk, g.tpr));
+    L.bump();
+    scalars(2, w.beta);
+    L.begin(KC_CG, (nu == 2 ? 3.0 : 5.0) * vec, 4.0 * rows * ldk);
+    T* pn;
+    if (nu == 2) {   // the residual is not needed again: the direction takes its place
+      pn = rn;
+      p0 = p;
+      launch(L, k_cg_pstep<T, 0>, sgrid, kBlock, 0, total, ldk, rn, p, pn, w.beta, nullptr, nullptr);
+    } else {
+      pn = it > 0 ? const_cast<T*>(p) : (r == R ? R : P);
+      if (x_zero && it == 0)
+        launch(L, k_cg_pstep<T, 1>, sgrid, kBlock, 0, total, ldk, rn, p, pn, w.beta, X, alpha[it & 1]);
+      else
+        launch(L, k_cg_pstep<T, 2>, sgrid, kBlock, 0, total, ldk, rn, p, pn, w.beta, X, alpha[it & 1]);
+    }
+    L.bump();
+    r = rn;
+    p = pn;
   }
 }
 template void cg_smooth<float>(const Launch&, const DCsr&, const float*, float*, bool, float*, float*, float*,

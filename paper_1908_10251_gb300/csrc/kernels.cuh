@@ -190,11 +190,11 @@ void update_pairs_identity(const Launch& L, int n, const double* W, const double
 // Conjugate-gradient smoothing (kernels.cu): nu CG steps for A x = F, every
 // column its own CG.  x_zero: start from x = 0 (X is written, not read).
 // R, P, Q are n x ldk scratch blocks; the work arrays hold per-block partial
-// sums (max_blocks x ldk) and the per-column scalars r.r, alpha, beta.
+// sums (2 x max_blocks x ldk) and the per-column scalars r.r, alpha (of two steps), beta.
 struct CgWork {
   double* partial = nullptr;
   int max_blocks = 0;
-  double *rr = nullptr, *alpha = nullptr, *beta = nullptr;
+  double *rr = nullptr, *alpha = nullptr, *alpha2 = nullptr, *beta = nullptr;
 };
 template <typename T>
 void cg_smooth(const Launch& L, const DCsr& A, const T* F, T* X, bool x_zero, T* R, T* P, T* Q, const CgWork& w,

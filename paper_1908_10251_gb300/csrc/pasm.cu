@@ -638,8 +638,8 @@ int alloc_k(pasm_ctx* c, int k) {
   AL(K, &c->nact, 1); AL(K, &c->diag, 8);
   if (c->opts.smoother == PASM_CG) {
     c->cg.max_blocks = 152 * 8;
-    AL(K, &c->cg.partial, (size_t)c->cg.max_blocks * ldk);
-    AL(K, &c->cg.rr, ldk); AL(K, &c->cg.alpha, ldk); AL(K, &c->cg.beta, ldk);
+    AL(K, &c->cg.partial, 2 * (size_t)c->cg.max_blocks * ldk);
+    AL(K, &c->cg.rr, ldk); AL(K, &c->cg.alpha, ldk); AL(K, &c->cg.alpha2, ldk); AL(K, &c->cg.beta, ldk);
   }
   if (c->proj_tc) {
     AL(K, &c->proj_hl, proj_scratch_words(c->NH, 2 * (int)ldk));
