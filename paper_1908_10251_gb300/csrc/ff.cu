@@ -471,6 +471,57 @@ __global__ void k_from_ff(int64_t total, const double* in, double* out) {
   }
 }
 
+// The caller's [n][k] block on the device -> [n][ldk], zero in the padded columns: float64 (U, may be
+// null) and pairs (may be null) in one pass.  Bound by memory: one read and one write per copy made
+// (a linear or pitched copy, a memset and a conversion took two to six passes).  The caller's rows
+// may be 8-byte aligned only.
+__global__ void __launch_bounds__(kBlock) k_put_block(int64_t n, int k, int ldk, const double* src, double* U,
+                                                      double* pairs) {
+  pdl_trigger();
+  pdl_wait();
+  const int sh = 31 - __clz(ldk / 2);   // ldk is a power of two
+  for (int64_t i = blockIdx.x * (int64_t)kBlock + threadIdx.x; i < n << sh; i += (int64_t)gridDim.x * kBlock) {
+    const int64_t row = i >> sh;
+    const int c = 2 * (int)(i & ((1 << sh) - 1));
+    const double* p = src + row * k + c;
+    const double a = c < k ? ld1(p) : 0.0, b = c + 1 < k ? ld1(p + 1) : 0.0;
+    if (U) *reinterpret_cast<double2*>(U + row * ldk + c) = make_double2(a, b);
+    if (pairs) {
+      float h0, l0, h1, l1;
+      ff_split(a, h0, l0);
+      ff_split(b, h1, l1);
+      store_pair<true>(pairs, (size_t)(row * ldk + c), ff2_pack(h0, h1), ff2_pack(l0, l1));
+    }
+  }
+}
+// The reverse: an [n][ldk] block (float64, or pairs with FF) -> the caller's [n][k] block on the device.
+template <bool FF>
+__global__ void __launch_bounds__(kBlock) k_get_block(int64_t n, int k, int ldk, const double* in, double* dst) {
+  pdl_trigger();
+  pdl_wait();
+  const int sh = 31 - __clz(ldk / 2);
+  for (int64_t i = blockIdx.x * (int64_t)kBlock + threadIdx.x; i < n << sh; i += (int64_t)gridDim.x * kBlock) {
+    const int64_t row = i >> sh;
+    const int c = 2 * (int)(i & ((1 << sh) - 1));
+    if (c >= k) continue;
+    double v[2];
+    if (FF) {
+      ff2 h, l;
+      load_pair<true>(in, (size_t)(row * ldk + c), h, l);
+      float h0, h1, l0, l1;
+      ff2_unpack(h, h0, h1);
+      ff2_unpack(l, l0, l1);
+      v[0] = ff_to_double(h0, l0);
+      v[1] = ff_to_double(h1, l1);
+    } else {
+      ldg16<double>(in + row * ldk + c, v);
+    }
+    double* p = dst + row * k + c;
+    p[0] = v[0];
+    if (c + 1 < k) p[1] = v[1];
+  }
+}
+
 // U[row][c] = upd[c] ? alpha[c] X[row][c] + (P W)[row][c] : U[row][c], X as
 // float pairs, W as float pairs (WFF) or float64; identity: P W = W.  Entries
 // of frozen pairs are neither read nor written.  With U null the state is the
@@ -683,6 +734,19 @@ void to_ff(const Launch& L, int64_t total, const double* in, double* out) {
 void from_ff(const Launch& L, int64_t total, const double* in, double* out) {
   L.begin(KC_CAST, (double)total * 16.0, (double)total);
   launch(L, k_from_ff, stream_grid(total), kBlock, 0, total, in, out);
+  L.bump();
+}
+
+void put_block_dev(const Launch& L, int64_t n, int k, int ldk, const double* src, double* U, double* pairs) {
+  L.begin(KC_CAST, (double)n * (k + ldk * ((U ? 1 : 0) + (pairs ? 1 : 0))) * 8.0, 0.0);
+  launch(L, k_put_block, stream_grid(n * ldk), kBlock, 0, n, k, ldk, src, U, pairs);
+  L.bump();
+}
+
+void get_block_dev(const Launch& L, int64_t n, int k, int ldk, const double* in, bool ff, double* dst) {
+  L.begin(KC_CAST, (double)n * (k + ldk) * 8.0, 0.0);
+  if (ff) launch(L, k_get_block<true>, stream_grid(n * ldk), kBlock, 0, n, k, ldk, in, dst);
+  else launch(L, k_get_block<false>, stream_grid(n * ldk), kBlock, 0, n, k, ldk, in, dst);
   L.bump();
 }
 

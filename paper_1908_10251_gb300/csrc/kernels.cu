@@ -982,6 +982,24 @@ void count_active(const Launch& L, const int* active, int k, int* out) {
   L.bump();
 }
 
+__global__ void k_set_pairs(int k, int ldk, int* active, int* steps, int* status, double* lam) {
+  pdl_trigger();
+  pdl_wait();
+  const int c = threadIdx.x;
+  if (c >= ldk) return;
+  if (active) {
+    active[c] = c < k ? 1 : 0;
+    steps[c] = 0;
+    status[c] = 0;
+  }
+  if (lam && c >= k) lam[c] = 1.0;
+}
+void set_pairs(const Launch& L, int k, int ldk, int* active, int* steps, int* status, double* lam) {
+  L.begin(KC_INIT, ldk * 12.0, 0.0);
+  launch(L, k_set_pairs, 1, ldk, 0, k, ldk, active, steps, status, lam);
+  L.bump();
+}
+
 __global__ void k_cast_d2f(const double* in, float* out, int64_t count) {
   pdl_trigger();
   pdl_wait();

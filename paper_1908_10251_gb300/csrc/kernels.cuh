@@ -226,6 +226,10 @@ void axpy_ff(const Launch& L, int n, const double* B, bool b_ff, const float* E,
 // Conversions of total entries: float64 -> pairs (may be in place), pairs -> float64.
 void to_ff(const Launch& L, int64_t total, const double* in, double* out);
 void from_ff(const Launch& L, int64_t total, const double* in, double* out);
+// Device copies of a block: the caller's [n][k] array -> [n][ldk] as float64 (U) and / or pairs, padded
+// columns zero; and back from float64 or pairs (ff).
+void put_block_dev(const Launch& L, int64_t n, int k, int ldk, const double* src, double* U, double* pairs);
+void get_block_dev(const Launch& L, int64_t n, int k, int ldk, const double* in, bool ff, double* dst);
 // U = alpha X + P W for updated pairs (X in pairs, W in pairs if w_ff); P ==
 // nullptr means P = identity on n rows.  With U given, U is float64 and Usplit
 // (optional) receives it as pairs; with U null the result goes to Usplit alone
@@ -268,6 +272,10 @@ cudaError_t proj_tc_prepare();
 void proj_tc(const Launch& L, const SplitMat& A, const double* B0, const double* B1, double* C0, double* C1,
              int ldk, int ncols, unsigned long long* hl, unsigned int* tickets, int* err, int wait_limit = 0,
              int skip_mma = 0);
+
+// A fresh set of k pairs: active[c] = c < k, steps = status = 0 for all ldk columns; lam (may be
+// null): 1 in the padded columns.
+void set_pairs(const Launch& L, int k, int ldk, int* active, int* steps, int* status, double* lam);
 
 // *out = number of nonzero entries of active[0..k)
 void count_active(const Launch& L, const int* active, int k, int* out);

@@ -441,24 +441,25 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
 
 // Algorithm 1 step 1 on level lt: X = result of the V-cycles for A x = lam M U from x = U,
 // each cycle a defect correction x += V(f - A x) with f = lam M U (float64 residual).
+// Mixed precision reads U from the pair array `pairs`; U given: it is formed from U first.
 template <typename T>
-void bvp_impl(pasm_ctx* c, int lt, const double* lam, const double* U, double* X, bool u_split) {
+void bvp_impl(pasm_ctx* c, int lt, const double* lam, const double* U, double* X, double* pairs) {
   const Launch L = launcher(c);
   LevelDev& v = c->lv[lt];
   T* Ftop = (T*)v.vF;
   if (Fused<T>::on) {
     // double-float outer residuals; X (the result u~) is left in (hi, lo) pairs
-    if (!u_split) to_ff(L, (int64_t)v.n * c->ldk, U, c->Uff);
-    outer_rhs_residual_ff(launcher(c, lt, PASM_TILE_OUTER_RHS), v.A, v.M, lam, c->Uff, c->Fd, (float*)Ftop, c->ldk);
+    if (U) to_ff(L, (int64_t)v.n * c->ldk, U, pairs);
+    outer_rhs_residual_ff(launcher(c, lt, PASM_TILE_OUTER_RHS), v.A, v.M, lam, pairs, c->Fd, (float*)Ftop, c->ldk);
     if (c->opts.res_tol > 0.0 && lt == c->nlev - 1) {  // the starting state's residual, for the freeze test
-      const int nb = residual_partials<float>(L, v.n, c->ldk, (const float*)Ftop, true, c->Fd, c->Uff, c->partials,
+      const int nb = residual_partials<float>(L, v.n, c->ldk, (const float*)Ftop, true, c->Fd, pairs, c->partials,
                                               c->max_border_blocks);
       column_sums(L, c->partials, nb, 2, c->ldk, c->rsum);
     }
     // x = u + e reads u from its pair copy (in a step the state lives there alone)
-    const TopOut first{c->Uff, true, X};
+    const TopOut first{pairs, true, X};
     T* e = vcycle<T>(c, lt, lt >= 1 ? &first : nullptr);
-    if (e) axpy_ff(L, v.n, c->Uff, true, (const float*)e, X, c->ldk);
+    if (e) axpy_ff(L, v.n, pairs, true, (const float*)e, X, c->ldk);
     for (int cyc = 1; cyc < c->opts.cycles_per_step; ++cyc) {
       outer_residual_ff(launcher(c, lt, PASM_TILE_OUTER_RES), v.A, c->Fd, X, (float*)Ftop, c->ldk);
       const TopOut next{X, true, X};
@@ -481,11 +482,12 @@ void bvp_impl(pasm_ctx* c, int lt, const double* lam, const double* U, double* X
   }
 }
 
-// u_split: c->Uff already holds U in pairs (the state U of a step: the update of
-// the previous step, or pasm_init, wrote it); otherwise it is formed here.
-void bvp(pasm_ctx* c, int lt, const double* lam, const double* U, double* X, bool u_split = false) {
-  if (c->opts.precision == PASM_MIXED) bvp_impl<float>(c, lt, lam, U, X, u_split);
-  else bvp_impl<double>(c, lt, lam, U, X, u_split);
+// U: the block in float64.  In mixed precision its pair form goes to `pairs` (null: c->Uff) and is
+// read from there; U null: `pairs` holds it already (the state of a step, which the previous step's
+// update or pasm_init wrote, is in c->Uff).
+void bvp(pasm_ctx* c, int lt, const double* lam, const double* U, double* X, double* pairs = nullptr) {
+  if (c->opts.precision == PASM_MIXED) bvp_impl<float>(c, lt, lam, U, X, pairs ? pairs : c->Uff);
+  else bvp_impl<double>(c, lt, lam, U, X, nullptr);
 }
 
 struct PairState {
@@ -575,7 +577,7 @@ void augmented(pasm_ctx* c, int lt, const double* X, const PairState& ps) {
 // One correction step for all active pairs on the finest level.
 void step_body(pasm_ctx* c) {
   const int lt = c->nlev - 1;
-  bvp(c, lt, c->lam, c->U, c->X, true);
+  bvp(c, lt, c->lam, c->opts.precision == PASM_MIXED ? nullptr : c->U, c->X);
   PairState ps{c->lam, c->active, c->steps, c->status, c->U, c->tol};
   augmented(c, lt, c->X, ps);
   count_active(launcher(c), c->active, c->k, c->nact);
@@ -652,27 +654,37 @@ int alloc_k(pasm_ctx* c, int k) {
     CK(cudaMemsetAsync(c->proj_tickets, 0, sizeof(unsigned int) * tickets, c->s));
   }
   for (double* z : {c->bq, c->cq, c->g, c->uH}) CK(cudaMemsetAsync(z, 0, sizeof(double) * nh, c->s));
-  CK(cudaMemsetAsync(c->U, 0, sizeof(double) * n * ldk, c->s));
-  CK(cudaMemsetAsync(c->X, 0, sizeof(double) * n * ldk, c->s));
+  if (!reuse) {   // later starts overwrite U, and every step X
+    CK(cudaMemsetAsync(c->U, 0, sizeof(double) * n * ldk, c->s));
+    CK(cudaMemsetAsync(c->X, 0, sizeof(double) * n * ldk, c->s));
+  }
   CK(cudaMemsetAsync(c->diag, 0, sizeof(int) * 8, c->s));
   return PASM_OK;
 }
 
 int set_active(pasm_ctx* c, int* active, int* steps, int* status) {
-  std::vector<int> h((size_t)c->ldk, 0);
-  for (int i = 0; i < c->k; ++i) h[(size_t)i] = 1;
-  CK(cudaMemcpyAsync(active, h.data(), sizeof(int) * c->ldk, cudaMemcpyHostToDevice, c->s));
-  CK(cudaMemsetAsync(steps, 0, sizeof(int) * c->ldk, c->s));
-  CK(cudaMemsetAsync(status, 0, sizeof(int) * c->ldk, c->s));
-  CK(cudaStreamSynchronize(c->s));
+  set_pairs(launcher(c), c->k, c->ldk, active, steps, status, nullptr);
   return PASM_OK;
 }
 
-// Copy an n x k user block (host or device, leading dim k) into an n x ldk device block.
-// Block copies between the caller's [n][k] array and the [n][ldk] device block.
-// When k == ldk the rows are contiguous on both sides and one linear copy moves
-// the block (a pitched copy of n short rows runs far below the link's rate).
+bool on_device(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  int dev = 0;
+  return a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && a.device == dev;
+}
+
+// Block copies between the caller's [n][k] array and the [n][ldk] device block: a kernel for memory of
+// this device; else, when k == ldk, one linear copy (the rows are contiguous on both sides; a pitched
+// copy of n short rows runs far below the link's rate).
 int put_block(pasm_ctx* c, const double* src, double* dst, int n) {
+  if (on_device(src)) {
+    put_block_dev(launcher(c), n, c->k, c->ldk, src, dst, nullptr);
+    return PASM_OK;
+  }
   if (c->k == c->ldk) {
     CK(cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)n * c->k, cudaMemcpyDefault, c->s));
     return PASM_OK;
@@ -683,6 +695,10 @@ int put_block(pasm_ctx* c, const double* src, double* dst, int n) {
   return PASM_OK;
 }
 int get_block(pasm_ctx* c, const double* src, double* dst, int n) {
+  if (on_device(dst)) {
+    get_block_dev(launcher(c), n, c->k, c->ldk, src, false, dst);
+    return PASM_OK;
+  }
   if (c->k == c->ldk) {
     CK(cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)n * c->k, cudaMemcpyDefault, c->s));
     return PASM_OK;
@@ -691,11 +707,10 @@ int get_block(pasm_ctx* c, const double* src, double* dst, int n) {
                        cudaMemcpyDefault, c->s));
   return PASM_OK;
 }
+// (the callers synchronise before they return: a source in host memory stays valid until then)
 int put_lambda(pasm_ctx* c, const double* src, double* dst) {
-  std::vector<double> ones((size_t)c->ldk, 1.0);
-  CK(cudaMemcpyAsync(dst, ones.data(), sizeof(double) * c->ldk, cudaMemcpyHostToDevice, c->s));
+  set_pairs(launcher(c), c->k, c->ldk, nullptr, nullptr, nullptr, dst);
   CK(cudaMemcpyAsync(dst, src, sizeof(double) * c->k, cudaMemcpyDefault, c->s));
-  CK(cudaStreamSynchronize(c->s));
   return PASM_OK;
 }
 
@@ -1140,9 +1155,15 @@ int pasm_init(pasm_ctx* c, int k, double tol, const double* lambda0, const doubl
   c->tol = tol;
   const int nf = c->lv.back().n;
   const Launch L = launcher(c);
+  bool paired = false;
   if (lambda0) {
     r = put_lambda(c, lambda0, c->lam);
-    if (!r) r = put_block(c, U0, c->U, nf);
+    if (!r && c->opts.precision == PASM_MIXED && on_device(U0)) {
+      put_block_dev(L, nf, k, c->ldk, U0, c->U, c->Uff);
+      paired = true;
+    } else if (!r) {
+      r = put_block(c, U0, c->U, nf);
+    }
     if (r) return r;
   } else if (c->opts.init == PASM_INIT_NESTED && c->nlev >= 3) {
     // Algorithm 2 with h_1 = H: pairs on V_H, then one correction step on every
@@ -1183,7 +1204,7 @@ int pasm_init(pasm_ctx* c, int k, double tol, const double* lambda0, const doubl
     CK(cudaMemsetAsync(c->nn.accepted, 0, sizeof(int) * 256, c->s));
   }
   // the pair copy of the state U that the first step's gathers read (later steps: the update)
-  if (c->opts.precision == PASM_MIXED) to_ff(L, (int64_t)nf * c->ldk, c->U, c->Uff);
+  if (c->opts.precision == PASM_MIXED && !paired) to_ff(L, (int64_t)nf * c->ldk, c->U, c->Uff);
   c->u_stale = false;
   CK(cudaMemsetAsync(c->diag, 0, sizeof(int) * 8, c->s));  // secular counters count the steps only
   CK(cudaGetLastError());
@@ -1251,7 +1272,9 @@ int pasm_get(pasm_ctx* c, double* lambda, double* U, int* steps, int* status) {
   if (!c || !c->initialized) return PASM_ESTATE;
   Scope sc(c);
   if (lambda) CK(cudaMemcpyAsync(lambda, c->lam, sizeof(double) * c->k, cudaMemcpyDefault, c->s));
-  if (U) {
+  if (U && c->u_stale && on_device(U)) {   // straight from the pairs
+    get_block_dev(launcher(c), c->lv.back().n, c->k, c->ldk, c->Uff, true, U);
+  } else if (U) {
     sync_state(c);
     int r = get_block(c, c->U, U, c->lv.back().n);
     if (r) return r;
@@ -1316,21 +1339,30 @@ int pasm_solve(pasm_ctx* c, int k, double tol, const double* lambda0, const doub
 int pasm_bvp(pasm_ctx* c, const double* lambda, const double* U, double* Uhat) {
   if (!c || !c->initialized || !lambda || !U || !Uhat) return PASM_ESTATE;
   Scope sc(c);
-  sync_state(c);  // the pair copy is rebuilt from U below
   const int nf = c->lv.back().n;
   int r = put_lambda(c, lambda, c->lam2);
-  if (!r) r = put_block(c, U, c->YM, nf);
   if (r) return r;
-  bvp(c, c->nlev - 1, c->lam2, c->YM, c->X);
-  CK(cudaGetLastError());
-  const double* xout = c->X;
-  if (c->opts.precision == PASM_MIXED) {  // u~ comes back in (hi, lo) pairs
-    from_ff(launcher(c), (int64_t)nf * c->ldk, c->X, c->YA);
-    xout = c->YA;
-    to_ff(launcher(c), (int64_t)nf * c->ldk, c->U, c->Uff);  // the step's pair copy of the state U again
+  if (c->opts.precision == PASM_MIXED) {
+    // in pairs throughout, beside the state: u in YM, u~ in X
+    const bool dev = on_device(U);
+    if (dev) put_block_dev(launcher(c), nf, c->k, c->ldk, U, nullptr, c->YM);
+    else r = put_block(c, U, c->YA, nf);
+    if (r) return r;
+    bvp(c, c->nlev - 1, c->lam2, dev ? nullptr : c->YA, c->X, c->YM);
+    if (on_device(Uhat)) {
+      get_block_dev(launcher(c), nf, c->k, c->ldk, c->X, true, Uhat);
+    } else {
+      from_ff(launcher(c), (int64_t)nf * c->ldk, c->X, c->YA);
+      r = get_block(c, c->YA, Uhat, nf);
+    }
+  } else {
+    r = put_block(c, U, c->YM, nf);
+    if (r) return r;
+    bvp(c, c->nlev - 1, c->lam2, c->YM, c->X);
+    r = get_block(c, c->X, Uhat, nf);
   }
-  r = get_block(c, xout, Uhat, nf);
   if (r) return r;
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(c->s));
   return PASM_OK;
 }
@@ -1704,8 +1736,7 @@ int pasm_nn_capture_residuals(pasm_ctx* c, int level, float* R_out) {
   if (r) return r;
   c->capture_level = level;
   c->capture_buf = c->nn.Rt;
-  sync_state(c);                               // the pair copy is rebuilt from U here
-  bvp(c, c->nlev - 1, c->lam, c->U, c->YA);   // scratch output; the pair state is not touched
+  bvp(c, c->nlev - 1, c->lam, nullptr, c->YA);   // the state's pairs; scratch output: the state is not touched
   c->capture_level = -1;
   c->capture_buf = nullptr;
   CK(cudaMemcpy2DAsync(R_out, sizeof(float) * c->k, c->nn.Rt, sizeof(float) * c->ldk, sizeof(float) * c->k, n,
