@@ -1627,6 +1627,10 @@ int pasm_nn_get_weights(pasm_ctx* c, float* weights) {
 
 // copy a user n x k float block into an n x ldk2 device block (zero padding)
 static int put_block_f(pasm_ctx* c, const float* src, float* dst, int n, int k, int ldk2) {
+  if (k == ldk2) {
+    CK(cudaMemcpyAsync(dst, src, sizeof(float) * (size_t)n * k, cudaMemcpyDefault, c->s));
+    return PASM_OK;
+  }
   CK(cudaMemsetAsync(dst, 0, sizeof(float) * (size_t)n * ldk2, c->s));
   CK(cudaMemcpy2DAsync(dst, sizeof(float) * ldk2, src, sizeof(float) * k, sizeof(float) * k, n, cudaMemcpyDefault,
                        c->s));
@@ -1649,9 +1653,16 @@ int pasm_nn_apply(pasm_ctx* c, int level, int k, const float* R, float* D) {
   r = nn_ensure(c, tc ? 0 : (int64_t)n * ldk2, (int64_t)n * ldk2, false);
   if (r) return r;
   auto& nn = c->nn;
+  NNGrid g{nn.nx[(size_t)level], nn.ny[(size_t)level], ldk2, k};
+  // blocks of this device without padded columns are read and written in place (16-byte loads)
+  if (tc && k == ldk2 && R != D && ((uintptr_t)R % 16) == 0 && on_device(R) && on_device(D)) {
+    nn_forward_tc(launcher(c), g, &nn.w13, nullptr, nn.w2, R, D, nn.err);
+    CK(cudaGetLastError());
+    CK(cudaStreamSynchronize(c->s));
+    return PASM_OK;
+  }
   r = put_block_f(c, R, nn.R, n, k, ldk2);
   if (r) return r;
-  NNGrid g{nn.nx[(size_t)level], nn.ny[(size_t)level], ldk2, k};
   if (tc)
     nn_forward_tc(launcher(c), g, &nn.w13, nullptr, nn.w2, nn.R, nn.D, nn.err);
   else

@@ -10,7 +10,7 @@
 //            an implicit GEMM over the 9 taps: M = 128 rows = 16 pixels x 8
 //            pairs, N = 16 output channels, K = 16 input channels per tap; the
 //            tap shift is a shift of the operand's start address;
-//   epilogue: tcgen05.ld of the accumulators, h = (relu(z2+) - relu(z2-)) / 2
+//   epilogue: tcgen05.ld of the accumulators, 2 h = relu(z2+) - relu(z2-)
 //            (float32, shared memory, reusing the a1 space, as [row][col][channel
 //            quad][pair][4] so that the 16-byte reads of layer 3 by consecutive
 //            pairs hit consecutive banks);
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   float* rs = reinterpret_cast<float*>(smem + kA1Bytes);        // [RR][RW][PB]
   uint8_t* w2 = smem + kA1Bytes + kRBytes;                      // 9 x [2 n-groups][2 k-chunks][8][8] bf16
   float* sw1 = reinterpret_cast<float*>(w2 + kW2Bytes);         // [tap][16]
-  float* sw3 = sw1 + 144;                                       // [tap][16]
+  float* sw3 = sw1 + 144;                                       // [tap][16], halved (2 h is stored)
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sw3 + 144);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
 
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(w2 + 16 * t)), "l"(w2g + 16 * t));
   if (tid < 144) {
     if (DEV) sw1[tid] = __ldg(Wd + tid);
-    sw3[tid] = DEV ? __ldg(Wd + 144 + 2304 + tid) : w13.w3[tid];
+    sw3[tid] = 0.5f * (DEV ? __ldg(Wd + 144 + 2304 + tid) : w13.w3[tid]);
   }
   // residual tile with a 3-pixel halo (zero outside the grid and for padded pairs).  A block of 8
   // real pairs is one 32-byte segment per pixel: two 16-byte asynchronous copies (cp.async, all in
@@ -172,14 +172,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
       }
     }
     const int pix = (row * AW + col) * PB + q;  // 16-byte row index inside a plane
+    // relu(+-z) in bf16: rounding is odd and monotone, so z is rounded once per pair of channels and
+    // the two branches are a packed maximum each (a NaN gives 0, as fmaxf does)
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
-      __align__(16) __nv_bfloat162 vp[4], vm[4];  // two channels per conversion
+      __align__(16) __nv_bfloat162 vp[4], vm[4];
 #pragma unroll
       for (int o = 0; o < 4; ++o) {
-        const float za = z[half * 8 + 2 * o], zb = z[half * 8 + 2 * o + 1];
-        vp[o] = __floats2bfloat162_rn(fmaxf(za, 0.f), fmaxf(zb, 0.f));
-        vm[o] = __floats2bfloat162_rn(fmaxf(-za, 0.f), fmaxf(-zb, 0.f));
+        const __nv_bfloat162 b = __floats2bfloat162_rn(z[half * 8 + 2 * o], z[half * 8 + 2 * o + 1]);
+        const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+        vp[o] = __hmax2(b, zero);
+        vm[o] = __hmax2(__hneg2(b), zero);
       }
       *reinterpret_cast<uint4*>(a1 + (0 * 2 + half) * kPlane + pix * 16) = *reinterpret_cast<uint4*>(vp);
       *reinterpret_cast<uint4*>(a1 + (1 * 2 + half) * kPlane + pix * 16) = *reinterpret_cast<uint4*>(vm);
@@ -212,14 +215,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
       }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar)));
   }
+  // one thread polls, the others wait at the barrier (512 polling threads took issue slots from the
+  // other CTA of the SM)
   uint32_t done = 0;
-  for (int it = 0; it < kWaitLimit && !done; ++it) {
-    asm volatile(
-        "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\nselp.u32 %0, 1, 0, q;\n}\n"
-        : "=r"(done)
-        : "r"(smem_u32(mbar)));
+  if (tid == 0) {
+    for (int it = 0; it < kWaitLimit && !done; ++it) {
+      asm volatile(
+          "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], 0;\nselp.u32 %0, 1, 0, q;\n}\n"
+          : "=r"(done)
+          : "r"(smem_u32(mbar)));
+    }
+    if (!done) atomicAdd(err, 1);
   }
-  if (!done && tid == 0) atomicAdd(err, 1);
+  done = (uint32_t)__syncthreads_or((int)done);
   asm volatile("tcgen05.fence::after_thread_sync;");
   if (done) {
     // epilogue: TMEM lane m = 32 * (warp % 4) + lane = (h pixel j, pair q) with m = j * PB + q;
@@ -236,13 +244,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
       const int x = x0 - 1 + j, y = y0 - 1 + i;
       const bool in = x >= 0 && x < nx && y >= 0 && y < ny;
       float* dst = hs + (i * HW + j) * 16 * PB + q * 4;
+      if (!in) {
+#pragma unroll
+        for (int o = 0; o < 16; ++o) vp[o] = vm[o] = 0.f;
+      }
+      // 2 h: layer 3 takes half its weights (exact)
 #pragma unroll
       for (int o = 0; o < 16; o += 4) {
         float4 h4;
-        h4.x = in ? 0.5f * (fmaxf(vp[o], 0.f) - fmaxf(vm[o], 0.f)) : 0.f;
-        h4.y = in ? 0.5f * (fmaxf(vp[o + 1], 0.f) - fmaxf(vm[o + 1], 0.f)) : 0.f;
-        h4.z = in ? 0.5f * (fmaxf(vp[o + 2], 0.f) - fmaxf(vm[o + 2], 0.f)) : 0.f;
-        h4.w = in ? 0.5f * (fmaxf(vp[o + 3], 0.f) - fmaxf(vm[o + 3], 0.f)) : 0.f;
+        h4.x = fmaxf(vp[o], 0.f) - fmaxf(vm[o], 0.f);
+        h4.y = fmaxf(vp[o + 1], 0.f) - fmaxf(vm[o + 1], 0.f);
+        h4.z = fmaxf(vp[o + 2], 0.f) - fmaxf(vm[o + 2], 0.f);
+        h4.w = fmaxf(vp[o + 3], 0.f) - fmaxf(vm[o + 3], 0.f);
         *reinterpret_cast<float4*>(dst + (o / 4) * PB * 4) = h4;
       }
     }

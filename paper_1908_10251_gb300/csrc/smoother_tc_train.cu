@@ -110,6 +110,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity) {
   return done != 0;
 }
 
+// The same for the whole CTA: one thread polls, the others wait at the barrier.
+__device__ __forceinline__ bool cta_wait(uint64_t* mbar, uint32_t parity) {
+  return __syncthreads_or(threadIdx.x == 0 && mbar_wait(mbar, parity)) != 0;
+}
+
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
@@ -267,10 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int half = 0; half < 2; ++half) {
         __align__(16) __nv_bfloat162 vp[4], vm[4];
 #pragma unroll
-        for (int o = 0; o < 4; ++o) {
-          const float za = z[half * 8 + 2 * o], zb = z[half * 8 + 2 * o + 1];
-          vp[o] = __floats2bfloat162_rn(fmaxf(za, 0.f), fmaxf(zb, 0.f));
-          vm[o] = __floats2bfloat162_rn(fmaxf(-za, 0.f), fmaxf(-zb, 0.f));
+        for (int o = 0; o < 4; ++o) {   // relu(+-z) of the rounded z, as in the inference kernel
+          const __nv_bfloat162 b = __floats2bfloat162_rn(z[half * 8 + 2 * o], z[half * 8 + 2 * o + 1]);
+          const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+          vp[o] = __hmax2(b, zero);
+          vm[o] = __hmax2(__hneg2(b), zero);
         }
         uint8_t* dst = sa + pix * kPix + half * 128 + q * 16;
         *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<uint4*>(vp);
@@ -316,7 +322,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-    ok = mbar_wait(mbar, phase);
+    ok = cta_wait(mbar, phase);
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
 #pragma unroll
@@ -393,8 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mma_commit(mbar + 2);
     }
     tap_sums<-1>(sf, sd, AW, 2, wc, wq, wg, acc3);
-    __syncthreads();   // h is read: gz1 takes its place
-    ok = mbar_wait(mbar + 1, phase);
+    ok = cta_wait(mbar + 1, phase);   // its barrier: h is read, gz1 takes its place
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
       for (int i = rowgrp; i < TR; i += 4) {
@@ -429,9 +434,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     ok = __syncthreads_and(ok);
     tap_sums<1>(sf, sr, RW, 3, wc, wq, wg, acc1);
     // the next tile overwrites the operands
-    const bool fin = mbar_wait(mbar + 2, phase);
+    ok = cta_wait(mbar + 2, phase) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;");
-    ok = __syncthreads_and(ok && fin);
   }
   if (!ok && tid == 0) {
     atomicAdd(err, 1);
