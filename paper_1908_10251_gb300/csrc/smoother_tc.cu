@@ -15,8 +15,10 @@
 //            quad][pair][4] so that the 16-byte reads of layer 3 by consecutive
 //            pairs hit consecutive banks);
 //   layer 3 (16 -> 1, CUDA cores, float32): d on the 14 x 6 tile.
-// One elected thread issues the MMAs and commits them to an mbarrier; the
-// wait is bounded and reports through an error counter instead of hanging.
+// One thread of every warp issues the 9 MMAs of one row and branch and commits them to
+// an mbarrier (an MMA this small costs its issuing thread about 90 cycles, several
+// times what the tensor core takes: 144 from one thread were the longest phase of a
+// tile: inference at h = 1/512, k = 64 1.09 -> 0.94 ms); the wait is bounded and reports through an error counter instead of hanging.
 #include "common.cuh"
 #include "smoother.cuh"
 
@@ -50,6 +52,8 @@ static_assert(kHBytes <= kA1Bytes, "h must fit in the a1 space");
 static_assert(HW * PB == 128, "one MMA block per h row");
 constexpr uint32_t kTmemCols = HR * 2 * 16;        // h rows x 2 branches x 16 columns
 static_assert(kTmemCols == 256 && kSmem * kCtasPerSm <= 227 * 1024, "two CTAs per SM");
+constexpr int kIssuers = HR * 2;                   // MMA-issuing threads: one per h row and branch
+static_assert(kIssuers == kThreads / 32, "one issuer per warp");
 constexpr int kWaitLimit = 1 << 22;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -108,7 +112,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   const int tx = blockIdx.x % tiles_x, ty = blockIdx.x / tiles_x;
   const int x0 = tx * TW, y0 = ty * TR, c0 = blockIdx.y * PB;
 
-  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)));
+  if (tid == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(kIssuers));
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(kTmemCols));
@@ -194,25 +198,22 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_nn_tc(int nx, int ny, 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
-  // layer 2: 16 h rows x 2 branches x 9 taps, issued by one thread
-  if (tid == 0) {
+  // layer 2: 8 h rows x 2 branches, one per warp: lane 0 issues its 9 taps and commits them
+  if (lane == 0) {
     // kind::f16, D f32, A and B bf16, both K-major, N = 16, M = 128
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(16 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     // The descriptors are formed once: the start-address field holds (address >> 4) in 14 bits, and
     // every operand here lies below 2^18 bytes, so shifting an operand by `off` bytes adds off >> 4.
-    const uint64_t a0 = smem_desc(smem_u32(a1), kPlane, PB * 16);
+    const int i = warp >> 1, b = warp & 1;
+    const uint32_t dcol = tmem + (uint32_t)((i * 2 + b) * 16);
+    const uint64_t ai = smem_desc(smem_u32(a1) + (uint32_t)(b * 2 * kPlane + i * AW * PB * 16), kPlane, PB * 16);
     const uint64_t b0 = smem_desc(smem_u32(w2), 128, 256);
-    for (int i = 0; i < HR; ++i)
-      for (int b = 0; b < 2; ++b) {
-        const uint32_t dcol = tmem + (uint32_t)((i * 2 + b) * 16);
-        const uint64_t ai = a0 + (uint64_t)((b * 2 * kPlane + i * AW * PB * 16) >> 4);
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-          const int dy = tap / 3, dx = tap % 3;  // a1 row i + dy, col j + dx for h pixel (i, j)
-          mma_bf16(dcol, ai + (uint64_t)(((dy * AW + dx) * PB * 16) >> 4), b0 + (uint64_t)(tap * 512 >> 4), idesc,
-                   tap > 0 ? 1u : 0u);
-        }
-      }
+    for (int tap = 0; tap < 9; ++tap) {
+      const int dy = tap / 3, dx = tap % 3;  // a1 row i + dy, col j + dx for h pixel (i, j)
+      mma_bf16(dcol, ai + (uint64_t)(((dy * AW + dx) * PB * 16) >> 4), b0 + (uint64_t)(tap * 512 >> 4), idesc,
+               tap > 0 ? 1u : 0u);
+    }
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(mbar)));
   }
   // one thread polls, the others wait at the barrier (512 polling threads took issue slots from the

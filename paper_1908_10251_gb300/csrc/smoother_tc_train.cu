@@ -21,12 +21,15 @@
 // and since groups 128 B apart run on into the next pixel, the 128 M rows are the 16 channels of 8
 // consecutive pixels: rows 0..47 are the taps dx = 0, 1, 2 of one dy (the others are not used).
 // So a K step (two pixels) takes 6 MMAs (3 dy x 2 branches) instead of one per tap and branch.
+// An MMA this small costs its issuing thread about 90 cycles, several times what the tensor core
+// takes, so one thread of every warp issues: a row and branch each of the convolutions, one dy and
+// quarter of the K steps each of the weight gradient.
 //
 // What bounds it: the phases of a tile are serial (one CTA fills the SM's shared memory), the
 // tensor pipe and the float32 pipe taking turns.  Before it, the backward pass went through HBM
 // with 13 launches and about 20 passes over [pixel][pair][16] float32 activations, and layers 1 and
 // 3 summed their weight gradients with 9 and 144 threads a block.  Loss and gradient at h = 1/256,
-// k = 64 (all kernels): 9.91 ms before, 1.44 ms with this kernel and the fused forward.
+// k = 64 (all kernels): 9.91 ms before, 1.32 ms with this kernel and the fused forward.
 //
 // Every mbarrier wait is bounded; a wait that gives up increments an error counter, the kernel
 // stops walking tiles, contributes zeros and frees its TMEM.
@@ -64,8 +67,12 @@ static_assert(kSmem <= 227 * 1024, "one CTA per SM");
 static_assert(HW * PB == 128, "one MMA block per row");
 // the weight gradient's M rows reach 7 pixels past the last K pixel of the last tap row
 static_assert((TR + 2) * AW + TW + 7 < AR * AW, "M rows of the weight gradient stay inside the operand");
-constexpr uint32_t kTmemCols = 512;                 // 256 of z2 / ga, 48 of gW2
+constexpr uint32_t kTmemCols = 512;                 // 256 of z2 / ga, 192 of gW2
 constexpr uint32_t kTmemW = HR * 2 * 16;            // first column of gW2
+constexpr int kGradIssuers = TR * 2;                // MMA-issuing threads after z2: one per row and branch
+constexpr int kGradParts = kGradIssuers / 3;        // gW2: 3 dy x kGradParts accumulators
+static_assert(kGradIssuers % 3 == 0 && kTmemW + kGradIssuers * 16 <= kTmemCols, "accumulators of gW2");
+static_assert(HR * 2 == kThreads / 32, "one issuer of z2 per warp");
 static_assert(kThreads * 9 * 4 <= kABytes, "the final reduction reuses the operand space");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -209,7 +216,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    for (int b = 0; b < 3; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + b)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(HR * 2));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + 1)), "r"(kGradIssuers));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar + 2)), "r"(kGradIssuers));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);
@@ -287,17 +296,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (tid == 0) {
-      const uint64_t a0 = smem_desc(smem_u32(sa), 128, kPix);
+    if (lane == 0) {   // one row and branch per warp
+      const int i = warp >> 1, b = warp & 1;
+      const uint64_t ai = smem_desc(smem_u32(sa) + (uint32_t)(b * kABranch + i * AW * kPix), 128, kPix);
       const uint64_t b0 = smem_desc(smem_u32(sw2f), 128, 256);
-      for (int i = 0; i < HR; ++i)
-        for (int b = 0; b < 2; ++b) {
-          const uint64_t ai = a0 + (uint64_t)((b * kABranch + i * AW * kPix) >> 4);
 #pragma unroll
-          for (int tap = 0; tap < 9; ++tap)
-            mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), ai + (uint64_t)(((tap / 3 * AW + tap % 3) * kPix) >> 4),
-                     b0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
-        }
+      for (int tap = 0; tap < 9; ++tap)
+        mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), ai + (uint64_t)(((tap / 3 * AW + tap % 3) * kPix) >> 4),
+                 b0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
       mma_commit(mbar);
     }
     pending = 1;
@@ -369,33 +375,30 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (!ok) break;
     pending = 6;
-    if (tid == 0) {
-      // input gradients ga+- of the tile's rows (outputs 14, 15 of a row are not used)
-      const uint64_t g0 = smem_desc(smem_u32(sg), 128, kPix);
+    if (lane == 0 && warp < kGradIssuers) {
+      // input gradients ga+- of one row and branch (outputs 14, 15 of a row are not used)
+      const int i = warp >> 1, b = warp & 1;
+      const uint64_t gi = smem_desc(smem_u32(sg) + (uint32_t)(b * kGBranch + i * HW * kPix), 128, kPix);
       const uint64_t t0 = smem_desc(smem_u32(sw2t), 128, 256);
-      for (int i = 0; i < TR; ++i)
-        for (int b = 0; b < 2; ++b) {
-          const uint64_t gi = g0 + (uint64_t)((b * kGBranch + i * HW * kPix) >> 4);
 #pragma unroll
-          for (int tap = 0; tap < 9; ++tap)
-            mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), gi + (uint64_t)(((tap / 3 * HW + tap % 3) * kPix) >> 4),
-                     t0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
-        }
+      for (int tap = 0; tap < 9; ++tap)
+        mma_bf16(tmem + (uint32_t)((i * 2 + b) * 16), gi + (uint64_t)(((tap / 3 * HW + tap % 3) * kPix) >> 4),
+                 t0 + (uint64_t)(tap * 512 >> 4), kIdesc, tap > 0 ? 1u : 0u);
       mma_commit(mbar + 1);
-      // weight gradient: K = two pixels of the tile a step; rows = 16 channels of the pixels dx = 0..7
+      // weight gradient of one dy over a quarter of the K steps, in an accumulator of its own: K = two
+      // pixels of the tile a step; rows = 16 channels of the pixels dx = 0..7
+      const int dy = warp % 3, part = warp / 3;
+      const uint32_t acc = tmem + kTmemW + (uint32_t)((part * 3 + dy) * 16);
       const uint64_t am = smem_desc(smem_u32(sa), kPix, 128);
       const uint64_t gm = smem_desc(smem_u32(sg), kPix, 128);
-      for (int i = 0; i < TR; ++i)
-        for (int j = 0; j < TW; j += 2)
+      for (int st = part; st < TR * TW / 2; st += kGradParts) {
+        const int r = st / (TW / 2), j = 2 * (st % (TW / 2));
 #pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const uint64_t gj = gm + (uint64_t)((b * kGBranch + ((i + 1) * HW + j + 1) * kPix) >> 4);
-            const uint64_t aj = am + (uint64_t)((b * kABranch + ((i + 1) * AW + j + 1) * kPix) >> 4);
-#pragma unroll
-            for (int dy = 0; dy < 3; ++dy)
-              mma_bf16(tmem + kTmemW + (uint32_t)(dy * 16), aj + (uint64_t)((dy * AW * kPix) >> 4), gj, kIdescMN,
-                       (walked > 0 || i > 0 || j > 0 || b > 0) ? 1u : 0u);
-          }
+        for (int q = 0; q < 2; ++q)
+          mma_bf16(acc, am + (uint64_t)((q * kABranch + ((r + 1 + dy) * AW + j + 1) * kPix) >> 4),
+                   gm + (uint64_t)((q * kGBranch + ((r + 1) * HW + j + 1) * kPix) >> 4), kIdescMN,
+                   (walked > 0 || st > part || q > 0) ? 1u : 0u);
+      }
       mma_commit(mbar + 2);
     }
     tap_sums<-1>(sf, sd, AW, 2, wc, wq, wg, acc3);
@@ -455,6 +458,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (have) {
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + kTmemW + (uint32_t)(dy * 16), v);
         asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll 1
+        for (int part = 1; part < kGradParts; ++part) {
+          float u[16];
+          tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + kTmemW + (uint32_t)((part * 3 + dy) * 16), u);
+          asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+          for (int o = 0; o < 16; ++o) v[o] += u[o];
+        }
       } else {
 #pragma unroll
         for (int o = 0; o < 16; ++o) v[o] = 0.f;
