@@ -316,6 +316,14 @@ template <> const float* dinv<float>(const LevelDev& v) { return v.dinv32; }
 template <typename T> struct Fused { static constexpr bool on = false; };
 template <> struct Fused<float> { static constexpr bool on = true; };
 
+// Where the coarse end of a V-cycle is one kernel (run_tail): levels of at most one row a thread (1521 rows
+// in float32 with the coarse solve of 361 unknowns: 827 -> 838 us for the call; 3375: 1037 -> 1173; up to
+// 1024: h = 1/64, k = 8, float64 998 -> 954, h = 1/512, k = 128, mixed 1701 -> 1694).  The
+// coarse solve is inside up to these many unknowns: a float64 one of 225 takes a single SM's pipe 15 us, as
+// long as the product spread over the chip, which then runs between two halves of the kernel (in float32
+// larger ones leave the levels to their own kernels).
+constexpr int kTailRows = 1024, kTailCoarse32 = 256, kTailCoarse64 = 160;
+
 // Hooks before float32 post-smoothing on level l (cur = iterate after the
 // coarse correction, tmp = free buffer): the residual capture for training
 // data, and the learned smoothing step with its per-pair Jacobi fallback.
@@ -349,6 +357,55 @@ struct TopOut {
   double* X;
 };
 
+// The kernels of a level's V-cycle in one launch (vcycle_tail.cu) from level l down, or null where that
+// path does not serve or is not the faster one.
+template <typename T> T* run_tail(pasm_ctx* c, int l) {
+  constexpr bool f32 = Fused<T>::on;
+  if (l >= kTailLevels || c->opts.smoother == PASM_CG || c->lv[(size_t)l].n > kTailRows)
+    return nullptr;
+  int n[kTailLevels];
+  for (int q = 0; q <= l; ++q) {
+    const LevelDev& v = c->lv[(size_t)q];
+    n[q] = v.n;
+    if (q == 0) continue;
+    if (f32 && (!v.RA.rp || !v.A.w32)) return nullptr;
+    // levels whose launch shapes someone chose, that capture training data or run the learned step
+    for (int t : c->geo[(size_t)q]) if (t) return nullptr;
+    if (f32 && c->capture_level == q) return nullptr;
+    if (f32 && c->opts.smoother == PASM_LEARNED && c->nn.ready && c->nn.nx[(size_t)q] != 0) return nullptr;
+  }
+  const bool solve = c->NH <= (f32 ? kTailCoarse32 : kTailCoarse64);
+  if (f32 && !solve) return nullptr;
+  if (!vcycle_tail_fits<T>(n, l, solve ? TAIL_DOWN | TAIL_UP : TAIL_DOWN)) return nullptr;
+  TailArgs<T> a = {};
+  for (int q = 0; q <= l; ++q) {
+    const LevelDev& v = c->lv[(size_t)q];
+    TailLevel<T>& t = a.lv[q];
+    t.n = v.n;
+    auto csr = [](const DCsr& m) { return TailCsr<T>{m.rp, m.ci, vals<T>(m), scaled_vals<T>(m)}; };
+    t.nnz = v.A.nnz;
+    t.A = csr(v.A); t.R = csr(v.R); t.RA = csr(v.RA); t.P = csr(v.P);
+    t.dinv = dinv<T>(v);
+    t.gF = (T*)v.vF;
+    t.gE = (T*)v.vE;
+  }
+  a.Ainv = ainv<T>(c);
+  a.omega = (T)c->opts.omega;
+  a.top = l; a.ldk = c->ldk; a.nu_pre = c->opts.nu_pre; a.nu_post = c->opts.nu_post;
+  const Launch L = launcher(c);
+  if (solve) {
+    a.parts = TAIL_DOWN | TAIL_UP;
+    vcycle_tail<T>(L, a);
+  } else {
+    a.parts = TAIL_DOWN;
+    vcycle_tail<T>(L, a);
+    dense_mm<T>(L, c->NH, c->NH, a.Ainv, c->NH, false, a.lv[0].gF, a.lv[0].gE, c->ldk);
+    a.parts = TAIL_UP;
+    vcycle_tail<T>(L, a);
+  }
+  return (T*)c->lv[(size_t)l].vE;
+}
+
 template <typename T>
 T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
   const Launch L = launcher(c);
@@ -361,6 +418,8 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
     dense_mm<T>(L, c->NH, c->NH, ainv<T>(c), c->NH, false, F, E, ldk);
     return E;
   }
+  if (!top)
+    if (T* e = run_tail<T>(c, l)) return e;
   const T om = (T)c->opts.omega;
   const bool fuse = Fused<T>::on;
   T* cur = E;
@@ -895,6 +954,7 @@ static int setup_impl(pasm_ctx* c, int n_levels, const pasm_csr* A, const pasm_c
       Ai[(size_t)i * NH + j] = s;
     }
   CK(secular_prepare(NH));
+  CK(vcycle_tail_prepare());
   CK(nn_tc_prepare());
   CK(nn_tc_train_prepare());
   AL(c->allocs, &c->lamH, (size_t)NH);
