@@ -40,6 +40,13 @@
 // the cluster barrier orders the exchange.  GB300's float64 pipe (2 FMA per
 // clock and SM) bounds the root solves, so more SMs per pair is more
 // throughput.  Rank 0 alone writes the results.
+//
+// With the roots spread out a solve is one chain of dependent float64 operations (about 60 clocks each) and
+// of code fetched for the first time, 118,000 clocks at N_H = 225: loads and sums 12,700, pole lists 6,600,
+// a root 58,000 (midpoint 4,400, float32 phase 11,000 to 14,000, float64 phase 25,000, vector sums 14,800),
+// selection 15,000, result 19,600.  Hence the reciprocals in groups, the four sums of a pass in one
+// exchange, the block's sums together and the float32 slots no larger than N_H needs: 76 -> 66 us at
+// N_H = 225, k = 24 to 64; 252 -> 223 us where certificates fail and more roots are solved.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -72,19 +79,36 @@ struct SecShared {
   int* solved;    // NH+1
 };
 
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  v = warp_sum(v);
+// Block sums of N values at once (every thread gets them): their shuffles overlap.
+template <int N>
+__device__ __forceinline__ void block_sums(double (&v)[N], double* red) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int q = 0; q < N; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
   __syncthreads();
-  if (l == 0) red[w] = v;
+  if (l == 0) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) red[q * kSecWarps + w] = v[q];
+  }
   __syncthreads();
-  double t = (threadIdx.x < kSecWarps) ? red[threadIdx.x] : 0.0;
-  if (w == 0) t = warp_sum(t);
-  if (threadIdx.x == 0) red[0] = t;
+  // warp 0: lane 8 q + r holds warp r's sum of value q
+  static_assert(kSecWarps == 8 && N <= 3, "");
+  if (w == 0) {
+    double t = l < 8 * N ? red[l] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((l & 7) == 0 && l < 8 * N) red[24 + l / 8] = t;
+  }
   __syncthreads();
-  double r = red[0];
-  __syncthreads();
-  return r;
+#pragma unroll
+  for (int q = 0; q < N; ++q) v[q] = red[24 + q];
+}
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  double t[1] = {v};
+  block_sums<1>(t, red);
+  return t[0];
 }
 
 // 1/x for the pole sums, by Newton-Raphson iteration y <- y + y (1 - x y)
@@ -95,10 +119,15 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // only the four FMAs use the float64 pipe, GB300's scarce one.  Exponents
 // outside 2^(+-120) (where the float32 seed would leave the normal range),
 // zero, Inf and NaN take the float64 division.
+// rcp_in_range: the exponents the steps serve; the callers take several reciprocals at a time and send
+// the others to the division afterwards, so that their chains overlap.
+__device__ __forceinline__ bool rcp_in_range(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7FF;
+  return e >= 1023 - 120 && e <= 1023 + 120;
+}
 __device__ __forceinline__ double rcp_nr(double x) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) & 0x7FF;
-  if (e < 1023 - 120 || e > 1023 + 120) return 1.0 / x;
   const unsigned fb = ((unsigned)hi & 0x80000000u) | ((unsigned)(e - 896) << 23) | (((unsigned)hi & 0xFFFFFu) << 3) |
                       ((unsigned)__double2loint(x) >> 29);
   const unsigned rb = __float_as_uint(__frcp_rn(__uint_as_float(fb)));
@@ -111,19 +140,85 @@ __device__ __forceinline__ double rcp_nr(double x) {
   return fma(y, r, y);
 }
 
+// Sum over a warp of four values (every lane gets them): halves of the lanes take two of them after the
+// first exchange and quarters one after the second, 6 additions instead of 20 with each value's tree of
+// warp_sum, so the same bits.
+template <typename T>
+__device__ __forceinline__ void warp_sum4(int lane, T& a, T& b, T& c, T& d) {
+  const bool u = lane & 16, w = lane & 8;
+  const T k0 = u ? c : a, k1 = u ? d : b;
+  const T g0 = __shfl_xor_sync(0xffffffffu, u ? a : c, 16), g1 = __shfl_xor_sync(0xffffffffu, u ? b : d, 16);
+  const T p = k0 + g0, q = k1 + g1;
+  T x = (w ? q : p) + __shfl_xor_sync(0xffffffffu, w ? p : q, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  a = __shfl_sync(0xffffffffu, x, 0);
+  b = __shfl_sync(0xffffffffu, x, 8);
+  c = __shfl_sync(0xffffffffu, x, 16);
+  d = __shfl_sync(0xffffffffu, x, 24);
+}
+
+// x <- 1/x for kPoles values: the chains of the steps overlap, values outside their range follow.
+constexpr int kPoles = 4;
+__device__ __forceinline__ void rcp_group(double (&x)[kPoles]) {
+  double r[kPoles];
+  bool good = true;
+#pragma unroll
+  for (int u = 0; u < kPoles; ++u) {
+    r[u] = rcp_nr(x[u]);
+    good = good && rcp_in_range(x[u]);
+  }
+  if (!good) {
+#pragma unroll
+    for (int u = 0; u < kPoles; ++u)
+      if (!rcp_in_range(x[u])) r[u] = 1.0 / x[u];
+  }
+#pragma unroll
+  for (int u = 0; u < kPoles; ++u) x[u] = r[u];
+}
+
+// s1 += w_j / (d_j - theta), s2 += w_j / (d_j - theta)^2 over this lane's poles t, t + 32, ... < end
+// (t is left at the first one beyond).
+__device__ __forceinline__ void pole_sums(const SecShared& S, int end, double origin, double tau, int& t, double& s1,
+                                          double& s2) {
+  while (t < end) {
+    double x[kPoles], w[kPoles];
+#pragma unroll
+    for (int u = 0; u < kPoles; ++u) {
+      x[u] = 1.0; w[u] = 0.0;
+      if (t + 32 * u < end) {
+        const int j = S.J[t + 32 * u];
+        x[u] = (S.d[j] - origin) - tau;
+        w[u] = S.w[j];
+      }
+    }
+    rcp_group(x);
+#pragma unroll
+    for (int u = 0; u < kPoles; ++u) {
+      if (t + 32 * u < end) {
+        const double term = w[u] * x[u];
+        s1 += term;
+        s2 = fma(term, x[u], s2);
+      }
+    }
+    t += 32 * min(kPoles, (end - t + 31) / 32);
+  }
+}
+
 // Sums over the non-deflated poles at theta = origin + tau, split into the
 // poles left of root m (indices t < m) and right of it.  Warp-cooperative.
 __device__ __forceinline__ void secular_sums(const SecShared& S, int nJ, int m, double origin, double tau, int lane,
                                              double& psi, double& dpsi, double& phi, double& dphi) {
   psi = dpsi = phi = dphi = 0.0;
-  for (int t = lane; t < nJ; t += 32) {
-    const int j = S.J[t];
-    const double r = rcp_nr((S.d[j] - origin) - tau);
-    const double term = S.w[j] * r;
-    if (t < m) { psi += term; dpsi = fma(term, r, dpsi); }
-    else { phi += term; dphi = fma(term, r, dphi); }
+  int t = lane;
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    double s1 = 0.0, s2 = 0.0;
+    pole_sums(S, side == 0 ? m : nJ, origin, tau, t, s1, s2);
+    if (side == 0) { psi = s1; dpsi = s2; }
+    else { phi = s1; dphi = s2; }
   }
-  psi = warp_sum(psi); dpsi = warp_sum(dpsi); phi = warp_sum(phi); dphi = warp_sum(dphi);
+  warp_sum4(lane, psi, dpsi, phi, dphi);
 }
 
 // One step of the rational model of f around the iterate (see the file
@@ -134,17 +229,17 @@ template <typename T>
 __device__ __forceinline__ bool rational_step(bool has_left, bool has_right, T da, T db, T th, T rho, T psi,
                                               T dpsi, T phi, T dphi, T& s) {
   if (has_left && has_right) {
-    const T Q1 = dpsi * da * da, P1 = psi - Q1 / da;
+    const T q1 = dpsi * da, q2 = (dphi + T(1)) * db;
+    const T Q1 = q1 * da, P1 = psi - q1;
     const T ft = th - rho + phi;
-    const T Q2 = (dphi + T(1)) * db * db, P2 = ft - Q2 / db;
+    const T Q2 = q2 * db, P2 = ft - q2;
     const T P = P1 + P2;
     const T A2 = P, B2 = -(P * (da + db) + Q1 + Q2), C2 = P * da * db + Q1 * db + Q2 * da;
     const T disc = fmax(B2 * B2 - T(4) * A2 * C2, T(0));
     const T q = T(-0.5) * (B2 + copysign(sqrt(disc), B2));
-    bool ok = false;
-    if (A2 != T(0)) { const T s1 = q / A2; if (s1 > da && s1 < db) { s = s1; ok = true; } }
-    if (q != T(0)) { const T s2 = C2 / q; if (s2 > da && s2 < db) { s = s2; ok = true; } }
-    return ok;
+    if (q != T(0)) { const T s2 = C2 / q; if (s2 > da && s2 < db) { s = s2; return true; } }
+    if (A2 != T(0)) { const T s1 = q / A2; if (s1 > da && s1 < db) { s = s1; return true; } }
+    return false;
   }
   if (has_right) {  // first interval: only poles to the right
     const T Q2 = dphi * db * db, P2 = phi - Q2 / db;
@@ -169,8 +264,8 @@ __device__ __forceinline__ bool rational_step(bool has_left, bool has_right, T d
 
 // float32 pre-solve: the pole offsets d_j - origin and the weights z_j^2 of this
 // lane's share of the poles live in registers (at most kPer per lane).
-static constexpr int kPer = 32;  // supports NH <= 1024
-
+// (8, 16 or 32: N_H <= 256, 512, 1024; the slots beyond are code that has to be fetched)
+template <int kPer>
 __device__ __forceinline__ void sums32(const float (&dd)[kPer], const float (&zz)[kPer], int nJ, int m, int lane,
                                        float tau, float& psi, float& dpsi, float& phi, float& dphi) {
   psi = dpsi = phi = dphi = 0.f;
@@ -188,19 +283,14 @@ __device__ __forceinline__ void sums32(const float (&dd)[kPer], const float (&zz
       else { phi += term; dphi += dterm; }
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    psi += __shfl_xor_sync(0xffffffffu, psi, o);
-    dpsi += __shfl_xor_sync(0xffffffffu, dpsi, o);
-    phi += __shfl_xor_sync(0xffffffffu, phi, o);
-    dphi += __shfl_xor_sync(0xffffffffu, dphi, o);
-  }
+  warp_sum4(lane, psi, dpsi, phi, dphi);
 }
 
 // Root m of the secular equation (0 <= m <= nJ), computed by one warp: a
 // float32 rational iteration locates it, then float64 iterations from there
 // polish it (usually one or two) inside the float64 bracket.
-__device__ void solve_root(const SecShared& S, int nJ, int m, double rho, double lower, double upper, int lane,
+template <int kPer>
+__device__ __forceinline__ void solve_root(const SecShared& S, int nJ, int m, double rho, double lower, double upper, int lane,
                            int* caps) {
   const bool has_left = m > 0, has_right = m < nJ;
   if (!has_left && !has_right) {  // every pole deflated: the bordered row alone, theta = rho
@@ -225,8 +315,8 @@ __device__ void solve_root(const SecShared& S, int nJ, int m, double rho, double
       }
     }
   };
-  if (!has_left) { origin = b; lo = lower - b; hi = 0.0; load_offsets(origin); }
-  else if (!has_right) { origin = a; lo = 0.0; hi = upper - a; load_offsets(origin); }
+  if (!has_left) { origin = b; lo = lower - b; hi = 0.0; }
+  else if (!has_right) { origin = a; lo = 0.0; hi = upper - a; }
   else {
     // which half holds the root: the sign of f at the midpoint, in float64 (in
     // float32 the sum cancels badly when rho and the weights are large)
@@ -235,8 +325,8 @@ __device__ void solve_root(const SecShared& S, int nJ, int m, double rho, double
     secular_sums(S, nJ, m, 0.0, mid, lane, psi, dpsi, phi, dphi);
     if (mid - rho + psi + phi >= 0.0) { origin = a; lo = 0.0; hi = mid - a; }
     else { origin = b; lo = mid - b; hi = 0.0; }
-    load_offsets(origin);
   }
+  load_offsets(origin);
   // float32 phase
   double tau;
   {
@@ -299,13 +389,30 @@ __device__ __forceinline__ void root_vector_sums(const SecShared& S, int nK, int
                                                  double& yc) {
   const double origin = S.orig[m], tau = S.tau[m];
   ny2 = 0.0; yc = 0.0;
-  for (int t = lane; t < nK; t += 32) {
-    const int j = S.K[t];
-    const double y = -S.z[j] * rcp_nr((S.d[S.pole[j]] - origin) - tau);
-    ny2 = fma(y, y, ny2);
-    yc = fma(y, S.cq[j], yc);
+  for (int t = lane; t < nK; t += 32 * kPoles) {
+    double x[kPoles], z[kPoles], q[kPoles];
+#pragma unroll
+    for (int u = 0; u < kPoles; ++u) {
+      x[u] = 1.0; z[u] = q[u] = 0.0;
+      if (t + 32 * u < nK) {
+        const int j = S.K[t + 32 * u];
+        x[u] = (S.d[S.pole[j]] - origin) - tau;
+        z[u] = S.z[j];
+        q[u] = S.cq[j];
+      }
+    }
+    rcp_group(x);
+#pragma unroll
+    for (int u = 0; u < kPoles; ++u) {
+      if (t + 32 * u < nK) {
+        const double y = -z[u] * x[u];
+        ny2 = fma(y, y, ny2);
+        yc = fma(y, q[u], yc);
+      }
+    }
   }
-  ny2 = warp_sum(ny2); yc = warp_sum(yc);
+  double none = 0.0, none2 = 0.0;
+  warp_sum4(lane, ny2, yc, none, none2);
 }
 
 // A selection candidate: score, Ritz value, preference order, kind (0 root,
@@ -401,6 +508,7 @@ __device__ __forceinline__ int block_min(int v, int* buf) {
   return r;
 }
 
+template <int kPer>
 __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
   extern __shared__ double smem[];
   __shared__ double red[32];
@@ -447,7 +555,11 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
     S.d[j] = dj; S.cq[j] = cj; S.z[j] = bj;  // z holds b' until rescaled
     scc = fma(cj, cj, scc); scb = fma(cj, bj, scb); sdcc = fma(dj * cj, cj, sdcc);
   }
-  scc = block_sum(scc, red); scb = block_sum(scb, red); sdcc = block_sum(sdcc, red);
+  {
+    double t[3] = {scc, scb, sdcc};
+    block_sums<3>(t, red);
+    scc = t[0]; scb = t[1]; sdcc = t[2];
+  }
   const double beta = a.beta[i], zeta = a.zeta[i];
   const double zt = zeta - scc;
   if (!(zt > 1e-14 * zeta)) {  // u~ numerically inside V_H: keep the pair for this step
@@ -551,7 +663,7 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
     const int mmax = phase == 0 ? -1 : (phase == 1 ? min(nJ, s_m0 + 8) : nJ);
     // a solved root's theta, origin, offset and score go to every CTA of the cluster
     auto solve_and_publish = [&](int m) {
-      solve_root(S, nJ, m, rho, lower, upper, lane, a.diag + 2);
+      solve_root<kPer>(S, nJ, m, rho, lower, upper, lane, a.diag + 2);
       double ny2, yc;
       root_vector_sums(S, nK, m, lane, ny2, yc);
       if (lane == 0) {
@@ -618,8 +730,10 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
         best.offer(sc, thj, NH + 1 + j, kind, j);
       }
       best = block_best(best, s_cand);
-      mass = block_sum(mass, red);
-      const double nsd = block_sum((double)nsolved, red);
+      double t[2] = {mass, (double)nsolved};
+      block_sums<2>(t, red);
+      mass = t[0];
+      const double nsd = t[1];
       m_unsolved = block_min(m_unsolved, s_imin);
       if (tid == 0) {
         int cert = 1;
@@ -718,8 +832,13 @@ static size_t secular_smem(int NH) {
   return sizeof(double) * (4 * (size_t)NH + 4 * ((size_t)NH + 1)) + sizeof(int) * (4 * (size_t)NH + (size_t)NH + 1);
 }
 
+using SecKernel = void (*)(SecularArgs);
+static SecKernel secular_kernel(int NH) {
+  return NH <= 256 ? k_secular<8> : NH <= 512 ? k_secular<16> : k_secular<32>;
+}
+
 cudaError_t secular_prepare(int NH) {
-  return allow_dynamic_smem((const void*)k_secular, secular_smem(NH));
+  return allow_dynamic_smem((const void*)secular_kernel(NH), secular_smem(NH));
 }
 
 // CTAs per pair: as many (up to 4) as keep all of them co-resident on the SMs.
@@ -754,7 +873,7 @@ void secular_select(const Launch& L, const SecularArgs& a0) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = L.pdl ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, k_secular, a);
+  cudaLaunchKernelEx(&cfg, secular_kernel(a.NH), a);
   L.bump();
 }
 
