@@ -126,8 +126,9 @@ template <typename T, int CH, int OP>
 __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                                                    const T* __restrict__ av, const T* __restrict__ X,
                                                    const T* Y, const T* Z, const T* __restrict__ dinv, T omega,
-                                                   T* out, int ldk, int tpr, int rpt) {
+                                                   T* out, const T* B, int ldk, int tpr, int rpt) {
   constexpr int V = Vec16<T>::N;
+  constexpr bool SWEEP = OP == OP_JACOBI || OP == OP_JACOBI_ADD;
   const int rpb = kBlock / tpr;
   const int lane = threadIdx.x % tpr;
   pdl_trigger();
@@ -143,16 +144,20 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int 
     for (int v = 0; v < V; ++v) acc[c][v] = T(0);
   // row-aligned operands first: their loads overlap the gather's round trips
   const size_t base = (size_t)row * ldk;
-  T y[CH][V], z[CH][V];
+  T y[CH][V], z[CH][V], b[CH][V];
   T w = T(0);
   if (OP != OP_SPMM) {
 #pragma unroll
     for (int c = 0; c < CH; ++c) ldg16<T>(Y + base + (c * tpr + lane) * V, y[c]);
   }
-  if (OP == OP_JACOBI) {
+  if (SWEEP) {
     w = omega * dinv[row];
 #pragma unroll
     for (int c = 0; c < CH; ++c) ldg16<T>(Z + base + (c * tpr + lane) * V, z[c]);
+  }
+  if (OP == OP_JACOBI_ADD) {
+#pragma unroll
+    for (int c = 0; c < CH; ++c) ldg16<T>(B + base + (c * tpr + lane) * V, b[c]);
   }
   gather_rows<T, CH>(ci, av, nullptr, T(0), X, rp[row], rp[row + 1], lane, tpr, ldk, acc);
 #pragma unroll
@@ -161,10 +166,11 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int 
     T r[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      if (OP == OP_JACOBI) r[v] = fma(w, y[c][v] - acc[c][v], z[c][v]);
+      if (SWEEP) r[v] = fma(w, y[c][v] - acc[c][v], z[c][v]);
       else if (OP == OP_RESID) r[v] = y[c][v] - acc[c][v];
       else if (OP == OP_SPMM) r[v] = acc[c][v];
       else r[v] = y[c][v] + acc[c][v];
+      if (OP == OP_JACOBI_ADD) r[v] = b[c][v] + r[v];
     }
     Vec16<T>::store(out + off, r);
   }
@@ -173,7 +179,7 @@ __global__ void __launch_bounds__(kBlock, (RowMinBlocks<T, CH>::v)) k_rowop(int 
 
 template <typename T>
 void rowop(const Launch& L, RowOp op, const DCsr& S, const T* X, const T* Y, const T* Z, const T* dinv, T omega,
-           T* out, int ldk) {
+           T* out, int ldk, const T* B) {
   if (S.n_rows == 0) return;
   Geo g = geometry<T>(ldk, L.geo);
   const int rpb = kBlock / g.tpr;
@@ -186,6 +192,7 @@ void rowop(const Launch& L, RowOp op, const DCsr& S, const T* X, const T* Y, con
     double flops = 2.0 * nnz * ldk;
     int cls = KC_SPMM;
     if (op == OP_JACOBI) { bytes += rows * ldk * sz + rows * sz; flops += 3.0 * rows * ldk; cls = KC_JACOBI; }
+    else if (op == OP_JACOBI_ADD) { bytes += 2.0 * rows * ldk * sz + rows * sz; flops += 4.0 * rows * ldk; cls = KC_SWEEP_UPDATE; }
     else if (op == OP_RESID) { bytes += rows * ldk * sz; flops += rows * ldk; cls = KC_RESID; }
     else if (op == OP_SPMM_ADD) { bytes += rows * ldk * sz; flops += rows * ldk; cls = KC_PROLONG; }
     L.rows(S.n_rows);
@@ -193,17 +200,21 @@ void rowop(const Launch& L, RowOp op, const DCsr& S, const T* X, const T* Y, con
   }
   PASM_DISPATCH_CH(g.ch,
     switch (op) {
-      case OP_JACOBI: launch(L, k_rowop<T, CH, OP_JACOBI>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_RESID: launch(L, k_rowop<T, CH, OP_RESID>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_SPMM: launch(L, k_rowop<T, CH, OP_SPMM>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
-      case OP_SPMM_ADD: launch(L, k_rowop<T, CH, OP_SPMM_ADD>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, ldk, g.tpr, rpt); break;
+      case OP_JACOBI: launch(L, k_rowop<T, CH, OP_JACOBI>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, B, ldk, g.tpr, rpt); break;
+      case OP_RESID: launch(L, k_rowop<T, CH, OP_RESID>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, B, ldk, g.tpr, rpt); break;
+      case OP_SPMM: launch(L, k_rowop<T, CH, OP_SPMM>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, B, ldk, g.tpr, rpt); break;
+      case OP_SPMM_ADD: launch(L, k_rowop<T, CH, OP_SPMM_ADD>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, B, ldk, g.tpr, rpt); break;
+      case OP_JACOBI_ADD:
+        if constexpr (sizeof(T) == 8)
+          launch(L, k_rowop<T, CH, OP_JACOBI_ADD>, grid, kBlock, 0, S.n_rows, S.rp, S.ci, av, X, Y, Z, dinv, omega, out, B, ldk, g.tpr, rpt);
+        break;
     });
   L.bump();
 }
 template void rowop<double>(const Launch&, RowOp, const DCsr&, const double*, const double*, const double*,
-                            const double*, double, double*, int);
+                            const double*, double, double*, int, const double*);
 template void rowop<float>(const Launch&, RowOp, const DCsr&, const float*, const float*, const float*,
-                           const float*, float, float*, int);
+                           const float*, float, float*, int, const float*);
 
 // ----------------------------------------------------------------------------------------------
 // Prolongate-and-correct fused with the first post-smoothing sweep (float32 cycles):

@@ -86,16 +86,17 @@ inline void launch(const Launch& L, void (*kernel)(P...), dim3 grid, dim3 block,
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-enum RowOp { OP_JACOBI = 0, OP_RESID = 1, OP_SPMM = 2, OP_SPMM_ADD = 3 };
+enum RowOp { OP_JACOBI = 0, OP_RESID = 1, OP_SPMM = 2, OP_SPMM_ADD = 3, OP_JACOBI_ADD = 4 };
 
 // out = op(S, X, Y, Z) row by row on n x ldk block vectors (row-major):
 //   OP_JACOBI : out = Z + omega * dinv .* (Y - S X)      (damped Jacobi sweep)
 //   OP_RESID  : out = Y - S X                            (residual)
 //   OP_SPMM   : out = S X                                (restriction / product)
 //   OP_SPMM_ADD: out = Y + S X                           (prolongate and correct)
+//   OP_JACOBI_ADD: out = B + the sweep of OP_JACOBI      (float64: a cycle's last sweep and the outer update)
 template <typename T>
 void rowop(const Launch& L, RowOp op, const DCsr& S, const T* X, const T* Y, const T* Z, const T* dinv,
-           T omega, T* out, int ldk);
+           T omega, T* out, int ldk, const T* B = nullptr);
 // out = xn + omega D^{-1} (F - A xn), xn = X + P Ec (prolongation fused with the first float32
 // post-smoothing sweep; the operations of rowop(OP_SPMM_ADD) then rowop(OP_JACOBI), in their order)
 void prolong_jacobi(const Launch& L, const DCsr& A, const DCsr& P, const float* X, const float* Ec, const float* F,

@@ -349,8 +349,8 @@ int post_hooks(pasm_ctx* c, int l, float* cur, float* tmp, float* F) {
   return 1;
 }
 
-// Top-level output of a mixed-precision V-cycle: the last post-smoothing sweep
-// writes X = B + e directly (double-float pairs) instead of e.
+// Top-level output of a V-cycle: the last post-smoothing sweep writes X = B + e
+// directly (mixed precision: double-float pairs) instead of e.
 struct TopOut {
   const double* B;
   bool b_ff;
@@ -418,7 +418,7 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
     dense_mm<T>(L, c->NH, c->NH, ainv<T>(c), c->NH, false, F, E, ldk);
     return E;
   }
-  if (!top)
+  if (!top || !Fused<T>::on)
     if (T* e = run_tail<T>(c, l)) return e;
   const T om = (T)c->opts.omega;
   const bool fuse = Fused<T>::on;
@@ -492,6 +492,14 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
                      top->B, top->b_ff, top->X, ldk);
       return nullptr;
     }
+    if constexpr (!Fused<T>::on) {
+      // the outer update in a pass of its own took 60 us at h = 1/512, k = 64 (the solve 4424 -> 4379 us)
+      if (top && s == c->opts.nu_post - 1) {
+        rowop<double>(launcher(c, l, PASM_TILE_JACOBI), OP_JACOBI_ADD, v.A, cur, F, cur, v.dinv64, om, top->X, ldk,
+                      top->B);
+        return nullptr;
+      }
+    }
     rowop<T>(launcher(c, l, PASM_TILE_JACOBI), OP_JACOBI, v.A, cur, F, cur, dinv<T>(v), om, tmp, ldk);
     std::swap(cur, tmp);
   }
@@ -532,12 +540,14 @@ void bvp_impl(pasm_ctx* c, int lt, const double* lam, const double* U, double* X
     const int nb = residual_partials<T>(L, v.n, c->ldk, Ftop, false, c->Fd, U, c->partials, c->max_border_blocks);
     column_sums(L, c->partials, nb, 2, c->ldk, c->rsum);
   }
-  T* e = vcycle<T>(c, lt);
-  outer_axpy<T>(L, v.n, U, e, X, c->ldk);
+  const TopOut first{U, false, X};
+  T* e = vcycle<T>(c, lt, lt >= 1 ? &first : nullptr);
+  if (e) outer_axpy<T>(L, v.n, U, e, X, c->ldk);
   for (int cyc = 1; cyc < c->opts.cycles_per_step; ++cyc) {
     outer_residual<T>(launcher(c, lt, PASM_TILE_OUTER_RES), v.A, c->Fd, X, Ftop, c->ldk);
-    e = vcycle<T>(c, lt);
-    outer_axpy<T>(L, v.n, X, e, X, c->ldk);
+    const TopOut next{X, false, X};
+    e = vcycle<T>(c, lt, lt >= 1 ? &next : nullptr);
+    if (e) outer_axpy<T>(L, v.n, X, e, X, c->ldk);
   }
 }
 
