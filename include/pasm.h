@@ -228,6 +228,9 @@ int pasm_project(pasm_ctx* ctx, const double* b, const double* c, double* bq, do
  * at setup, faster than both forms of R (f - A e); it then runs instead.  It
  * also runs where neither it nor PASM_TILE_RESID_RESTRICT has a shape (both 0:
  * levels the autotuner leaves out, and autotune = 0), in mixed precision.
+ * Levels of at most 1024 rows run as one kernel with those below them while no
+ * shape is set on any of them (same results); a level with one, and those
+ * above it, run a kernel per operation.
  * Errors: PASM_EINVAL. */
 int pasm_tiles(pasm_ctx* ctx, int level, int* chunks_per_thread);
 
@@ -291,7 +294,8 @@ enum {
   PASM_KC_RESID,        /* multigrid residual f - A e                             */
   PASM_KC_SPMM,         /* restriction P^T r and float64 transfer chains          */
   PASM_KC_PROLONG,      /* prolongate and correct e += P e_c                      */
-  PASM_KC_DENSE,        /* coarse dense products (A_H^-1, Q^T, Q)                 */
+  PASM_KC_DENSE,        /* coarse dense products (A_H^-1, Q^T, Q); the V-cycle on
+                           the levels that run as one kernel                      */
   PASM_KC_OUTER_RHS,    /* f = lambda M u and the first float64 residual          */
   PASM_KC_OUTER_RES,    /* later float64 residuals of the defect correction       */
   PASM_KC_AXPY,         /* x += e                                                 */
