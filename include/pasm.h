@@ -352,7 +352,7 @@ int pasm_nn_setup(pasm_ctx* ctx, const int32_t* nx, const float* weights);
 int pasm_nn_get_weights(pasm_ctx* ctx, float* weights);
 
 /* D = N(R) for the k columns of R on level `level` (n_l x k float32 row-major,
- * host or device).  Synchronises. */
+ * host or device; R and D may share memory).  Synchronises. */
 int pasm_nn_apply(pasm_ctx* ctx, int level, int k, const float* R, float* D);
 
 /* loss L and its gradient dL/dW (2592 float32, host or device) for the

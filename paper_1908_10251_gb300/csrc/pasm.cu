@@ -1724,8 +1724,11 @@ int pasm_nn_apply(pasm_ctx* c, int level, int k, const float* R, float* D) {
   if (r) return r;
   auto& nn = c->nn;
   NNGrid g{nn.nx[(size_t)level], nn.ny[(size_t)level], ldk2, k};
-  // blocks of this device without padded columns are read and written in place (16-byte loads)
-  if (tc && k == ldk2 && R != D && ((uintptr_t)R % 16) == 0 && on_device(R) && on_device(D)) {
+  // blocks of this device without padded columns are read and written in place (16-byte loads); not
+  // blocks that share memory: a tile's output would fall on the halo that another tile still reads
+  const uintptr_t r0 = (uintptr_t)R, d0 = (uintptr_t)D, size = sizeof(float) * (uintptr_t)n * (uintptr_t)k;
+  const bool apart = r0 + size <= d0 || d0 + size <= r0;
+  if (tc && k == ldk2 && apart && r0 % 16 == 0 && on_device(R) && on_device(D)) {
     nn_forward_tc(launcher(c), g, &nn.w13, nullptr, nn.w2, R, D, nn.err);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(c->s));
