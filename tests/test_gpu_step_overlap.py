@@ -56,3 +56,18 @@ def test_secular_blocks_spread_over_the_sms(precision):
         alone.append(sum(v[0] for v in pg.pasm_trace_step(ctx).values()) * 1e3)
     assert replay_us(pg, ctx, restart) <= float(np.median(alone[1:]))
     pg.pasm_destroy(ctx)
+
+
+def test_coarse_levels_in_one_kernel_are_no_slower(k=8):
+    """The coarse end of the float64 cycle (961 rows over 225 coarse unknowns), a block per column, against the same
+    levels with a kernel per operation (which a set launch shape selects)."""
+    from paper_1908_10251_gb300 import build
+    build.build()
+    import paper_1908_10251_gb300 as pg
+    ctx, restart = start(pg, (2, 64, 16), k, 0)
+    sep, restart_sep = start(pg, (2, 64, 16), k, 0)
+    restart_sep()
+    pg.pasm_set_tiles(sep, 1, {"jacobi": 1})
+    assert replay_us(pg, ctx, restart) <= replay_us(pg, sep, restart_sep)
+    pg.pasm_destroy(ctx)
+    pg.pasm_destroy(sep)
