@@ -698,8 +698,9 @@ __global__ void __launch_bounds__(kBlock) k_border(int n, const int* __restrict_
 #pragma unroll
   for (int c = 0; c < CH; ++c) sA[c][0] = sA[c][1] = sM[c][0] = sM[c][1] = 0.0;
   pdl_trigger();
-  prefetch_row(arp, aci, aval, blockIdx.x * rpb + grp, n);
-  prefetch_row(mrp, mci, mval, blockIdx.x * rpb + grp, n);
+  // no prefetch of the first rows: it gained nothing in a step, and in pasm_border_noalloc, which launches
+  // this kernel plainly, it was a chain of two loads before the first gather (3D, h = 1/64, k = 8: 125.7 us
+  // against 122.3)
   pdl_wait();
   for (int row = blockIdx.x * rpb + grp; row < n; row += gridDim.x * rpb) {
     double ya[CH][2], ym[CH][2];
@@ -765,6 +766,7 @@ __global__ void __launch_bounds__(128) k_colsum(const double* __restrict__ parti
   pdl_wait();
   const int t = blockIdx.x;
   double s = 0.0;
+#pragma unroll 4
   for (int b = threadIdx.x; b < nblk; b += 128) s += ld1(partials + (size_t)b * width + t);
   s = warp_sum(s);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
