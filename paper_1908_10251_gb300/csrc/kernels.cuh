@@ -156,7 +156,7 @@ template <typename T> struct TailCsr {
 };
 template <typename T> struct TailLevel {
   int n;
-  int64_t nnz;                                 // of A (accounting)
+  int64_t nnz_A, nnz_R, nnz_RA, nnz_P;         // (accounting)
   TailCsr<T> A, R, RA, P;                      // RA: float32 only
   const T* dinv;
   T *gF, *gE;                                  // n x ldk: right-hand side; iterate

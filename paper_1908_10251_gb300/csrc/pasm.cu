@@ -383,7 +383,7 @@ template <typename T> T* run_tail(pasm_ctx* c, int l) {
     TailLevel<T>& t = a.lv[q];
     t.n = v.n;
     auto csr = [](const DCsr& m) { return TailCsr<T>{m.rp, m.ci, vals<T>(m), scaled_vals<T>(m)}; };
-    t.nnz = v.A.nnz;
+    t.nnz_A = v.A.nnz; t.nnz_R = v.R.nnz; t.nnz_RA = v.RA.nnz; t.nnz_P = v.P.nnz;
     t.A = csr(v.A); t.R = csr(v.R); t.RA = csr(v.RA); t.P = csr(v.P);
     t.dinv = dinv<T>(v);
     t.gF = (T*)v.vF;

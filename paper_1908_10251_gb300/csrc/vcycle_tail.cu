@@ -278,17 +278,37 @@ void vcycle_tail(const Launch& L, TailArgs<T> a) {
   const size_t smem = tail_layout<T>(a);
   const bool down = (a.parts & TAIL_DOWN) != 0, up = (a.parts & TAIL_UP) != 0;
   {
-    double bytes = 0.0, flops = 0.0;
+    // matrices once (the second sweep from zero has values of its own), what leaves and enters the kernel once
+    const bool f32 = sizeof(T) == 4, two = f32 && a.nu_pre >= 2;
+    const double w = sizeof(T), ldk = a.ldk, n0 = a.lv[0].n;
+    const int down_sweeps = down ? std::max(0, a.nu_pre - (two ? 2 : 1)) : 0, up_sweeps = up ? a.nu_post : 0;
+    double bytes = 0.0, flops = 0.0, vec = 0.0;
     for (int l = 1; l <= a.top; ++l) {
-      const double n = a.lv[l].n, nnz = (double)a.lv[l].nnz;
-      const int passes = (down ? a.nu_pre + 1 : 0) + (up ? a.nu_post + 1 : 0);
-      bytes += nnz * (4.0 + sizeof(T));
-      flops += (double)passes * (2.0 * nnz + 3.0 * n) * a.ldk;
+      const TailLevel<T>& v = a.lv[l];
+      const double n = v.n, nc = a.lv[l - 1].n, A = (double)v.nnz_A, R = (double)v.nnz_R, RA = (double)v.nnz_RA,
+                   P = (double)v.nnz_P, row = 4.0, entry = 4.0 + w;
+      const int products = down_sweeps + up_sweeps + (down && !f32 ? 1 : 0);   // with A's own values
+      if (products > 0 || (down && two)) bytes += (n + 1) * row + A * 4.0;
+      if (products > 0) bytes += A * w;
+      if (down && two) bytes += A * w;
+      if (down) bytes += (nc + 1) * row + R * entry + (f32 ? (nc + 1) * row + RA * entry : 0.0);
+      if (up) bytes += (n + 1) * row + P * entry;
+      if ((down && a.nu_pre > 0) || up_sweeps > 0) bytes += n * w;
+      flops += ldk * ((down_sweeps + up_sweeps) * (2.0 * A + 3.0 * n));
+      if (down) {
+        flops += ldk * (two ? 2.0 * A + 3.0 * n : a.nu_pre >= 1 ? n : 0.0);
+        flops += ldk * (f32 ? 2.0 * (R + RA) + nc : 2.0 * (A + R) + n);
+      }
+      if (up) flops += ldk * (2.0 * P + n);
+      if (!up) vec += n + nc;                            // iterate; right-hand side below
+      if (!down) vec += n + (l == 1 ? nc : 0.0) + n;     // both read back
     }
-    bytes += 2.0 * a.lv[a.top].n * a.ldk * sizeof(T);
+    if (down) vec += a.lv[a.top].n;
+    if (up) vec += a.lv[a.top].n;
+    bytes += vec * ldk * w;
     if (down && up) {
-      bytes += (double)a.lv[0].n * a.lv[0].n * sizeof(T);
-      flops += 2.0 * (double)a.lv[0].n * a.lv[0].n * a.ldk;
+      bytes += n0 * n0 * w;
+      flops += 2.0 * n0 * n0 * ldk;
     }
     L.rows(a.lv[a.top].n);
     L.begin(KC_DENSE, bytes, flops);
