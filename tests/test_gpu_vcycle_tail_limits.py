@@ -93,3 +93,43 @@ def test_traced_bytes_and_flops(precision, sizes, top, nu_pre, nu_post):
     want = [accounted(levels, top, ldk, precision == 1, nu_pre, nu_post, *p) for p in parts]
     assert got == want * 2                       # two cycles a step
     pg.pasm_destroy(ctx)
+
+
+# (precision, rows of the levels, the highest level in the kernel or None): at most 1024 rows; a coarse solve of at
+# most 160 unknowns in float64 (above, it runs between two halves of the kernel) and 256 in mixed precision (above, a
+# kernel per operation); mixed precision's finest level stays outside; shared memory; eight levels
+ROUTES = [(0, (160, 1024, 2050), 1), (0, (161, 1024, 2050), 1), (0, (160, 1025, 2050), None), (0, (100, 1000), 1),
+          (1, (256, 1024, 2050), 1), (1, (257, 1024, 2050), None), (1, (160, 1025, 2050), None), (1, (100, 1000), None),
+          (0, (160, 900, 1000, 1024, 2100), 3), (1, (256, 900, 1000, 1024, 2100), 2),
+          (0, (8, 12, 18, 27, 40, 60, 90, 135, 200, 300), 7), (1, (8, 12, 18, 27, 40, 60, 90, 135, 200, 300), 7)]
+
+
+@pytest.mark.parametrize("precision,sizes,top", ROUTES)
+@pytest.mark.parametrize("k", [5, 40])
+def test_route_and_bits(precision, sizes, top, k):
+    """The kernel runs where it should (its launches in a traced step) and nowhere else, and gives the bits of a kernel
+    per operation (which a set launch shape selects)."""
+    from paper_1908_10251_gb300 import build
+    build.build()
+    import paper_1908_10251_gb300 as pg
+    levels = hierarchy(sizes)
+    n = sizes[-1]
+    U = np.random.default_rng(n + k).standard_normal((n, k))
+    lam = 10.0 + np.arange(k, dtype=np.float64)
+    out, ran, launches = [], [], []
+    for separate in (False, True):
+        ctx = context(pg, levels, k, precision, 2, 2)
+        if separate:
+            for level in range(1, len(sizes)):
+                pg.pasm_set_tiles(ctx, level, {"jacobi": 1})
+        Uh = np.zeros((n, k))
+        pg.pasm_bvp(ctx, lam, U, Uh)
+        out.append(Uh)
+        pg.pasm_trace_step(ctx)
+        ran.append([rows for c, rows, *_ in pg.pasm_trace_launches(ctx) if c == "dense" and rows])
+        launches.append(len(pg.pasm_trace_launches(ctx)))
+        pg.pasm_destroy(ctx)
+    halves = 2 if precision == 0 and sizes[0] > 160 else 1
+    assert ran == [[] if top is None else [sizes[top]] * 2 * halves, []]   # two cycles a step
+    assert (launches[0] < launches[1]) == (top is not None)
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
