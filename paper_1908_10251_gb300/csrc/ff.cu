@@ -263,13 +263,16 @@ __global__ void __launch_bounds__(kBlock, kMinBlocksGather)
   ff2 axh[CH], axl[CH];
   gather_row_ff<CH, true, AEX>(arp, aci, aval, X, row, lane, tpr, ldk, axh, axl);
   const size_t base = (size_t)row * ldk;
+  // every chunk's Fd before the first store: a load after a store that it might alias waits for its turn, and
+  // the chunks' round trips went one by one (h = 1/1024, k = 64: 331 us against 270)
+  ff2 fh[CH], fl[CH];
 #pragma unroll
-  for (int c = 0; c < CH; ++c) {
-    const int col = (c * tpr + lane) * 2;
-    ff2 fh, fl;
-    load_pair<true>(reinterpret_cast<const double*>(Fd), base + col, fh, fl);
-    *reinterpret_cast<ff2*>(R + base + col) = ff2_addrn(ff2_subrn(fh, axh[c]), ff2_subrn(fl, axl[c]));
-  }
+  for (int c = 0; c < CH; ++c)
+    load_pair<true>(reinterpret_cast<const double*>(Fd), base + (c * tpr + lane) * 2, fh[c], fl[c]);
+#pragma unroll
+  for (int c = 0; c < CH; ++c)
+    *reinterpret_cast<ff2*>(R + base + (c * tpr + lane) * 2) =
+        ff2_addrn(ff2_subrn(fh[c], axh[c]), ff2_subrn(fl[c], axl[c]));
   }
 }
 
