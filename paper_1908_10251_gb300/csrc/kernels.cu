@@ -1035,9 +1035,10 @@ namespace pasm {
 // The last Jacobi sweep of the top-level V-cycle fused with the outer update of
 // the mixed path: e' = z + omega dinv (y - A z) in float32 as k_rowop<float, JACOBI>,
 // then X = B + e' in double-float ((hi, lo) float pairs, B in pairs or float64),
-// so e' is never stored.
+// so e' is never stored.  Bound by memory: one chunk per thread is held to 32 registers for 2048
+// threads an SM (left to the compiler it takes 40: 267 us against 249 at h = 1/1024, k = 64).
 template <int CH, bool BFF>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, CH == 1 ? 8 : 0)
     k_jacobi_axpy_ff(int n, const int* __restrict__ rp, const int* __restrict__ ci, const float* __restrict__ av,
                      const float* __restrict__ E, const float* __restrict__ F, const float* __restrict__ dinv,
                      float omega, const double* B, double* X, int ldk, int tpr, int rpt) {
