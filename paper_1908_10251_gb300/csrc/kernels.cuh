@@ -54,7 +54,8 @@ struct Launch {
   int geo = 0;  // row-group kernels: 16-byte chunks per thread (0 = default; set by the autotuner)
   int rpt = 0;  // float32 row kernels: row blocks each block walks (0 = by size; set by the autotuner)
   bool pdl = true;  // programmatic dependent launch (see `launch`); off where an operand that is static in a
-                    // context may have been written by the kernel before
+                    // context may have been written by the kernel before, and by plain()
+  Launch plain() const { Launch q = *this; q.pdl = false; return q; }
   void begin(int cls, double bytes, double flops) const { if (tr) tracer_begin(tr, s, cls, bytes, flops); }
   void rows(int n) const { if (tr) tracer_rows(tr, n); }
   void bump() const {
@@ -71,6 +72,9 @@ struct Launch {
 // other kernels write is loaded through the volatile loads of common.cuh: a load through a const
 // __restrict__ pointer or __ldg is one the compiler may move above the wait.
 // A launch gap between two small kernels costs 1 to 1.5 us; a step has 40 to 80.
+// Kernels whose blocks are each bound by their SM (the float64 pipe, one chain of latencies) are launched
+// plainly (Launch::plain): blocks that start while the kernel before drains go to the SMs that free up
+// first and share them, while others stay empty.  Figures stand at each of them.
 template <typename... P, typename... A>
 inline void launch(const Launch& L, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
   cudaLaunchConfig_t cfg = {};

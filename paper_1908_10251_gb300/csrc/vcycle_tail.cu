@@ -316,9 +316,7 @@ void vcycle_tail(const Launch& L, TailArgs<T> a) {
   // Not a programmatic launch: blocks that start while the kernel before drains go to the SMs that free up
   // first, two to one SM (to one float64 pipe) while others stay empty (a float64 step at h = 1/64, N_H = 225,
   // k = 8: 233 us against 290, and 277 with a kernel per operation).
-  Launch plain = L;
-  plain.pdl = false;
-  launch(plain, k_vcycle_tail<T>, a.ldk / TailCols<T>::v, kTailThreads, smem, a);
+  launch(L.plain(), k_vcycle_tail<T>, a.ldk / TailCols<T>::v, kTailThreads, smem, a);
   L.bump();
 }
 
