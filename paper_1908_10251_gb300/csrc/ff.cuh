@@ -44,8 +44,10 @@ __device__ __forceinline__ double ff_to_double(float hi, float lo) { return __da
 // ----------------------------------------------------------------------------------------------
 // The arithmetic, on two values at once: the packed float32 instructions of sm_100 and later (f32x2)
 // take one issue slot for two lanes' worth of work.  The float32 pipe's rate is the same and so are the
-// results; the kernels of ff.cu were bound by issue (65 % of the slots at h = 1/320, k = 37).  A block vector "in pairs" stores two columns as one
-// 16-byte chunk (hi0, hi1, lo0, lo1), so that a 16-byte load gives both packed operands.
+// results.  It takes the bordering kernel from 266 to 174 thread instructions an entry and its issue slots
+// from 65 to 46 % busy (h = 1/512, k = 64; 182 -> 172 us): what is left is the latency of the gathers at
+// half occupancy, beside a float32 pipe that is 53 % busy.  A block vector "in pairs" stores two columns as
+// one 16-byte chunk (hi0, hi1, lo0, lo1), so that a 16-byte load gives both packed operands.
 typedef unsigned long long ff2;  // two float32
 
 __device__ __forceinline__ ff2 ff2_pack(float a, float b) {

@@ -15,10 +15,10 @@
 //            quad][pair][4] so that the 16-byte reads of layer 3 by consecutive
 //            pairs hit consecutive banks);
 //   layer 3 (16 -> 1, CUDA cores, float32): d on the 14 x 6 tile.
-// One thread of every warp issues the 9 MMAs of one row and branch and commits them to
-// an mbarrier (an MMA this small costs its issuing thread about 90 cycles, several
-// times what the tensor core takes: 144 from one thread were the longest phase of a
-// tile: inference at h = 1/512, k = 64 1.09 -> 0.94 ms); the wait is bounded and reports through an error counter instead of hanging.
+// One thread of every warp issues the 9 MMAs of one row and branch and commits them to an mbarrier: the 144
+// of a tile took 10,600 clocks to issue from one thread and 4,800 from 16 (two CTAs on the SM; 33 clocks an
+// MMA, in which 128 bytes a clock deliver its 4 KB of A): inference at h = 1/512, k = 64 1.09 -> 0.94 ms.
+// The wait is bounded and reports through an error counter instead of hanging.
 #include "common.cuh"
 #include "smoother.cuh"
 
