@@ -230,11 +230,10 @@ int pasm_project(pasm_ctx* ctx, const double* b, const double* c, double* bq, do
  * levels the autotuner leaves out, and autotune = 0), in mixed precision.
  * Levels of at most 1024 rows (level 7 at most, as far as their vectors fit one
  * block's shared memory) run as one kernel with those below them, with the same
- * results: two kernels around the coarse product in float64 with more than 160
- * coarse unknowns.  They run a kernel per operation with the CG smoother, in
- * mixed precision with more than 256 coarse unknowns, from a level on whose shape
- * is set, and in mixed precision from a level on that is the finest, takes the
- * learned step or has its residual captured.
+ * results.  They run a kernel per operation with the CG smoother, with more than
+ * 100 (float64) or 256 (mixed precision) coarse unknowns, from a level on whose
+ * shape is set, and in mixed precision from a level on that is the finest, takes
+ * the learned step or has its residual captured.
  * Errors: PASM_EINVAL. */
 int pasm_tiles(pasm_ctx* ctx, int level, int* chunks_per_thread);
 

@@ -153,7 +153,6 @@ void dense_mm(const Launch& L, int m, int p, const T* D, int ldd, bool trans, co
 // The coarse end of a V-cycle, levels 1 .. top around the solve on level 0 (vcycle_tail.cu).
 constexpr int kTailLevels = 8;                 // levels 0 .. top
 constexpr size_t kTailSmem = 144 * 1024;
-enum { TAIL_DOWN = 1, TAIL_UP = 2 };           // both: the coarse solve too; else it is the caller's
 template <typename T> struct TailCsr {
   const int *rp, *ci;
   const T *v, *w;                              // w: values of the second sweep from zero (A only)
@@ -163,20 +162,19 @@ template <typename T> struct TailLevel {
   int64_t nnz_A, nnz_R, nnz_RA, nnz_P;         // (accounting)
   TailCsr<T> A, R, RA, P;                      // RA: float32 only
   const T* dinv;
-  T *gF, *gE;                                  // n x ldk: right-hand side; iterate
 };
 template <typename T> struct TailArgs {
   TailLevel<T> lv[kTailLevels];
+  const T* gF;                                 // n x ldk on level top: right-hand side
+  T* gE;                                       // and the result
   const T* Ainv;                               // NH x NH, symmetric
   T omega;
-  int top, ldk, nu_pre, nu_post, parts;
+  int top, ldk, nu_pre, nu_post;
   int off[kTailLevels], off_red;               // shared memory (set by the launcher)
 };
 // Whether levels 0 .. top of n[] rows fit one block's shared memory.
-template <typename T> bool vcycle_tail_fits(const int* n, int top, int parts);
-// gE of level top = the V-cycle on A e = gF from zero (DOWN and UP).  DOWN alone: gE of levels 1 .. top =
-// the iterates before the coarse correction, gF of levels 0 .. top - 1; UP alone goes on from these and gE
-// of level 0.
+template <typename T> bool vcycle_tail_fits(const int* n, int top);
+// gE = the V-cycle on A e = gF from zero.
 template <typename T> void vcycle_tail(const Launch& L, TailArgs<T> a);
 cudaError_t vcycle_tail_prepare();
 

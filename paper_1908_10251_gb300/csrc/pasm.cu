@@ -317,12 +317,12 @@ template <typename T> struct Fused { static constexpr bool on = false; };
 template <> struct Fused<float> { static constexpr bool on = true; };
 
 // Where the coarse end of a V-cycle is one kernel (run_tail): levels of at most one row a thread (1521 rows
-// in float32 with the coarse solve of 361 unknowns: 827 -> 838 us for the call; 3375: 1037 -> 1173; up to
-// 1024: h = 1/64, k = 8, float64 998 -> 954, h = 1/512, k = 128, mixed 1701 -> 1694).  The
-// coarse solve is inside up to these many unknowns: a float64 one of 225 takes a single SM's pipe 15 us, as
-// long as the product spread over the chip, which then runs between two halves of the kernel (in float32
-// larger ones leave the levels to their own kernels).
-constexpr int kTailRows = 1024, kTailCoarse32 = 256, kTailCoarse64 = 160;
+// in float32 with the coarse solve of 361 unknowns: 827 -> 838 us for the call; 3375: 1037 -> 1173), and
+// coarse solves of at most these many unknowns.  Steps against a kernel per operation: float32, h = 1/64,
+// k = 8 187 -> 167 us with 49 unknowns, 188 -> 179 with 225.  A float64 block's pipe is its SM's: 224 -> 212
+// with 64 unknowns, 226 -> 223 with 81, 239 -> 240 with 100 (h = 1/72, 1/80 and 1/88, k = 8); 121: h = 1/48,
+// k = 32 237 -> 249; 225, with the solve spread over the chip between two halves of the kernel: 216 -> 234.
+constexpr int kTailRows = 1024, kTailCoarse32 = 256, kTailCoarse64 = 100;
 
 // Hooks before float32 post-smoothing on level l (cur = iterate after the
 // coarse correction, tmp = free buffer): the residual capture for training
@@ -361,7 +361,8 @@ struct TopOut {
 // path does not serve or is not the faster one.
 template <typename T> T* run_tail(pasm_ctx* c, int l) {
   constexpr bool f32 = Fused<T>::on;
-  if (l >= kTailLevels || c->opts.smoother == PASM_CG || c->lv[(size_t)l].n > kTailRows)
+  if (l >= kTailLevels || c->opts.smoother == PASM_CG || c->lv[(size_t)l].n > kTailRows ||
+      c->NH > (f32 ? kTailCoarse32 : kTailCoarse64))
     return nullptr;
   int n[kTailLevels];
   for (int q = 0; q <= l; ++q) {
@@ -374,9 +375,7 @@ template <typename T> T* run_tail(pasm_ctx* c, int l) {
     if (f32 && c->capture_level == q) return nullptr;
     if (f32 && c->opts.smoother == PASM_LEARNED && c->nn.ready && c->nn.nx[(size_t)q] != 0) return nullptr;
   }
-  const bool solve = c->NH <= (f32 ? kTailCoarse32 : kTailCoarse64);
-  if (f32 && !solve) return nullptr;
-  if (!vcycle_tail_fits<T>(n, l, solve ? TAIL_DOWN | TAIL_UP : TAIL_DOWN)) return nullptr;
+  if (!vcycle_tail_fits<T>(n, l)) return nullptr;
   TailArgs<T> a = {};
   for (int q = 0; q <= l; ++q) {
     const LevelDev& v = c->lv[(size_t)q];
@@ -386,24 +385,14 @@ template <typename T> T* run_tail(pasm_ctx* c, int l) {
     t.nnz_A = v.A.nnz; t.nnz_R = v.R.nnz; t.nnz_RA = v.RA.nnz; t.nnz_P = v.P.nnz;
     t.A = csr(v.A); t.R = csr(v.R); t.RA = csr(v.RA); t.P = csr(v.P);
     t.dinv = dinv<T>(v);
-    t.gF = (T*)v.vF;
-    t.gE = (T*)v.vE;
   }
+  a.gF = (const T*)c->lv[(size_t)l].vF;
+  a.gE = (T*)c->lv[(size_t)l].vE;
   a.Ainv = ainv<T>(c);
   a.omega = (T)c->opts.omega;
   a.top = l; a.ldk = c->ldk; a.nu_pre = c->opts.nu_pre; a.nu_post = c->opts.nu_post;
-  const Launch L = launcher(c);
-  if (solve) {
-    a.parts = TAIL_DOWN | TAIL_UP;
-    vcycle_tail<T>(L, a);
-  } else {
-    a.parts = TAIL_DOWN;
-    vcycle_tail<T>(L, a);
-    dense_mm<T>(L, c->NH, c->NH, a.Ainv, c->NH, false, a.lv[0].gF, a.lv[0].gE, c->ldk);
-    a.parts = TAIL_UP;
-    vcycle_tail<T>(L, a);
-  }
-  return (T*)c->lv[(size_t)l].vE;
+  vcycle_tail<T>(launcher(c), a);
+  return a.gE;
 }
 
 template <typename T>

@@ -120,103 +120,87 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(const __grid_const
   const bool flip = ((max(a.nu_pre, first) - first) & 1) != 0;
   pdl_trigger();
   pdl_wait();
-  if (a.parts & TAIL_DOWN) {
-    fetch<T, C>(a.lv[a.top].gF + col, F(a.top), a.lv[a.top].n, a.ldk);
-    __syncthreads();
-    for (int l = a.top; l >= 1; --l) {
-      const TailLevel<T>& L = a.lv[l];
-      T *cur = E(l), *tmp = W(l);
-      for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
-        T f[C], r[C];
-        lds<T, C>(F(l) + i * C, f);
-        const T w = a.omega * __ldg(L.dinv + i);
-        if (first == 2) {   // two sweeps from zero, as jacobi2_zero
-          T acc[C];
-          row_product<T, C>(L.A, L.A.w, F(l), i, acc);
+  fetch<T, C>(a.gF + col, F(a.top), a.lv[a.top].n, a.ldk);
+  __syncthreads();
+  for (int l = a.top; l >= 1; --l) {
+    const TailLevel<T>& L = a.lv[l];
+    T *cur = E(l), *tmp = W(l);
+    for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
+      T f[C], r[C];
+      lds<T, C>(F(l) + i * C, f);
+      const T w = a.omega * __ldg(L.dinv + i);
+      if (first == 2) {   // two sweeps from zero, as jacobi2_zero
+        T acc[C];
+        row_product<T, C>(L.A, L.A.w, F(l), i, acc);
 #pragma unroll
-          for (int c = 0; c < C; ++c) r[c] = w * (T(2) * f[c] - acc[c]);
-        } else {
-#pragma unroll
-          for (int c = 0; c < C; ++c) r[c] = first == 1 ? w * f[c] : T(0);
-        }
-        put<T, C>(cur + i * C, r);
-      }
-      __syncthreads();
-      for (int q = first; q < a.nu_pre; ++q) {
-        sweep<T, C>(L, a.omega, F(l), cur, tmp);
-        __syncthreads();
-        T* t = cur; cur = tmp; tmp = t;
-      }
-      const int nc = a.lv[l - 1].n;
-      if (F32) {   // as restrict_first
-        for (int i = threadIdx.x; i < nc; i += kTailThreads) {
-          T rf[C], qe[C];
-          row_product<T, C>(L.R, L.R.v, F(l), i, rf);
-          row_product<T, C>(L.RA, L.RA.v, cur, i, qe);
-#pragma unroll
-          for (int c = 0; c < C; ++c) rf[c] = rf[c] - qe[c];
-          put<T, C>(F(l - 1) + i * C, rf);
-        }
+        for (int c = 0; c < C; ++c) r[c] = w * (T(2) * f[c] - acc[c]);
       } else {
-        for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
-          T acc[C], f[C];
-          row_product<T, C>(L.A, L.A.v, cur, i, acc);
-          lds<T, C>(F(l) + i * C, f);
 #pragma unroll
-          for (int c = 0; c < C; ++c) f[c] = f[c] - acc[c];
-          put<T, C>(tmp + i * C, f);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < nc; i += kTailThreads) {
-          T acc[C];
-          row_product<T, C>(L.R, L.R.v, tmp, i, acc);
-          put<T, C>(F(l - 1) + i * C, acc);
-        }
+        for (int c = 0; c < C; ++c) r[c] = first == 1 ? w * f[c] : T(0);
       }
-      __syncthreads();
-    }
-    if (!(a.parts & TAIL_UP)) {   // the coarse solve is another kernel's
-      for (int l = 1; l <= a.top; ++l) {
-        flush<T, C>(flip ? W(l) : E(l), a.lv[l].gE + col, a.lv[l].n, a.ldk);
-        if (l < a.top) flush<T, C>(F(l), a.lv[l].gF + col, a.lv[l].n, a.ldk);
-      }
-      flush<T, C>(F(0), a.lv[0].gF + col, a.lv[0].n, a.ldk);
-      return;
-    }
-    // E_0 = A_H^{-1} F_0 (the inverse is symmetric bit for bit, so its rows are read as columns), the
-    // order of dense_mm: interleaved parts, then the parts' sums in order
-    const int n0 = a.lv[0].n, part = threadIdx.x / kPartThreads;
-    T* const red = s + a.off_red;
-    const T* const f0 = F(0);
-    for (int i0 = threadIdx.x % kPartThreads; i0 < n0; i0 += 2 * kPartThreads) {
-      const int i1 = min(i0 + kPartThreads, n0 - 1);
-      T s0[C], s1[C];
-#pragma unroll
-      for (int c = 0; c < C; ++c) s0[c] = s1[c] = T(0);
-#pragma unroll 8
-      for (int j = part; j < n0; j += kParts) {
-        const T d0 = __ldg(a.Ainv + (size_t)j * n0 + i0), d1 = __ldg(a.Ainv + (size_t)j * n0 + i1);
-        T x[C];
-        lds<T, C>(f0 + j * C, x);
-#pragma unroll
-        for (int c = 0; c < C; ++c) { s0[c] = fma(d0, x[c], s0[c]); s1[c] = fma(d1, x[c], s1[c]); }
-      }
-      put<T, C>(red + (part * n0 + i0) * C, s0);
-      if (i0 + kPartThreads < n0) put<T, C>(red + (part * n0 + i1) * C, s1);
+      put<T, C>(cur + i * C, r);
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < n0 * C; q += kTailThreads) {
-      T x = red[q];
+    for (int q = first; q < a.nu_pre; ++q) {
+      sweep<T, C>(L, a.omega, F(l), cur, tmp);
+      __syncthreads();
+      T* t = cur; cur = tmp; tmp = t;
+    }
+    const int nc = a.lv[l - 1].n;
+    if (F32) {   // as restrict_first
+      for (int i = threadIdx.x; i < nc; i += kTailThreads) {
+        T rf[C], qe[C];
+        row_product<T, C>(L.R, L.R.v, F(l), i, rf);
+        row_product<T, C>(L.RA, L.RA.v, cur, i, qe);
 #pragma unroll
-      for (int p = 1; p < kParts; ++p) x += red[p * n0 * C + q];
-      E(0)[q] = x;
+        for (int c = 0; c < C; ++c) rf[c] = rf[c] - qe[c];
+        put<T, C>(F(l - 1) + i * C, rf);
+      }
+    } else {
+      for (int i = threadIdx.x; i < L.n; i += kTailThreads) {
+        T acc[C], f[C];
+        row_product<T, C>(L.A, L.A.v, cur, i, acc);
+        lds<T, C>(F(l) + i * C, f);
+#pragma unroll
+        for (int c = 0; c < C; ++c) f[c] = f[c] - acc[c];
+        put<T, C>(tmp + i * C, f);
+      }
+      __syncthreads();
+      for (int i = threadIdx.x; i < nc; i += kTailThreads) {
+        T acc[C];
+        row_product<T, C>(L.R, L.R.v, tmp, i, acc);
+        put<T, C>(F(l - 1) + i * C, acc);
+      }
     }
-  } else {
-    fetch<T, C>(a.lv[0].gE + col, E(0), a.lv[0].n, a.ldk);
-    for (int l = 1; l <= a.top; ++l) {
-      fetch<T, C>(a.lv[l].gE + col, flip ? W(l) : E(l), a.lv[l].n, a.ldk);
-      fetch<T, C>(a.lv[l].gF + col, F(l), a.lv[l].n, a.ldk);
+    __syncthreads();
+  }
+  // E_0 = A_H^{-1} F_0 (the inverse is symmetric bit for bit, so its rows are read as columns), the
+  // order of dense_mm: interleaved parts, then the parts' sums in order
+  const int n0 = a.lv[0].n, part = threadIdx.x / kPartThreads;
+  T* const red = s + a.off_red;
+  const T* const f0 = F(0);
+  for (int i0 = threadIdx.x % kPartThreads; i0 < n0; i0 += 2 * kPartThreads) {
+    const int i1 = min(i0 + kPartThreads, n0 - 1);
+    T s0[C], s1[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) s0[c] = s1[c] = T(0);
+#pragma unroll 8
+    for (int j = part; j < n0; j += kParts) {
+      const T d0 = __ldg(a.Ainv + (size_t)j * n0 + i0), d1 = __ldg(a.Ainv + (size_t)j * n0 + i1);
+      T x[C];
+      lds<T, C>(f0 + j * C, x);
+#pragma unroll
+      for (int c = 0; c < C; ++c) { s0[c] = fma(d0, x[c], s0[c]); s1[c] = fma(d1, x[c], s1[c]); }
     }
+    put<T, C>(red + (part * n0 + i0) * C, s0);
+    if (i0 + kPartThreads < n0) put<T, C>(red + (part * n0 + i1) * C, s1);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < n0 * C; q += kTailThreads) {
+    T x = red[q];
+#pragma unroll
+    for (int p = 1; p < kParts; ++p) x += red[p * n0 * C + q];
+    E(0)[q] = x;
   }
   __syncthreads();
   const T* ec = E(0);
@@ -239,7 +223,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(const __grid_const
     }
     ec = cur;
   }
-  flush<T, C>(ec, a.lv[a.top].gE + col, a.lv[a.top].n, a.ldk);
+  flush<T, C>(ec, a.gE + col, a.lv[a.top].n, a.ldk);
 }
 
 // Offsets of the levels' vectors in shared memory; bytes in all.
@@ -251,18 +235,17 @@ size_t tail_layout(TailArgs<T>& a) {
     at += (l == 0 ? 2 : 3) * (size_t)a.lv[l].n * TailCols<T>::v;
   }
   a.off_red = (int)at;
-  if ((a.parts & (TAIL_DOWN | TAIL_UP)) == (TAIL_DOWN | TAIL_UP)) at += (size_t)kParts * a.lv[0].n * TailCols<T>::v;
+  at += (size_t)kParts * a.lv[0].n * TailCols<T>::v;
   return at * sizeof(T);
 }
 
 }  // namespace
 
 template <typename T>
-bool vcycle_tail_fits(const int* n, int top, int parts) {
+bool vcycle_tail_fits(const int* n, int top) {
   if (top < 1 || top >= kTailLevels) return false;
   TailArgs<T> a = {};
   a.top = top;
-  a.parts = parts;
   for (int l = 0; l <= top; ++l) a.lv[l].n = n[l];
   return tail_layout<T>(a) <= kTailSmem;
 }
@@ -276,52 +259,35 @@ cudaError_t vcycle_tail_prepare() {
 template <typename T>
 void vcycle_tail(const Launch& L, TailArgs<T> a) {
   const size_t smem = tail_layout<T>(a);
-  const bool down = (a.parts & TAIL_DOWN) != 0, up = (a.parts & TAIL_UP) != 0;
   {
     // matrices once (the second sweep from zero has values of its own), what leaves and enters the kernel once
     const bool f32 = sizeof(T) == 4, two = f32 && a.nu_pre >= 2;
     const double w = sizeof(T), ldk = a.ldk, n0 = a.lv[0].n;
-    const int down_sweeps = down ? std::max(0, a.nu_pre - (two ? 2 : 1)) : 0, up_sweeps = up ? a.nu_post : 0;
-    double bytes = 0.0, flops = 0.0, vec = 0.0;
+    const int sweeps = std::max(0, a.nu_pre - (two ? 2 : 1)) + a.nu_post;
+    const bool own = sweeps > 0 || !f32;   // products with A's own values
+    double bytes = 2.0 * a.lv[a.top].n * ldk * w + n0 * n0 * w, flops = 2.0 * n0 * n0 * ldk;
     for (int l = 1; l <= a.top; ++l) {
       const TailLevel<T>& v = a.lv[l];
       const double n = v.n, nc = a.lv[l - 1].n, A = (double)v.nnz_A, R = (double)v.nnz_R, RA = (double)v.nnz_RA,
                    P = (double)v.nnz_P, row = 4.0, entry = 4.0 + w;
-      const int products = down_sweeps + up_sweeps + (down && !f32 ? 1 : 0);   // with A's own values
-      if (products > 0 || (down && two)) bytes += (n + 1) * row + A * 4.0;
-      if (products > 0) bytes += A * w;
-      if (down && two) bytes += A * w;
-      if (down) bytes += (nc + 1) * row + R * entry + (f32 ? (nc + 1) * row + RA * entry : 0.0);
-      if (up) bytes += (n + 1) * row + P * entry;
-      if ((down && a.nu_pre > 0) || up_sweeps > 0) bytes += n * w;
-      flops += ldk * ((down_sweeps + up_sweeps) * (2.0 * A + 3.0 * n));
-      if (down) {
-        flops += ldk * (two ? 2.0 * A + 3.0 * n : a.nu_pre >= 1 ? n : 0.0);
-        flops += ldk * (f32 ? 2.0 * (R + RA) + nc : 2.0 * (A + R) + n);
-      }
-      if (up) flops += ldk * (2.0 * P + n);
-      if (!up) vec += n + nc;                            // iterate; right-hand side below
-      if (!down) vec += n + (l == 1 ? nc : 0.0) + n;     // both read back
-    }
-    if (down) vec += a.lv[a.top].n;
-    if (up) vec += a.lv[a.top].n;
-    bytes += vec * ldk * w;
-    if (down && up) {
-      bytes += n0 * n0 * w;
-      flops += 2.0 * n0 * n0 * ldk;
+      if (own || two) bytes += (n + 1) * row + A * (4.0 + w * ((own ? 1 : 0) + (two ? 1 : 0)));
+      bytes += (nc + 1) * row + R * entry + (n + 1) * row + P * entry;
+      if (f32) bytes += (nc + 1) * row + RA * entry;
+      if (a.nu_pre > 0 || a.nu_post > 0) bytes += n * w;
+      flops += ldk * (sweeps * (2.0 * A + 3.0 * n) + (two ? 2.0 * A + 3.0 * n : a.nu_pre >= 1 ? n : 0.0) +
+                      (f32 ? 2.0 * (R + RA) + nc : 2.0 * (A + R) + n) + 2.0 * P + n);
     }
     L.rows(a.lv[a.top].n);
     L.begin(KC_DENSE, bytes, flops);
   }
-  // Not a programmatic launch: blocks that start while the kernel before drains go to the SMs that free up
-  // first, two to one SM (to one float64 pipe) while others stay empty (a float64 step at h = 1/64, N_H = 225,
-  // k = 8: 233 us against 290, and 277 with a kernel per operation).
+  // plainly, as the other kernels bound by their SM (a float64 step at h = 1/96, k = 16, when it took the 121
+  // coarse unknowns there: 274 us programmatically, 265 plainly; others within 1 %)
   launch(L.plain(), k_vcycle_tail<T>, a.ldk / TailCols<T>::v, kTailThreads, smem, a);
   L.bump();
 }
 
-template bool vcycle_tail_fits<float>(const int*, int, int);
-template bool vcycle_tail_fits<double>(const int*, int, int);
+template bool vcycle_tail_fits<float>(const int*, int);
+template bool vcycle_tail_fits<double>(const int*, int);
 template void vcycle_tail<float>(const Launch&, TailArgs<float>);
 template void vcycle_tail<double>(const Launch&, TailArgs<double>);
 

@@ -58,14 +58,15 @@ def test_secular_blocks_spread_over_the_sms(precision):
     pg.pasm_destroy(ctx)
 
 
-def test_coarse_levels_in_one_kernel_are_no_slower(k=8):
-    """The coarse end of the float64 cycle (961 rows over 225 coarse unknowns), a block per column, against the same
-    levels with a kernel per operation (which a set launch shape selects)."""
+@pytest.mark.parametrize("precision,NH", [(0, 8), (1, 8), (1, 16)])
+def test_coarse_levels_in_one_kernel_are_no_slower(precision, NH, k=8):
+    """The coarse end of the cycle, a block per column group, where it runs as one kernel, against the same levels with
+    a kernel per operation (which a set launch shape selects)."""
     from paper_1908_10251_gb300 import build
     build.build()
     import paper_1908_10251_gb300 as pg
-    ctx, restart = start(pg, (2, 64, 16), k, 0)
-    sep, restart_sep = start(pg, (2, 64, 16), k, 0)
+    ctx, restart = start(pg, (2, 64, NH), k, precision)
+    sep, restart_sep = start(pg, (2, 64, NH), k, precision)
     restart_sep()
     pg.pasm_set_tiles(sep, 1, {"jacobi": 1})
     assert replay_us(pg, ctx, restart) <= replay_us(pg, sep, restart_sep)

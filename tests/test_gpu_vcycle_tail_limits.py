@@ -40,7 +40,7 @@ def context(pg, levels, k, precision, nu_pre, nu_post):
     return ctx
 
 
-def accounted(levels, top, ldk, f32, nu_pre, nu_post, down, up):
+def accounted(levels, top, ldk, f32, nu_pre, nu_post):
     """Bytes (matrices, and the vectors that enter or leave, once) and flops of the kernel over levels top .. 1."""
     A, _, P = levels
     w = 4 if f32 else 8
@@ -48,37 +48,24 @@ def accounted(levels, top, ldk, f32, nu_pre, nu_post, down, up):
     csr = lambda rows, nnz, values=1: 4 * (rows + 1) + nnz * (4 + w * values)  # noqa: E731
     n = [a.shape[0] for a in A]
     pattern = lambda m: sp.csr_matrix((np.ones(m.nnz), m.indices, m.indptr), shape=m.shape)  # noqa: E731
-    by = fl = 0
+    by, fl = 2 * n[top] * ldk * w + n[0] ** 2 * w, 2 * n[0] ** 2
     for l in range(1, top + 1):
         a, p = A[l].nnz, P[l - 1].nnz
         ra = (pattern(P[l - 1]).T @ pattern(A[l])).nnz
-        sweeps = (max(0, nu_pre - (2 if two else 1)) if down else 0) + (nu_post if up else 0)
-        own = sweeps > 0 or (down and not f32)
-        if own or (down and two):
-            by += csr(n[l], a, int(own) + int(down and two))
-        if down:
-            by += csr(n[l - 1], p) + (csr(n[l - 1], ra) if f32 else 0)
-            first = 2 * a + 3 * n[l] if two else (n[l] if nu_pre else 0)
-            fl += first + (2 * (p + ra) + n[l - 1] if f32 else 2 * (a + p) + n[l])
-        if up:
-            by += csr(n[l], p)
-            fl += 2 * p + n[l]
-        if (down and nu_pre) or (up and nu_post):
-            by += n[l] * w
-        fl += sweeps * (2 * a + 3 * n[l])
-    vec = n[top] if down and up else sum(n[1:top + 1]) + sum(n[:top])        # down: out; up: the iterates in ...
-    if up and not down:
-        vec = sum(n[:top + 1]) + sum(n[1:top + 1])                           # ... with right-hand sides above level 0
-    vec += n[top]                                                            # in (down alone) or out
-    by += vec * ldk * w
-    if down and up:
-        by += n[0] ** 2 * w
-        fl += 2 * n[0] ** 2
+        sweeps = max(0, nu_pre - (2 if two else 1)) + nu_post
+        own = sweeps > 0 or not f32
+        if own or two:
+            by += csr(n[l], a, int(own) + int(two))
+        by += csr(n[l - 1], p) + (csr(n[l - 1], ra) if f32 else 0) + csr(n[l], p)
+        by += n[l] * w if nu_pre or nu_post else 0
+        fl += 2 * a + 3 * n[l] if two else (n[l] if nu_pre else 0)
+        fl += 2 * (p + ra) + n[l - 1] if f32 else 2 * (a + p) + n[l]
+        fl += 2 * p + n[l] + sweeps * (2 * a + 3 * n[l])
     return by, fl * ldk
 
 
 @pytest.mark.parametrize("precision,sizes,top", [(1, (100, 300, 900, 2000), 2), (0, (100, 300, 900, 2000), 2),
-                                                 (0, (200, 600, 2000), 1)])
+                                                 (1, (200, 600, 2000), 1)])
 @pytest.mark.parametrize("nu_pre,nu_post", [(2, 2), (1, 0), (4, 1), (0, 3)])
 def test_traced_bytes_and_flops(precision, sizes, top, nu_pre, nu_post):
     from paper_1908_10251_gb300 import build
@@ -89,18 +76,17 @@ def test_traced_bytes_and_flops(precision, sizes, top, nu_pre, nu_post):
     ctx = context(pg, levels, k, precision, nu_pre, nu_post)
     pg.pasm_trace_step(ctx)
     got = [(b, f) for c, rows, _, b, f in pg.pasm_trace_launches(ctx) if c == "dense" and rows == sizes[top]]
-    parts = [(True, True)] if sizes[0] <= 160 or precision == 1 else [(True, False), (False, True)]
-    want = [accounted(levels, top, ldk, precision == 1, nu_pre, nu_post, *p) for p in parts]
-    assert got == want * 2                       # two cycles a step
+    assert got == [accounted(levels, top, ldk, precision == 1, nu_pre, nu_post)] * 2   # two cycles a step
     pg.pasm_destroy(ctx)
 
 
-# (precision, rows of the levels, the highest level in the kernel or None): at most 1024 rows; a coarse solve of at
-# most 160 unknowns in float64 (above, it runs between two halves of the kernel) and 256 in mixed precision (above, a
-# kernel per operation); mixed precision's finest level stays outside; shared memory; eight levels
-ROUTES = [(0, (160, 1024, 2050), 1), (0, (161, 1024, 2050), 1), (0, (160, 1025, 2050), None), (0, (100, 1000), 1),
+# (precision, rows of the levels, the highest level in the kernel or None): at most 1024 rows; at most 100 coarse
+# unknowns in float64 and 256 in mixed precision; mixed precision's finest level stays outside; shared memory; eight
+# levels
+ROUTES = [(0, (100, 1024, 2050), 1), (0, (101, 1024, 2050), None), (0, (100, 1025, 2050), None), (0, (100, 1000), 1),
+          (0, (161, 1000), None),
           (1, (256, 1024, 2050), 1), (1, (257, 1024, 2050), None), (1, (160, 1025, 2050), None), (1, (100, 1000), None),
-          (0, (160, 900, 1000, 1024, 2100), 3), (1, (256, 900, 1000, 1024, 2100), 2),
+          (0, (100, 900, 1000, 1024, 2100), 3), (1, (256, 900, 1000, 1024, 2100), 2),
           (0, (8, 12, 18, 27, 40, 60, 90, 135, 200, 300), 7), (1, (8, 12, 18, 27, 40, 60, 90, 135, 200, 300), 7)]
 
 
@@ -129,7 +115,6 @@ def test_route_and_bits(precision, sizes, top, k):
         ran.append([rows for c, rows, *_ in pg.pasm_trace_launches(ctx) if c == "dense" and rows])
         launches.append(len(pg.pasm_trace_launches(ctx)))
         pg.pasm_destroy(ctx)
-    halves = 2 if precision == 0 and sizes[0] > 160 else 1
-    assert ran == [[] if top is None else [sizes[top]] * 2 * halves, []]   # two cycles a step
+    assert ran == [[] if top is None else [sizes[top]] * 2, []]   # two cycles a step
     assert (launches[0] < launches[1]) == (top is not None)
     assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
