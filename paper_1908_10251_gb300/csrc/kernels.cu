@@ -1410,11 +1410,8 @@ void cg_smooth(const Launch& L, const DCsr& A, const T* F, T* X, bool x_zero, T*
     const bool last = it + 1 == nu, rr = x_zero && it == 0;
     L.rows(A.n_rows);
     L.begin(KC_CG, mat + (last ? 1.0 : 2.0) * vec, 2.0 * nnz * ldk + 2.0 * rows * ldk);
-  // plainly where there is a block for every SM: blocks that start early crowd the SMs that free up first (a
-  // float64 step in 3D, h = 1/32, k = 8: 668 us programmatically, 582 plainly); with fewer blocks the early
-  // start is worth more (h = 1/64, k = 8: 518 us against 532)
 #define PASM_CG_DIR(QO, RRV)                                                                                     \
-  PASM_DISPATCH_CH(g.ch, launch(grid >= 152 ? L.plain() : L, k_cg_dir<T, CH, QO, RRV>, grid, kBlock, smem, A.n_rows, A.rp, A.ci, av, p, Q,    \
+  PASM_DISPATCH_CH(g.ch, launch(L, k_cg_dir<T, CH, QO, RRV>, grid, kBlock, smem, A.n_rows, A.rp, A.ci, av, p, Q,    \
                                 w.partial, partial2, ldk, g.tpr))
     if (last) {
       if (rr) { PASM_CG_DIR(false, true); } else { PASM_CG_DIR(false, false); }
