@@ -894,10 +894,9 @@ void dense_mm(const Launch& L, int m, int p, const T* D, int ldd, bool trans, co
   const int cols = std::min(ldk, 32), rows = kDenseRows * (32 / cols);
   dim3 grid(ldk / cols, (m + rows - 1) / rows);
   L.begin(KC_DENSE, ((double)m * p + (double)p * ldk + (double)m * ldk) * sizeof(T), 2.0 * m * p * ldk);
-  // float64 plainly: programmatically a step at N_H = 289 took 499 us instead of 413 (h = 1/144, k = 24) and
-  // 718 instead of 635 (k = 64); in float32, whose pipe is not the scarce part, the early start is worth more
-  // (multigrid solve with CG smoothing, h = 1/320, k = 37: 1447 us, plainly 1475)
-  launch(sizeof(T) == 8 ? L.plain() : L, k_dense_mm<T>, grid, kBlock, 0, m, p, D, ldd, trans ? 1 : 0, B, C, ldk, cols);
+  // (in float32, whose pipe is not the scarce part, the early start is worth more: multigrid solve with CG
+  // smoothing, h = 1/320, k = 37: 1447 us, plainly 1475)
+  launch(sizeof(T) == 8 ? L.spread((int)(grid.x * grid.y)) : L, k_dense_mm<T>, grid, kBlock, 0, m, p, D, ldd, trans ? 1 : 0, B, C, ldk, cols);
   L.bump();
 }
 template void dense_mm<double>(const Launch&, int, int, const double*, int, bool, const double*, double*, int);

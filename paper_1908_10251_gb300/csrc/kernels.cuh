@@ -47,6 +47,7 @@ void tracer_end(Tracer* t, cudaStream_t s);
 // Launch bookkeeping shared by every launcher: the stream, a launch counter
 // and an optional tracer that brackets each launch with CUDA events and
 // records its algorithmic bytes and flops.
+constexpr int kSpreadBlocks = 64;   // see `launch`
 struct Launch {
   cudaStream_t s = nullptr;
   int* counter = nullptr;
@@ -54,8 +55,8 @@ struct Launch {
   int geo = 0;  // row-group kernels: 16-byte chunks per thread (0 = default; set by the autotuner)
   int rpt = 0;  // float32 row kernels: row blocks each block walks (0 = by size; set by the autotuner)
   bool pdl = true;  // programmatic dependent launch (see `launch`); off where an operand that is static in a
-                    // context may have been written by the kernel before, and by plain()
-  Launch plain() const { Launch q = *this; q.pdl = false; return q; }
+                    // context may have been written by the kernel before, and by spread()
+  Launch spread(int blocks) const { Launch q = *this; q.pdl = pdl && blocks < kSpreadBlocks; return q; }
   void begin(int cls, double bytes, double flops) const { if (tr) tracer_begin(tr, s, cls, bytes, flops); }
   void rows(int n) const { if (tr) tracer_rows(tr, n); }
   void bump() const {
@@ -73,8 +74,10 @@ struct Launch {
 // __restrict__ pointer or __ldg is one the compiler may move above the wait.
 // A launch gap between two small kernels costs 1 to 1.5 us; a step has 40 to 80.
 // Kernels whose blocks are each bound by their SM (the float64 pipe, one chain of latencies) are launched
-// plainly (Launch::plain): blocks that start while the kernel before drains go to the SMs that free up
-// first and share them, while others stay empty.  Figures stand at each of them.
+// plainly from kSpreadBlocks blocks on (Launch::spread): blocks that start while the kernel before drains go
+// to the SMs that free up first and share them, while others stay empty (figures stand at each of them).
+// With few blocks the early start is worth more (augmented step at N_H = 16, k = 4: 141 us programmatically,
+// 147 plainly).
 template <typename... P, typename... A>
 inline void launch(const Launch& L, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
   cudaLaunchConfig_t cfg = {};

@@ -404,7 +404,12 @@ T* vcycle(pasm_ctx* c, int l, const TopOut* top = nullptr) {
   T* Tm = (T*)v.vT;
   const int ldk = c->ldk;
   if (l == 0) {
-    dense_mm<T>(L, c->NH, c->NH, ainv<T>(c), c->NH, false, F, E, ldk);
+    // float64, whose pipe is the SM's scarce part, plainly (see `launch`): early blocks share the SMs that the
+    // restriction leaves first (h = 1/144, N_H = 289: four steps with k = 8 1643 us programmatically, 1330
+    // plainly; a step with k = 24 499 and 413, with k = 64 718 and 635)
+    Launch q = L;
+    if (!Fused<T>::on) q.pdl = false;
+    dense_mm<T>(q, c->NH, c->NH, ainv<T>(c), c->NH, false, F, E, ldk);
     return E;
   }
   if (!top || !Fused<T>::on)

@@ -452,8 +452,8 @@ void proj_tc(const Launch& L, const SplitMat& A, const double* B0, const double*
   dim3 grid((ncols + kN - 1) / kN, A.mtiles, (A.Kpad + kKC - 1) / kKC);
   const double m = A.m, K = A.K, n = ncols;
   L.begin(KC_PROJ, (m * K + K * n + m * n) * 8.0, 2.0 * m * K * n);
-  // plainly: programmatically a step took 1 to 3 % longer (h = 1/128, k = 64, float64: 639 us against 627)
-  launch(L.plain(), k_proj_tc, grid, kThreads, kSmem, A.m, A.K, A.Kpad, A.planes, A.rexp, B0, B1, C0, C1, ldk, ncols, hl,
+  // programmatically a step took 1 to 3 % longer (h = 1/128, k = 64, float64: 639 us against 627)
+  launch(L.spread((int)(grid.x * grid.y * grid.z)), k_proj_tc, grid, kThreads, kSmem, A.m, A.K, A.Kpad, A.planes, A.rexp, B0, B1, C0, C1, ldk, ncols, hl,
                                             tickets, err, wait_limit > 0 ? wait_limit : kWaitLimit, skip_mma);
   L.bump();
 }

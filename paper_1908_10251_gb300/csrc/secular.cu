@@ -40,9 +40,9 @@
 // the cluster barrier orders the exchange.  GB300's float64 pipe (2 FMA per
 // clock and SM) bounds the root solves, so more SMs per pair is more
 // throughput.  Rank 0 alone writes the results.
-// For the same reason the launch is not a programmatic one: blocks that start while the kernel before drains
-// go to the SMs that free up first, several to one float64 pipe while others stay empty (a step at N_H = 289,
-// mixed, k = 64: 376 us against 437 programmatically, k = 152: 1021 against 1400).
+// For the same reason the launch is not a programmatic one from 64 blocks on: blocks that start while the
+// kernel before drains go to the SMs that free up first, several to one float64 pipe while others stay empty
+// (a step at N_H = 289, mixed, k = 64: 376 us against 437 programmatically, k = 152: 1021 against 1400).
 //
 // With the roots spread out a solve is one chain of dependent float64 operations (about 60 clocks each) and
 // of code fetched for the first time, 118,000 clocks at N_H = 225: loads and sums 12,700, pole lists 6,600,
@@ -532,6 +532,7 @@ __global__ void __launch_bounds__(kSecThreads) k_secular(SecularArgs a) {
   // the block-wide pole lists below)
   const int gwarp = warp * cs + rank, nwarps = cs * kSecWarps;
   pdl_trigger();
+  pdl_wait();
   if (!a.active[i]) {
     if (tid == 0 && lead) a.upd[i] = 0;
     return;
@@ -866,13 +867,15 @@ void secular_select(const Launch& L, const SecularArgs& a0) {
   cfg.blockDim = dim3(kSecThreads);
   cfg.dynamicSmemBytes = secular_smem(a.NH);
   cfg.stream = L.s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)a.cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = L.spread(a.k * a.cs).pdl ? 2 : 1;
   cudaLaunchKernelEx(&cfg, secular_kernel(a.NH), a);
   L.bump();
 }

@@ -280,9 +280,7 @@ void vcycle_tail(const Launch& L, TailArgs<T> a) {
     L.rows(a.lv[a.top].n);
     L.begin(KC_DENSE, bytes, flops);
   }
-  // plainly, as the other kernels bound by their SM (a float64 step at h = 1/96, k = 16, when it took the 121
-  // coarse unknowns there: 274 us programmatically, 265 plainly; others within 1 %)
-  launch(L.plain(), k_vcycle_tail<T>, a.ldk / TailCols<T>::v, kTailThreads, smem, a);
+  launch(L.spread(a.ldk / TailCols<T>::v), k_vcycle_tail<T>, a.ldk / TailCols<T>::v, kTailThreads, smem, a);
   L.bump();
 }
 
